@@ -28,6 +28,8 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "../../include/bbx.h"
 
 namespace bbx {
@@ -56,7 +58,7 @@ struct TissueArgs {  // (CUtensorMap members impose its alignment)
     CUtensorMap tm_u[2];  // V of buffer b with halo (box TX+8 x TY+2)
     CUtensorMap tm_s[2];  // non-diffusing variables of buffer b (box TX x TY x S-1; with 16-bit gates: Ca only)
     CUtensorMap tm_g[2];  // 16-bit gates of buffer b (box TX x TY x 6 uint16), when stored so
-    CUtensorMap tm_f;     // unit fibres, x stored from -4 with clamped padding (box TX x TY x 3, no halo)
+    CUtensorMap tm_f;     // unit fibres (box TX x TY x 3, no halo)
     CUtensorMap tm_d;     // the W-tilde sums of every node (box TX x TY x 3)
     CUtensorMap tm_m;     // tissue mask bytes
     float* state[2];      // the ping-pong buffers, var v at state[b] + v*vol (32-bit variables)
@@ -79,6 +81,16 @@ struct TissueArgs {  // (CUtensorMap members impose its alignment)
     float mp[8];  // model parameters in kernel form
     const struct SurrogateData* surr;  // reaction surrogate (Beeler-Reuter), or nullptr
     const float4* tab;                 // V-table of the model (kTabN x 4 float4), or nullptr
+};
+
+// Where the done flags of a piece's column are (a launch of several steps over
+// unmasked grids): the flag of computed plane z (a sheet: tile row z) at
+// base + z; len planes from z0 on; the columns one tile further in y lie `row`
+// flags away, those in x len flags; which of them exist.
+struct PieceFlags {
+    long long base;
+    int row, len, z0;
+    int has;  // bit 0, 1: column at x - 1, x + 1; bit 2, 3: at y - 1, y + 1
 };
 
 // One launch: a balanced schedule of pieces over the grids of one kernel type.
@@ -120,6 +132,10 @@ struct LaunchArgs {
     int reg_len, reg_nbx, reg_ty, reg_ctas;  // column length (nz), columns in x, tile rows, CTAs
     long long reg_planes;                    // column-planes of the schedule
     int reg_z0;                              // first computed plane of every column (0; 1 below a halo plane)
+    int n_steps;         // time steps of this launch (more than one: unmasked grids only, all CTAs resident)
+    const PieceFlags* piece_flags;  // per slot
+    int* flags;          // per grid column and computed plane: the last step done, as a running number
+    int epoch;           // that number before this launch's first step
 };
 
 struct Coef {
@@ -170,6 +186,20 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     return ok != 0;
 }
 
+// The same without waiting (a try_wait that fails has waited for a
+// system-dependent time, several microseconds here).
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_addr(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
 // Wait for the barrier phase with the given parity; gives up (returns false)
 // after `limit` SM clock cycles instead of spinning forever.
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, long long limit) {
@@ -207,6 +237,25 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, i
         : "memory");
 }
 
+// Done flags of a launch of several steps.
+__device__ __forceinline__ int ld_flag(const int* p) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_flag(int* p, int v) {
+    asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+__device__ __forceinline__ int ld_shared_acquire(const int* p) {
+    int v;
+    asm volatile("ld.acquire.cta.shared::cta.s32 %0, [%1];" : "=r"(v) : "r"(smem_addr(p)) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_shared_release(int* p, int v) {
+    asm volatile("st.release.cta.shared::cta.s32 [%0], %1;" ::"r"(smem_addr(p)), "r"(v) : "memory");
+}
+
 __device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
@@ -218,6 +267,28 @@ __device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
 struct F2 {
     float hi, lo;
 };
+
+// Packed FP32 pairs (the two x-adjacent nodes of a thread): one instruction
+// slot per pair.  The FP32 pipe runs them at the rate of two scalar
+// operations (measured: 2.2 cycles a warp against 1.1), but the step kernels
+// are bound by instruction issue, where a pair costs one slot instead of two;
+// broadcast scalars, immediates and negated operands are free.  Every
+// operation is rounded on its own (no contraction), so a node's result does
+// not depend on the kernel variant it is computed in.
+__device__ __forceinline__ float2 splat2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+// TwoSum of a running pair of sums: the rounding error of each addition goes
+// to lo, as two_sum_add does for one.
+__device__ __forceinline__ void two_sum_add2(float2& hi, float2& lo, float2 b) {
+    const float2 s = add2(hi, b);
+    const float2 bb = sub2(s, hi);
+    lo = add2(lo, add2(sub2(hi, sub2(s, bb)), sub2(b, bb)));
+    hi = s;
+}
 
 __device__ __forceinline__ void two_sum_add(F2& a, float b) {
     float s = a.hi + b;
@@ -277,9 +348,11 @@ __device__ __forceinline__ void start_ticket(const LaunchArgs& L, const TissueDy
     const unsigned int t = atomicAdd(L.ticket, 1u);
     if (t == gridDim.x - 1) {
         TissueDyn* d = L.t0.dyn;
-        d->t = d0.t + L.t0.dt_d;
-        d->n = d0.n + 1;
-        d->cur = d0.cur ^ 1;
+        double tn = d0.t;
+        for (int s = 0; s < L.n_steps; ++s) tn = tn + L.t0.dt_d;
+        d->t = tn;
+        d->n = d0.n + L.n_steps;
+        d->cur = d0.cur ^ (L.n_steps & 1);
         d->total_pending = 1;
         *L.ticket = 0u;
     }
@@ -311,9 +384,11 @@ __device__ __forceinline__ void finish_grid(const LaunchArgs& L, int ti, double 
     TissueDyn* d = T->dyn;
     if (!isfinite(s)) atomicOr(L.err, ERRBIT_NAN);
     d->total = s;
-    d->t = d->t + T->dt_d;
-    d->n = d->n + 1;
-    d->cur = d->cur ^ 1;
+    double tn = d->t;
+    for (int k = 0; k < L.n_steps; ++k) tn = tn + T->dt_d;
+    d->t = tn;
+    d->n = d->n + L.n_steps;
+    d->cur = d->cur ^ (L.n_steps & 1);
     d->total_pending = 0;
 }
 
@@ -382,6 +457,15 @@ struct Model<BBX_FHN> {
         y[0] = u + dt * du;
         y[1] = v + dt * dv;
     }
+    // the same for a pair of nodes, L the diffusion term plus the stimulus
+    __device__ static __forceinline__ void update2(const float* mp, float2* y, float2 L, float dt) {
+        const float2 u = y[0], v = y[1];
+        const float2 c = fma2(mul2(u, u), splat2(-1.0f / 3.0f), splat2(1.0f));
+        const float2 du = fma2(sub2(mul2(u, c), v), splat2(mp[0]), L);
+        const float2 dv = mul2(fma2(v, splat2(-mp[3]), add2(u, splat2(mp[2]))), splat2(mp[1]));
+        y[0] = fma2(splat2(dt), du, u);
+        y[1] = fma2(splat2(dt), dv, v);
+    }
     // right-hand side with the source I (diffusion term + stimulus) on u
     __device__ static __forceinline__ void rhs(const float* mp, const float* y, float I, float* dy) {
         const float u = y[0], v = y[1];
@@ -400,6 +484,14 @@ struct Model<BBX_BARKLEY> {
         y[0] = u + dt * du;
         y[1] = v + dt * (u - v);
     }
+    __device__ static __forceinline__ void update2(const float* mp, float2* y, float2 L, float dt) {
+        const float2 u = y[0], v = y[1];
+        const float2 q = mul2(u, sub2(splat2(1.0f), u));
+        const float2 w = fma2(add2(v, splat2(mp[1])), splat2(-mp[0]), u);
+        const float2 du = fma2(mul2(q, w), splat2(mp[2]), L);
+        y[0] = fma2(splat2(dt), du, u);
+        y[1] = fma2(splat2(dt), sub2(u, v), v);
+    }
     __device__ static __forceinline__ void rhs(const float* mp, const float* y, float I, float* dy) {
         const float u = y[0], v = y[1];
         dy[0] = u * (1.0f - u) * (u - (v + mp[1]) * mp[0]) * mp[2] + I;
@@ -415,6 +507,11 @@ struct Model<BBX_ZFK> {
         const float u = y[0];
         y[0] = u + dt * (u * (u - mp[0]) * (1.0f - u) + L + Is);
     }
+    __device__ static __forceinline__ void update2(const float* mp, float2* y, float2 L, float dt) {
+        const float2 u = y[0];
+        const float2 q = mul2(u, sub2(u, splat2(mp[0])));
+        y[0] = fma2(splat2(dt), fma2(q, sub2(splat2(1.0f), u), L), u);
+    }
     __device__ static __forceinline__ void rhs(const float* mp, const float* y, float I, float* dy) {
         const float u = y[0];
         dy[0] = u * (u - mp[0]) * (1.0f - u) + I;
@@ -427,6 +524,9 @@ struct Model<BBX_DIFFUSION> {
     static constexpr int S = 1;
     __device__ static __forceinline__ void update(const float*, float* y, float L, float Is, float dt) {
         y[0] = y[0] + dt * (L + Is);
+    }
+    __device__ static __forceinline__ void update2(const float*, float2* y, float2 L, float dt) {
+        y[0] = fma2(splat2(dt), L, y[0]);
     }
     __device__ static __forceinline__ void rhs(const float*, const float*, float I, float* dy) { dy[0] = I; }
 };
@@ -810,11 +910,20 @@ struct Model<BBX_BR_FCA> {
 // ---------------------------------------------------------------------------
 
 constexpr int kTileX = 64;  // nodes per brick along x: 32 threads x 2 nodes
-// Consumer warps per CTA (plus one producer warp) for a tile of TY rows: 7
-// warps of 1 or 2 rows each for TY = 7, 14 (two CTAs per SM), 14 warps of 2
-// rows for TY = 28 (one CTA of 480 threads per SM, whose warps share one
-// ring of planes and so finish together).
-__host__ __device__ constexpr int rows_of_threads(int ty) { return ty == 28 ? 14 : 7; }
+// Several steps in one launch: unmasked grids of the light models (the
+// others' steps are long next to a launch, and the further warp it takes would
+// cost the registers their consumers need).
+__host__ __device__ constexpr bool has_flow(bool masked, int s) { return !masked && s <= 2; }
+// Consumer warps per CTA (plus the producer warp, plus the sync warp) for a
+// tile of TY rows: 7 warps of 1 or 2 rows each for TY = 7, 14; for 28 rows 7
+// warps of 4 rows, or 14 warps of 2 rows (one CTA of 480 threads per SM, whose
+// warps share one ring of planes and so finish together) without a sync warp.
+// (8 warps and 16 rows with the sync warp, which load the four schedulers
+// evenly, were slower: 256x256x64 slab 24.9 -> 29.5 us, sheets 60 -> 73 us.)
+__host__ __device__ constexpr int rows_of_threads(int ty, bool flow) { return ty == 28 && !flow ? 14 : 7; }
+__host__ __device__ constexpr int step_threads(int ty, bool masked, int s) {
+    return 32 * rows_of_threads(ty, has_flow(masked, s)) + 32 + (has_flow(masked, s) ? 32 : 0);
+}
 
 // Anisotropy of a step kernel variant: isotropic (c_iso only), anisotropic
 // with the W-tilde sums read from memory, or anisotropic for grids whose
@@ -825,7 +934,8 @@ enum : int { AN_ISO = 0, AN_SUMS = 1, AN_NO_SUMS = 2 };
 // two CTAs of 256 threads allow 128 registers a thread; the masked
 // anisotropic stencil with 2 rows a thread and the surrogate need more; the
 // unmasked isotropic variants fit in 64, so four CTAs hide more latency).
-__host__ __device__ constexpr int ctas_per_sm(bool masked, bool aniso, int ty, bool surr) {
+__host__ __device__ constexpr int ctas_per_sm(bool masked, bool aniso, int ty, bool surr, int s) {
+    if (has_flow(masked, s)) return aniso ? (ty == 28 ? 1 : 2) : 3;
     return (masked && aniso && ty != 7) || ty == 28 || (surr && ty != 7) ? 1 : (!masked && !aniso && !surr ? 4 : 2);
 }
 constexpr int align128(int b) { return (b + 127) & ~127; }
@@ -873,10 +983,11 @@ struct Plan {
     static constexpr int S = Model<MODEL>::S;
     static constexpr int NG = GATES ? 6 : 0;  // variables stored in 16 bits (the gates, last in the state)
     static constexpr int TX = kTileX;
-    static constexpr int RY = rows_of_threads(TY);
-    static constexpr int CTAS = ctas_per_sm(MASKED, ANISO != AN_ISO, TY, SURR);
+    static constexpr int RY = rows_of_threads(TY, has_flow(MASKED, S));
+    static constexpr int CTAS = ctas_per_sm(MASKED, ANISO != AN_ISO, TY, SURR, S);
     static constexpr int CY = TY / RY;  // nodes per thread along y (each a pair in x)
-    static constexpr int THREADS = 32 * RY + 32;  // consumer warps + producer warp
+    static constexpr bool FLOW = has_flow(MASKED, S);
+    static constexpr int THREADS = step_threads(TY, MASKED, S);  // consumer warps + producer warp (+ sync warp)
     static constexpr int UW = TX + 8;   // x from x0-4 to x0+TX+3 (16-byte aligned start)
     static constexpr int UH = TY + 2;   // y from y0-1 to y0+TY
     static constexpr int MW = TX + 32;  // mask bytes: x from x0-16 (16-byte aligned start)
@@ -886,7 +997,9 @@ struct Plan {
     static constexpr int M_RAW = MASKED ? MW * UH : 0;
     static constexpr int U_OFF = 0;
     static constexpr int M_OFF = U_OFF + align128(U_RAW);
-    static constexpr int A_STAGE = M_OFF + align128(M_RAW);
+    // (each stage ends with its two mbarriers, so a stage's address gives them)
+    static constexpr int A_BAR = M_OFF + align128(M_RAW);
+    static constexpr int A_STAGE = A_BAR + 128;
     static constexpr uint32_t A_BYTES = U_RAW + M_RAW;
     // ring B, one stage per computed plane: the node's own unit fibre and
     // W-tilde sums (3 x TX x TY floats each), the other variables
@@ -899,17 +1012,19 @@ struct Plan {
     static constexpr int D_OFF = F_OFF + F_RAW;    // (each part a multiple of 128 bytes)
     static constexpr int S_OFF = D_OFF + D_RAW;
     static constexpr int G_OFF = S_OFF + S32_RAW;
-    static constexpr int B_STAGE = align128(F_RAW + D_RAW + S_RAW);
+    static constexpr int B_BAR = align128(F_RAW + D_RAW + S_RAW);
+    static constexpr int B_STAGE = B_BAR + 128;
     static constexpr uint32_t B_BYTES = F_RAW + D_RAW + S_RAW;
     static constexpr bool HAS_B = B_BYTES > 0;
-    static constexpr int BUDGET = (CTAS == 1 ? 200 : 112) * 1024;  // dynamic shared memory per CTA
-    static constexpr int NB = !HAS_B ? 0 : (3 * B_STAGE + 5 * A_STAGE <= BUDGET ? 3 : 2);
+    static constexpr int BUDGET = (CTAS == 1 ? 200 : (CTAS == 2 ? 112 : (CTAS == 3 ? 72 : 54))) * 1024;  // dynamic shared memory per CTA
+    static constexpr int NB_FIT = HAS_B ? (BUDGET - 5 * A_STAGE) / B_STAGE : 0;
+    static constexpr int NB = !HAS_B ? 0 : (NB_FIT > 5 ? 5 : (NB_FIT < 2 ? 2 : NB_FIT));
     static constexpr int NA_FIT = (BUDGET - NB * B_STAGE) / A_STAGE;
     static constexpr int NA = NA_FIT > 8 ? 8 : (NA_FIT < 4 ? 4 : NA_FIT);
     static constexpr int WBUF = SURR ? RY * 2048 : 0;  // per consumer warp: 64 rows of 32 bytes
-    static constexpr int BAR_OFF = NA * A_STAGE + NB * B_STAGE + WBUF;
-    // stages, warp buffers, full/empty barriers of both rings, piece contexts
-    static constexpr int SMEM = 128 + BAR_OFF + 2 * (NA + NB) * 8 + NA * 176;
+    static constexpr int RING_OFF = NA * A_STAGE + NB * B_STAGE + WBUF;
+    // stages with their barriers, warp buffers, piece contexts
+    static constexpr int SMEM = 128 + RING_OFF + NA * 176;
     static_assert(TY % RY == 0 && CY >= 1, "tile rows must be a multiple of the thread rows");
     static_assert(U_RAW % 16 == 0 && F_RAW % 128 == 0 && D_RAW % 128 == 0 && S32_RAW % 128 == 0, "stage layout");
 };
@@ -932,62 +1047,45 @@ struct Nb {
 // sum_j (f_j f_k at p + q_j minus at p - q_j), with a void neighbour's fibre
 // replaced by f at p (computed once per grid, k_divergence).
 
-// (L u)_p for a node whose 18 neighbours are all tissue: the weights of
-// Eq. (Lu) with psi = 1 everywhere, in difference form.  c_perp = Dperp/h^2,
-// c_d = (Dpar-Dperp)/h^2, c_dh = c_d/2, c_s = c_d/4.
-template <int ANISO>
-__device__ __forceinline__ float lap_interior(const Coef& a, const Nb& n, F3 f, F3 sd) {
-    if (!ANISO) {
-        return a.c_iso * (((n.xp + n.xm) + (n.yp + n.ym)) + (n.zp + n.zm) - 6.0f * n.u0);
-    }
-    const float Dxx = fmaf(a.c_d, f.x * f.x, a.c_perp);
-    const float Dyy = fmaf(a.c_d, f.y * f.y, a.c_perp);
-    const float Dzz = fmaf(a.c_d, f.z * f.z, a.c_perp);
-    const float hx = a.c_dh * f.x;
-    const float Dxy = hx * f.y, Dxz = hx * f.z, Dyz = a.c_dh * f.y * f.z;
-    const float two_u = 2.0f * n.u0;
-    float L = Dxx * ((n.xp + n.xm) - two_u);
-    L = fmaf(Dyy, (n.yp + n.ym) - two_u, L);
-    L = fmaf(Dzz, (n.zp + n.zm) - two_u, L);
-    if (ANISO == AN_SUMS) {
-        float dv = sd.x * (n.xp - n.xm);
-        dv = fmaf(sd.y, n.yp - n.ym, dv);
-        dv = fmaf(sd.z, n.zp - n.zm, dv);
-        L = fmaf(a.c_s, dv, L);
-    }
-    L = fmaf(Dxy, (n.pp + n.mm) - (n.pm + n.mp), L);
-    L = fmaf(Dxz, (n.xpzp + n.xmzm) - (n.xpzm + n.xmzp), L);
-    L = fmaf(Dyz, (n.ypzp + n.ymzm) - (n.ypzm + n.ymzp), L);
-    return L;
-}
+// The differences of V around a pair of nodes from which (L u)_p is formed:
+// second differences along the axes (void neighbours counted out), the
+// four-point cross differences, and the central differences for W-tilde.
+struct Diffs {
+    float2 xx, yy, zz;  // u(+) + u(-) - (psi(+) + psi(-)) u0
+    float2 xy, xz, yz;  // (u(+,+) - u(+,-)) - (u(-,+) - u(-,-))
+    float2 x1, y1, z1;  // u(+) - u(-)
+};
 
-// (L u)_p for a node of an unmasked grid whose y and z neighbours are inside
-// the array; px, mx in {0, 1} are psi of the x+1 and x-1 neighbours (0 only
-// at the array's x faces).
-template <int ANISO>
-__device__ __forceinline__ float lap_xbound(const Coef& a, const Nb& n, float px, float mx, F3 f, F3 sd) {
-    const float ex = px * (n.xp - n.u0) + mx * (n.xm - n.u0);
-    if (!ANISO) {
-        return a.c_iso * ((ex + (n.yp + n.ym)) + (n.zp + n.zm) - 4.0f * n.u0);
+// (L u)_p of Eq. (Lu) for the pair, from the unit fibres f: with D = Dperp I +
+// (Dpar - Dperp) f f^T the weights sum to
+//   c_perp (xx + yy + zz) + c_d f.(H f), H_kk the second differences and
+//   H_jk a quarter of the cross differences, plus c_s times the W-tilde sums'
+// dot product with the central differences.  c_perp = Dperp/h^2, c_d =
+// (Dpar-Dperp)/h^2, c_s = c_d/4.  PLANAR: no z terms (a sheet).  Adding a
+// vanishing W-tilde term leaves L as it is, so the variants with and without
+// the sums agree bitwise where they all vanish.
+template <int ANISO, bool PLANAR>
+__device__ __forceinline__ float2 lap_pair(const Coef& a, const Diffs& d, const float2* f, const float2* sd) {
+    const float2 hy = mul2(splat2(0.5f), f[1]);
+    float2 t1 = fma2(hy, d.xy, mul2(f[0], d.xx));
+    float2 t2 = mul2(f[1], d.yy);
+    float2 lap = add2(d.xx, d.yy);
+    float2 q;
+    if (PLANAR) {
+        q = fma2(f[1], t2, mul2(f[0], t1));
+    } else {
+        const float2 hz = mul2(splat2(0.5f), f[2]);
+        t1 = fma2(hz, d.xz, t1);
+        t2 = fma2(hz, d.yz, t2);
+        lap = add2(d.xx, add2(d.yy, d.zz));
+        q = fma2(f[2], mul2(f[2], d.zz), fma2(f[1], t2, mul2(f[0], t1)));
     }
-    const float Dxx = fmaf(a.c_d, f.x * f.x, a.c_perp);
-    const float Dyy = fmaf(a.c_d, f.y * f.y, a.c_perp);
-    const float Dzz = fmaf(a.c_d, f.z * f.z, a.c_perp);
-    const float hx = a.c_dh * f.x;
-    const float Dxy = hx * f.y, Dxz = hx * f.z, Dyz = a.c_dh * f.y * f.z;
-    const float two_u = 2.0f * n.u0;
-    float L = Dxx * ex;
-    L = fmaf(Dyy, (n.yp + n.ym) - two_u, L);
-    L = fmaf(Dzz, (n.zp + n.zm) - two_u, L);
+    float2 L = fma2(splat2(a.c_d), q, mul2(splat2(a.c_perp), lap));
     if (ANISO == AN_SUMS) {
-        float dv = (px * mx) * sd.x * (n.xp - n.xm);
-        dv = fmaf(sd.y, n.yp - n.ym, dv);
-        dv = fmaf(sd.z, n.zp - n.zm, dv);
-        L = fmaf(a.c_s, dv, L);
+        float2 dv = fma2(sd[1], d.y1, mul2(sd[0], d.x1));
+        if (!PLANAR) dv = fma2(sd[2], d.z1, dv);
+        L = fma2(splat2(a.c_s), dv, L);
     }
-    L = fmaf(Dxy, px * (n.pp - n.pm) + mx * (n.mm - n.mp), L);
-    L = fmaf(Dxz, px * (n.xpzp - n.xpzm) + mx * (n.xmzm - n.xmzp), L);
-    L = fmaf(Dyz, (n.ypzp + n.ymzm) - (n.ypzm + n.ymzp), L);
     return L;
 }
 
@@ -1176,6 +1274,89 @@ struct PieceSlot : Coef {
 static_assert(sizeof(PieceSlot) <= 176, "piece ring slot size");
 
 
+// The kinetics step of a pair of nodes: y the state at the start of the step
+// (the half-step voltage under Lie splitting), L the diffusion term (0 then),
+// Is the stimulus.  All 32 lanes of a warp call it.
+template <int MODEL, bool SURR, bool GEN>
+__device__ __forceinline__ void react_pair(const PieceSlot& a, const float* mp, float dt, unsigned char* wbufs,
+                                           const bool* live, float2* y, float2 L, float2 Is) {
+    constexpr int S = Model<MODEL>::S;
+    if constexpr (MODEL == BBX_BR || MODEL == BBX_BR_MRL || MODEL == BBX_BR_FCA) {
+        float ys[2][S];
+        const float Ls[2] = {L.x, L.y}, Iss[2] = {Is.x, Is.y};
+#pragma unroll
+        for (int v = 0; v < S; ++v) {
+            ys[0][v] = y[v].x;
+            ys[1][v] = y[v].y;
+        }
+        if constexpr (SURR && MODEL == BBX_BR) {
+            // the surrogate where the state is inside the training envelope and V
+            // below the upstroke threshold; the exact model elsewhere
+            const SurrogateData* W = a.surr;
+            bool want[2] = {false, false};
+            if (W) {
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    bool in = live[e] && ys[e][0] < W->v_up;
+#pragma unroll
+                    for (int v = 0; v < S; ++v) in = in && ys[e][v] >= W->norm[32 + v] && ys[e][v] <= W->norm[40 + v];
+                    want[e] = in;
+                }
+            }
+            if (__any_sync(0xffffffffu, want[0] || want[1])) {
+                float dsur[2][8];
+                surrogate_warp64(W, wbufs + (threadIdx.x >> 5) * 2048, ys, dsur);
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    if (want[e]) {
+#pragma unroll
+                        for (int v = 0; v < S; ++v) ys[e][v] += dsur[e][v];
+                        ys[e][0] += dt * (Ls[e] + Iss[e]);
+                    } else {
+                        Model<MODEL>::update(mp, ys[e], Ls[e], Iss[e], dt);
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int e = 0; e < 2; ++e) Model<MODEL>::update(mp, ys[e], Ls[e], Iss[e], dt);
+            }
+        } else {
+            // tabulated Rush-Larsen coefficients (of BBX_BR in the general
+            // variants only, so the default kernel carries no code for them)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                if constexpr (MODEL != BBX_BR) {
+                    Model<MODEL>::update_tab(mp, a.tab, ys[e], Ls[e], Iss[e], dt);
+                } else {
+                    if (GEN && a.tab)
+                        Model<MODEL>::update_tab(mp, a.tab, ys[e], Ls[e], Iss[e], dt);
+                    else
+                        Model<MODEL>::update(mp, ys[e], Ls[e], Iss[e], dt);
+                }
+            }
+        }
+#pragma unroll
+        for (int v = 0; v < S; ++v) y[v] = make_float2(ys[0][v], ys[1][v]);
+    } else {
+        const float2 src = add2(L, Is);
+        if (GEN && a.rk4) {
+            float ys[2][S];
+#pragma unroll
+            for (int v = 0; v < S; ++v) {
+                ys[0][v] = y[v].x;
+                ys[1][v] = y[v].y;
+            }
+            rk4_update<MODEL>(mp, ys[0], src.x, 0.0f, dt);
+            rk4_update<MODEL>(mp, ys[1], src.y, 0.0f, dt);
+#pragma unroll
+            for (int v = 0; v < S; ++v) y[v] = make_float2(ys[0][v], ys[1][v]);
+        } else {
+            Model<MODEL>::update2(mp, y, src, dt);
+        }
+    }
+}
+
+
 // Barrier over the consumer warps only (named barrier 1), returning the OR of
 // a per-thread predicate.
 __device__ __forceinline__ bool consumers_sync_or(bool p, int nthreads) {
@@ -1221,7 +1402,7 @@ __device__ __forceinline__ int tile_row_of(int4 pc, int off) {
 // taken per plane.
 template <int MODEL, bool MASKED, int ANISO, int TY, bool SURR = false, bool PLANAR = false, bool GEN = false,
           int GATES = GATES_F32>
-__global__ void __launch_bounds__(32 * rows_of_threads(TY) + 32, ctas_per_sm(MASKED, ANISO != AN_ISO, TY, SURR))
+__global__ void __launch_bounds__(step_threads(TY, MASKED, Model<MODEL>::S), ctas_per_sm(MASKED, ANISO != AN_ISO, TY, SURR, Model<MODEL>::S))
 step_kernel(const __grid_constant__ LaunchArgs L) {
     using P = Plan<MODEL, MASKED, ANISO, TY, SURR, GATES>;
     static_assert(GATES == GATES_F32 || (MODEL == BBX_BR && !SURR), "16-bit gates: Beeler-Reuter without surrogate");
@@ -1239,13 +1420,17 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
     unsigned char* smem = smem_raw + ((128u - (smem_addr(smem_raw) & 127u)) & 127u);
     unsigned char* bstages = smem + NS * P::A_STAGE;    // ring B
     unsigned char* wbufs = bstages + NB * P::B_STAGE;   // surrogate buffers (SURR only)
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + P::BAR_OFF);
-    uint64_t* empty = full + NS;
-    uint64_t* fullb = empty + NS;
-    uint64_t* emptyb = fullb + NB;
-    PieceSlot* ring = reinterpret_cast<PieceSlot*>(emptyb + NB);
+    PieceSlot* ring = reinterpret_cast<PieceSlot*>(smem + P::RING_OFF);
+    // full (the copies have landed) and empty (the consumer warps are done)
+    // barriers of a stage of ring A and of ring B
+    auto full = [&](int slot) { return reinterpret_cast<uint64_t*>(smem + slot * P::A_STAGE + P::A_BAR); };
+    auto empty = [&](int slot) { return full(slot) + 1; };
+    auto fullb = [&](int slot) { return reinterpret_cast<uint64_t*>(bstages + slot * P::B_STAGE + P::B_BAR); };
+    auto emptyb = [&](int slot) { return fullb(slot) + 1; };
     __shared__ double red_scratch[32];
     __shared__ volatile int abort_flag;
+    // launch of several steps: planes each consumer warp has left, loads allowed
+    __shared__ int sync_done[P::RY], sync_allowed;
 
     const int tid = threadIdx.x;
     const int warp = tid / 32, lane = tid % 32;
@@ -1269,14 +1454,16 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
     const uint32_t b_bytes = skip_d ? P::B_BYTES - P::D_RAW : P::B_BYTES;
     if (tid == 0) {
         for (int s = 0; s < NS; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], NCW);
+            mbar_init(full(s), 1);
+            mbar_init(empty(s), NCW);
         }
         for (int s = 0; s < NB; ++s) {
-            mbar_init(&fullb[s], 1);
-            mbar_init(&emptyb[s], NCW);
+            mbar_init(fullb(s), 1);
+            mbar_init(emptyb(s), NCW);
         }
         abort_flag = 0;
+        for (int w = 0; w < NCW; ++w) sync_done[w] = 0;
+        sync_allowed = 0;
         mbar_init_fence();
     }
     __syncthreads();
@@ -1289,62 +1476,69 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
     const int piece_begin = blockIdx.x * L.cta_stride, piece_end = piece_begin + L.cta_count[blockIdx.x];
-    int issued = 0;   // producer lane 0: plane loads issued (ring A)
-    int issuedb = 0;  // producer lane 0: computed planes issued (ring B)
+    int issued = 0;   // producer: plane loads issued (ring A)
+    int issuedb = 0;  // producer: computed planes issued (ring B)
+    const int n_pieces = piece_end - piece_begin;
+    // A launch of several steps: odd CTAs walk their share (a range of the
+    // schedule's planes) from its end, so that neighbours along z begin every
+    // step at their common border and no CTA waits there for planes that its
+    // neighbour has only just done.
+    const bool down = P::FLOW && L.n_steps > 1 && (blockIdx.x & 1);
+
+    auto piece_slot = [&](int i) { return down ? piece_end - 1 - i : piece_begin + i; };
 
     if (warp == NCW) {
         // ---------------- producer warp ----------------
-        if (lane == 0) {
-            bool stop = false;
-            int lp = 0;
-            // the loads the first plane waits for, issued together: the first
-            // piece (its slot always exists) and, for one grid, its t, n, parity
-            int4 pc_next = L.pieces[piece_begin];
-            TissueDyn d0 = {};
-            bool ticketed = !L.single;  // a single-grid launch takes one start ticket per CTA
-            if (L.single) {
-                const TissueDyn* D = L.t0.dyn;
-                d0.t = D->t;
-                d0.n = D->n;
-                d0.cur = D->cur;
+        bool stop = false;
+        int lp = 0;
+        // the loads the first plane waits for, issued together: the first
+        // piece (its slot always exists) and, for one grid, its t, n, parity
+        int4 pc_next = L.pieces[n_pieces > 0 ? piece_slot(0) : piece_begin];
+        TissueDyn d0 = {};
+        bool ticketed = !L.single;  // a single-grid launch takes one start ticket per CTA
+        if (L.single) {
+            const TissueDyn* D = L.t0.dyn;
+            d0.t = D->t;
+            d0.n = D->n;
+            d0.cur = D->cur;
+        }
+        // ring B copies of the computed plane z (tile rows from y0) of grid T
+        auto load_b = [&](const TissueArgs* T, int src, int x0, int y0, int z, int bslot, uint64_t* bar) {
+            unsigned char* sb = bstages + bslot * P::B_STAGE;
+            if (ANISO) {
+                tma_load_4d(sb + P::F_OFF, &T->tm_f, x0, y0, z, 0, bar);
+                if (ANISO == AN_SUMS && !skip_d) tma_load_4d(sb + P::D_OFF, &T->tm_d, x0, y0, z, 0, bar);
             }
-            // Single-grid launch of an unmasked grid with a known parity: the
-            // first piece from the schedule's shape and its first plane copies
-            // (three planes; two tile rows of a sheet) issued now, expected on
-            // their barriers but not yet arrived on (the arrival follows the
-            // piece context, below).
-            // ring B copies of the computed plane z (tile rows from y0) of grid T
-            auto load_b = [&](const TissueArgs* T, int src, int x0, int y0, int z, int bslot, uint64_t* bar) {
-                unsigned char* sb = bstages + bslot * P::B_STAGE;
-                if (ANISO) {
-                    tma_load_4d(sb + P::F_OFF, &T->tm_f, x0 + 4, y0, z, 0, bar);  // fibres stored from x = -4
-                    if (ANISO == AN_SUMS && !skip_d) tma_load_4d(sb + P::D_OFF, &T->tm_d, x0, y0, z, 0, bar);
-                }
-                if (S > 1 && S32 > 1) tma_load_4d(sb + P::S_OFF, &T->tm_s[src], x0, y0, z, 1, bar);
-                if (NG) tma_load_4d(sb + P::G_OFF, &T->tm_g[src], x0, y0, z, 0, bar);
-            };
-            bool early = false;
-            int n_early = 0;
-            int4 pc_early = make_int4(0, 0, 0, 0);
-            if (L.single && L.cur_hint >= 0 && L.reg_len > 0 && !L.poison_first_load) {
-                const long long p0 = (long long)blockIdx.x * L.reg_planes / L.reg_ctas;
-                const long long p1 = ((long long)blockIdx.x + 1) * L.reg_planes / L.reg_ctas;
-                if (p1 > p0) {
-                    const int col = (int)(p0 / L.reg_len), z0 = L.reg_z0 + (int)(p0 % L.reg_len);
-                    const int z1 = (int)min((long long)(L.reg_z0 + L.reg_len), z0 + (p1 - p0));
-                    pc_early = make_int4((col % L.reg_nbx) * TX, (col / L.reg_nbx) * L.reg_ty, z0, z1);
-                    early = true;
-                    const TissueArgs* T = &L.t0;
-                    const int src = L.cur_hint;
-                    const int nl = PLANAR ? z1 - z0 : z1 - z0 + 2;
-                    n_early = PLANAR ? min(nl, 2) : 3;  // (3D: at most 2 computed planes; NB >= 2)
-                    if (HB && PLANAR && n_early > NB) n_early = NB;
+            if (S > 1 && S32 > 1) tma_load_4d(sb + P::S_OFF, &T->tm_s[src], x0, y0, z, 1, bar);
+            if (NG) tma_load_4d(sb + P::G_OFF, &T->tm_g[src], x0, y0, z, 0, bar);
+        };
+        // Single-grid launch of an unmasked grid with a known parity: the
+        // first piece from the schedule's shape and its first plane copies
+        // (three planes; two tile rows of a sheet) issued now, expected on
+        // their barriers but not yet arrived on (the arrival follows the
+        // piece context, below).
+        bool early = false;
+        int n_early = 0;
+        int4 pc_early = make_int4(0, 0, 0, 0);
+        if (L.single && L.cur_hint >= 0 && L.reg_len > 0 && !L.poison_first_load && !down) {
+            const long long p0 = (long long)blockIdx.x * L.reg_planes / L.reg_ctas;
+            const long long p1 = ((long long)blockIdx.x + 1) * L.reg_planes / L.reg_ctas;
+            if (p1 > p0) {
+                const int col = (int)(p0 / L.reg_len), z0 = L.reg_z0 + (int)(p0 % L.reg_len);
+                const int z1 = (int)min((long long)(L.reg_z0 + L.reg_len), z0 + (p1 - p0));
+                pc_early = make_int4((col % L.reg_nbx) * TX, (col / L.reg_nbx) * L.reg_ty, z0, z1);
+                early = true;
+                const TissueArgs* T = &L.t0;
+                const int src = L.cur_hint;
+                const int nl = PLANAR ? z1 - z0 : z1 - z0 + 2;
+                n_early = PLANAR ? min(nl, 2) : 3;  // (3D: at most 2 computed planes; NB >= 2)
+                if (HB && PLANAR && n_early > NB) n_early = NB;
+                if (lane == 0) {
 #pragma unroll 1
                     for (int off = 0; off < n_early; ++off) {
-                        const int z = PLANAR ? 0 : z0 - 1 + off;
-                        if (z < 0 || z >= T->nz) continue;
+                        const int z = PLANAR ? 0 : z0 - 1 + off;  // (outside the array: the copy fills zeros)
                         const int y0 = tile_row_of<PLANAR, TY>(pc_early, off);
-                        uint64_t* bar = &full[off];
+                        uint64_t* bar = full(off);
                         unsigned char* st = smem + off * P::A_STAGE;
                         const bool halo = !PLANAR && ((off == 0) || (off == nl - 1));
                         mbar_expect_tx(bar, P::A_BYTES);
@@ -1352,430 +1546,540 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
                         if (MASKED) tma_load_3d(st + P::M_OFF, &T->tm_m, pc_early.x - 16, y0 - 1, z, bar);
                         if (HB && !halo) {  // computed plane b = off - 1 (3D) or off (sheet): slot b
                             const int b = PLANAR ? off : off - 1;
-                            mbar_expect_tx(&fullb[b], b_bytes);
-                            load_b(T, src, pc_early.x, y0, z, b, &fullb[b]);
+                            mbar_expect_tx(fullb(b), b_bytes);
+                            load_b(T, src, pc_early.x, y0, z, b, fullb(b));
                         }
                     }
                 }
             }
-            if (L.single && L.cur_hint >= 0 &&
-                (d0.cur != L.cur_hint ||
-                 (early && (pc_early.x != pc_next.x || pc_early.y != pc_next.y || pc_early.z != pc_next.z ||
-                            pc_early.w != pc_next.w))))
-                atomicOr(L.err, ERRBIT_HINT);
-            for (int pi = piece_begin; pi < piece_end && !stop; ++pi, ++lp) {
-                const int4 pc = pc_next;
-                if (pi + 1 < piece_end) pc_next = L.pieces[pi + 1];
-                const TissueArgs* T = L.single ? &L.t0 : L.tissues + L.piece_tissue[pi];
-                const TissueDyn* D = T->dyn;
-                const int src = L.single ? (L.cur_hint >= 0 ? L.cur_hint : d0.cur) : D->cur;
-                const int nz = T->nz;
-                const int nload = PLANAR ? pc.w - pc.z : pc.w - pc.z + 2;
-                for (int off = 0; off < nload; ++off) {
-                    const int slot = issued % NS;
-                    const bool comp = PLANAR || (off >= 1 && off <= pc.w - pc.z);  // a computed plane: ring B too
-                    const int bslot = NB ? issuedb % NB : 0;
-                    if (!ticketed && issued == NS) {
-                        // the ring is full: the ticket's round trip overlaps the copies
-                        start_ticket(L, d0);
-                        ticketed = true;
-                    }
-                    if (L.poison_first_load && blockIdx.x == 0 && issued == 0) {
-                        // fault injection: wait for an empty-slot phase that no
-                        // consumer completes; the bounded wait runs out
-                        (void)mbar_wait_bounded(&empty[slot], 0, L.wait_limit);
-                        stop = true;
-                    } else if (issued >= NS &&
-                               !mbar_wait_bounded(&empty[slot], ((issued / NS) - 1) & 1, L.wait_limit)) {
-                        stop = true;
-                    } else if (HB && comp && issuedb >= NB &&
-                               !mbar_wait_bounded(&emptyb[bslot], ((issuedb / NB) - 1) & 1, L.wait_limit)) {
-                        stop = true;
-                    }
-                    if (stop || abort_flag) {
-                        stop = true;
-                        break;
-                    }
-                    if (off == 0) {
-                        PieceSlot& r = ring[lp % NS];
-                        const double tn = L.single ? d0.t : D->t;
-                        r.x0 = pc.x; r.y0 = pc.y; r.z0 = pc.z; r.z1 = pc.w;
-                        r.nx = T->nx; r.ny = T->ny; r.nz = nz; r.px = T->px;
-                        r.plane = T->plane; r.vol = T->vol;
-                        r.dst = T->state[src ^ 1];
-                        r.dst16 = T->gate16[src ^ 1];
-                        r.act = T->act;
-                        r.stim = T->stim;
-                        r.stim_amp = (T->stim && T->stim_amp != 0.0f && tn >= T->t_on && tn < T->t_off) ? T->stim_amp
-                                                                                                       : 0.0f;
-                        r.dt = T->dt;
-                        r.theta = T->theta;
-                        r.step_next = (int)((L.single ? d0.n : D->n) + 1);
-                        r.split = T->split;
-                        r.rk4 = T->rk4;
-                        r.c_perp = T->c_perp; r.c_d = T->c_d; r.c_dh = T->c_dh; r.c_s = T->c_s; r.c_iso = T->c_iso;
-                        r.surr = T->surr;
-                        r.tab = T->tab;
+        }
+        if (lane == 0 && L.single && L.cur_hint >= 0 &&
+            (d0.cur != L.cur_hint ||
+             (early && (pc_early.x != pc_next.x || pc_early.y != pc_next.y || pc_early.z != pc_next.z ||
+                        pc_early.w != pc_next.w))))
+            atomicOr(L.err, ERRBIT_HINT);
+
+        if (lane == 0) {
+            const bool stim_s = L.t0.stim && L.t0.stim_amp != 0.0f;
+            double t_now = d0.t;  // start time of the step (single-grid launch)
+            // the slots and the parities of the empty phases to wait for (a
+            // fresh barrier's preceding phase counts as complete)
+            int as = 0, ap = 1, bs = 0, bp = 1;
+            int n_ready = 0;  // loads the sync warp allows (launch of several steps)
+            for (int s = 0; s < L.n_steps && !stop; ++s) {
+                for (int i = 0; i < n_pieces && !stop; ++i, ++lp) {
+                    const int pi = piece_slot(i);
+                    const int4 pc = pc_next;
+                    if (n_pieces > 1) pc_next = L.pieces[piece_slot(i + 1 < n_pieces ? i + 1 : 0)];
+                    const TissueArgs* T = L.single ? &L.t0 : L.tissues + L.piece_tissue[pi];
+                    const TissueDyn* D = L.single ? nullptr : T->dyn;
+                    const int src = (L.single ? (L.cur_hint >= 0 ? L.cur_hint : d0.cur) : D->cur) ^ (s & 1);
+                    const int nz = MASKED ? (L.single ? L.t0.nz : T->nz) : 0;
+                    const int ncomp = pc.w - pc.z, nload = PLANAR ? ncomp : ncomp + 2;
+                    // plane of the next load (a sheet: its tile row), walked by dir
+                    const int dir = down ? -1 : 1;
+                    int zt = down ? (PLANAR ? pc.w - 1 : pc.w) : (PLANAR ? pc.z : pc.z - 1);
+                    for (int off = 0; off < nload; ++off, zt += dir) {
+                        const bool comp = PLANAR || (off >= 1 && off <= ncomp);  // a computed plane: ring B too
+                        if (!ticketed && issued == NS) {
+                            // the ring is full: the ticket's round trip overlaps the copies
+                            start_ticket(L, d0);
+                            ticketed = true;
+                        }
+                        if (L.poison_first_load && blockIdx.x == 0 && issued == 0) {
+                            // fault injection: wait for an empty-slot phase that no
+                            // consumer completes; the bounded wait runs out
+                            (void)mbar_wait_bounded(empty(0), 0, L.wait_limit);
+                            stop = true;
+                        } else if (!mbar_wait_bounded(empty(as), ap, L.wait_limit)) {
+                            stop = true;
+                        } else if (HB && comp && !mbar_wait_bounded(emptyb(bs), bp, L.wait_limit)) {
+                            stop = true;
+                        }
+                        if (P::FLOW && s > 0 && issued >= n_ready && !stop) {
+                            const long long t0 = clock64();
+                            while ((n_ready = ld_shared_acquire(&sync_allowed)) <= issued) {
+                                if (abort_flag || clock64() - t0 > L.wait_limit) {
+                                    stop = true;
+                                    break;
+                                }
+                            }
+                        }
+                        if (stop || abort_flag) {
+                            stop = true;
+                            break;
+                        }
+                        if (off == 0) {
+                            PieceSlot& r = ring[lp % NS];
+                            r.x0 = pc.x; r.y0 = pc.y; r.z0 = pc.z; r.z1 = pc.w;
+                            r.dst = L.single ? (src ? L.t0.state[0] : L.t0.state[1]) : T->state[src ^ 1];
+                            r.dst16 = L.single ? (src ? L.t0.gate16[0] : L.t0.gate16[1]) : T->gate16[src ^ 1];
+                            r.stim_amp = 0.0f;
+                            if (L.single ? stim_s : T->stim && T->stim_amp != 0.0f) {
+                                double tn = L.single ? t_now : D->t;
+                                if (!L.single)
+                                    for (int q = 0; q < s; ++q) tn = tn + T->dt_d;
+                                if (tn >= T->t_on && tn < T->t_off) r.stim_amp = T->stim_amp;
+                            }
+                            r.step_next = (int)((L.single ? d0.n : D->n) + s + 1);
+                            if (!L.single || lp < NS) {  // the rest of a single grid's contexts stays in the ring
+                                r.nx = T->nx; r.ny = T->ny; r.nz = T->nz; r.px = T->px;
+                                r.plane = T->plane; r.vol = T->vol;
+                                r.act = T->act;
+                                r.stim = T->stim;
+                                r.dt = T->dt;
+                                r.theta = T->theta;
+                                r.split = T->split;
+                                r.rk4 = T->rk4;
+                                r.c_perp = T->c_perp; r.c_d = T->c_d; r.c_dh = T->c_dh; r.c_s = T->c_s; r.c_iso = T->c_iso;
+                                r.surr = T->surr;
+                                r.tab = T->tab;
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) r.mp[i] = T->mp[i];
-                    }
-                    const int z = PLANAR ? 0 : pc.z - 1 + off;
-                    const int y0 = tile_row_of<PLANAR, TY>(pc, off);  // first row of the tile
-                    uint64_t* bar = &full[slot];
-                    unsigned char* st = smem + slot * P::A_STAGE;
-                    if (early && lp == 0 && off < n_early) {
-                        mbar_arrive(bar);  // its copies were issued at the start
-                        if (HB && comp) mbar_arrive(&fullb[bslot]);
-                    } else if (z < 0 || z >= nz) {
-                        mbar_arrive(bar);  // plane outside the array: nothing to load (never a computed one)
-                    } else {
-                        mbar_arrive_expect_tx(bar, P::A_BYTES);
-                        tma_load_3d(st + P::U_OFF, &T->tm_u[src], pc.x - 4, y0 - 1, z, bar);
-                        if (MASKED) tma_load_3d(st + P::M_OFF, &T->tm_m, pc.x - 16, y0 - 1, z, bar);
+                                for (int q = 0; q < 8; ++q) r.mp[q] = T->mp[q];
+                            }
+                        }
+                        const int z = PLANAR ? 0 : zt;
+                        const int y0 = PLANAR ? zt * TY : pc.y;  // first row of the tile
+                        uint64_t* bar = full(as);
+                        unsigned char* st = smem + as * P::A_STAGE;
+                        if (early && issued < n_early) {
+                            mbar_arrive(bar);  // its copies were issued at the start
+                            if (HB && comp) mbar_arrive(fullb(bs));
+                        } else if (MASKED && (z < 0 || z >= nz)) {
+                            mbar_arrive(bar);  // plane outside the array: not read (never a computed one)
+                        } else {
+                            // (an unmasked grid's plane outside the array: the copy fills zeros)
+                            mbar_arrive_expect_tx(bar, P::A_BYTES);
+                            tma_load_3d(st + P::U_OFF, &T->tm_u[src], pc.x - 4, y0 - 1, z, bar);
+                            if (MASKED) tma_load_3d(st + P::M_OFF, &T->tm_m, pc.x - 16, y0 - 1, z, bar);
+                            if (HB && comp) {
+                                mbar_arrive_expect_tx(fullb(bs), b_bytes);
+                                load_b(T, src, pc.x, y0, z, bs, fullb(bs));
+                            }
+                        }
+                        ++issued;
+                        if (++as == NS) {
+                            as = 0;
+                            ap ^= 1;
+                        }
                         if (HB && comp) {
-                            mbar_arrive_expect_tx(&fullb[bslot], b_bytes);
-                            load_b(T, src, pc.x, y0, z, bslot, &fullb[bslot]);
+                            ++issuedb;
+                            if (++bs == NB) {
+                                bs = 0;
+                                bp ^= 1;
+                            }
                         }
                     }
-                    ++issued;
-                    if (HB && comp) ++issuedb;
                 }
+                if (L.single) t_now = t_now + L.t0.dt_d;
             }
             if (!ticketed) start_ticket(L, d0);  // every CTA takes it, also on a short or aborted run
             if (stop) abort_flag = 1;
         }
         __syncwarp();
+    } else if (P::FLOW && warp == NCW + 1) {
+        // ---------------- sync warp (launch of several steps) ----------------
+        // flags[] holds, per column and computed plane, the running number of
+        // the last step done there.  A plane of V may be copied for step s
+        // (after the first) once the step before is done at that plane in the
+        // 3 x 3 columns around it (the box's halo; a sheet: the 3 x 3 tiles):
+        // the copies of planes z-1 .. z+1 then also show that no CTA still
+        // reads, for the step before, the plane z that step s overwrites in
+        // the other buffer.  This warp sets the flags of the planes its CTA
+        // has done and tells the producer how many loads may go; in the
+        // producer itself the fence before a flag (1100 to 2300 cycles, the
+        // SM's stores in flight) and the flags' round trips would each stall
+        // the copies (512x512x256 slab: 2970 cycles a plane against 2420).
+        if (L.n_steps > 1 && n_pieces > 0) {
+            int4 fg_pc = L.pieces[piece_slot(0)], al_pc = fg_pc;
+            PieceFlags fg_pf = L.piece_flags[piece_slot(0)], al_pf = fg_pf;
+            // next flag to set, next load to allow: the piece and the place in it
+            int fg_i = 0, fg_t = 0, fg_step = 0, n_flag = 0;
+            int al_i = 0, al_off = 0, al_step = 1, n_allow = 0;
+            int planes = 0;  // computed planes of a step
+            for (int i = 0; i < n_pieces; ++i) {
+                const int4 q = n_pieces > 1 ? L.pieces[piece_slot(i)] : fg_pc;
+                planes += q.w - q.z;
+                n_allow += q.w - q.z + (PLANAR ? 0 : 2);
+            }
+            const int n_all = planes * (L.n_steps - 1);
+            const int j = lane / 9, c = lane - 9 * j, dx = c % 3 - 1, dy = c / 3 - 1;
+            long long t0 = clock64();
+            while (n_flag < n_all || al_step < L.n_steps) {
+                bool moved = false;
+                // planes that every consumer warp has left (the counts are released after the warp's stores)
+                int done = lane < NCW ? ld_shared_acquire(&sync_done[lane]) : 0x7fffffff;
+                done = min(__reduce_min_sync(0xffffffffu, done), n_all);
+                if (done > n_flag) {
+                    __syncwarp();
+                    if (lane == 0) asm volatile("fence.acq_rel.gpu;" ::: "memory");
+                    while (n_flag < done) {
+                        const int n = min(done - n_flag, fg_pc.w - fg_pc.z - fg_t);  // planes of one column
+                        int* f = L.flags + fg_pf.base + (down ? fg_pc.w - 1 - fg_t : fg_pc.z + fg_t);
+                        if (lane == 0)
+                            for (int q = 0; q < n; ++q) st_flag(f + (down ? -q : q), L.epoch + fg_step + 1);
+                        n_flag += n;
+                        fg_t += n;
+                        if (fg_t == fg_pc.w - fg_pc.z) {
+                            fg_t = 0;
+                            if (++fg_i == n_pieces) {
+                                fg_i = 0;
+                                ++fg_step;
+                            }
+                            if (n_pieces > 1) {
+                                fg_pc = L.pieces[piece_slot(fg_i)];
+                                fg_pf = L.piece_flags[piece_slot(fg_i)];
+                            }
+                        }
+                    }
+                    moved = true;
+                }
+                if (al_step < L.n_steps) {
+                    // nine flags of each of the next 12 loads' planes
+                    const int nload = al_pc.w - al_pc.z + (PLANAR ? 0 : 2);
+                    const bool col_in = lane < 27 && (dx == 0 || (al_pf.has & (dx < 0 ? 1 : 2))) &&
+                                        (PLANAR || dy == 0 || (al_pf.has & (dy < 0 ? 4 : 8)));
+                    const int* fl = L.flags + al_pf.base + dx * al_pf.len + (PLANAR ? 0 : dy * al_pf.row);
+                    const int want = L.epoch + al_step;
+                    int v[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int o = al_off + j + 3 * q;
+                        const int z = (down ? al_pc.w - (PLANAR ? 1 : 0) - o : al_pc.z - (PLANAR ? 0 : 1) + o) + (PLANAR ? dy : 0);
+                        v[q] = want;
+                        if (col_in && o < nload && z >= al_pf.z0 && z < al_pf.z0 + al_pf.len) v[q] = ld_flag(fl + z);
+                    }
+                    int ok = 0;
+                    bool run = true;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const unsigned m = __ballot_sync(0xffffffffu, (int)((unsigned)v[q] - (unsigned)want) >= 0);
+#pragma unroll
+                        for (int e = 0; e < 3; ++e) {
+                            run = run && ((m >> (9 * e)) & 0x1ffu) == 0x1ffu;
+                            if (run) ok = 3 * q + e + 1;
+                        }
+                    }
+                    ok = min(ok, nload - al_off);
+                    if (ok > 0) {
+                        // the other CTAs' stores (acquired with the flags) before this CTA's copies of them
+                        __syncwarp();
+                        asm volatile("fence.proxy.async;" ::: "memory");
+                        __syncwarp();
+                        n_allow += ok;
+                        if (lane == 0) st_shared_release(&sync_allowed, n_allow);
+                        al_off += ok;
+                        if (al_off == nload) {
+                            al_off = 0;
+                            if (++al_i == n_pieces) {
+                                al_i = 0;
+                                ++al_step;
+                            }
+                            if (n_pieces > 1) {
+                                al_pc = L.pieces[piece_slot(al_i)];
+                                al_pf = L.piece_flags[piece_slot(al_i)];
+                            }
+                        }
+                        moved = true;
+                    }
+                }
+                if (moved) t0 = clock64();
+                if (__any_sync(0xffffffffu, abort_flag || clock64() - t0 > L.wait_limit)) {
+                    abort_flag = 1;
+                    break;
+                }
+            }
+        }
     } else {
         // ---------------- consumer warps ----------------
         const int tx = tid % 32, row0 = (tid / 32) * CY;  // node pair (x, x+1) = x0 + 2 tx
-        F2 vsum = {0.0f, 0.0f};
+        float2 vhi = splat2(0.0f), vlo = splat2(0.0f);  // the tissue sums of the pair's two columns
         bool timed_out = false;
-        int jb = 0, lp = 0;  // load index of the first plane of the piece, local piece index
-        int sb = 0, pb = 0;  // ring B: slot and phase parity of the next computed plane
+        int lr = 0;                // slot of the piece's context
+        int aw = 0, apar = 0;  // ring A: byte offset and phase parity of the next plane to wait for
+        int bw = 0, bpar = 0;  // ring B: the same
+        // The wait for a phase; false when it ran out (or another part of the CTA gave up).
         auto wait_bar = [&](uint64_t* bar, int parity) {
-            if (timed_out || abort_flag) {
-                timed_out = true;
-                return;
-            }
-            if (!mbar_wait_bounded(bar, parity, L.wait_limit)) {
-                timed_out = true;
-                abort_flag = 1;
-            }
-        };
-        auto wait_slot = [&](int slot, int parity) { wait_bar(&full[slot], parity); };
-        auto wait_full = [&](int j) { wait_slot(j % NS, (j / NS) & 1); };
-        for (int pi = piece_begin; pi < piece_end; ++pi, ++lp) {
-            wait_full(jb);  // the piece's first load carries its context
-            const PieceSlot& a = ring[lp % NS];  // read from shared memory where used
-            const float* mp = a.mp;
-            const float theta = a.theta;
-            int4 pc = make_int4(a.x0, a.y0, a.z0, a.z1);
-            if (timed_out) pc.w = pc.z = 0;  // context unreliable: compute nothing
-            const int x = pc.x + 2 * tx;  // first node of this thread's pair
-            const bool x_in = x < a.nx && !timed_out;  // (folded into the per-node flags)
-            const int ncomp = pc.w - pc.z;
-            if (!PLANAR) wait_full(jb + 1);
-            // stage slots of loads jb + t (sp), jb + t + 1 (sc), jb + t + 2 (sn)
-            // and the slot and phase parity of the next load to wait for,
-            // advanced per plane without divisions
-            int sp = jb % NS;
-            int sc = sp + 1 == NS ? 0 : sp + 1;
-            int sn = sc + 1 == NS ? 0 : sc + 1;
-            const int jw = jb + (PLANAR ? 1 : 2);
-            int sw = jw % NS, pw = (jw / NS) & 1;
-            for (int t = 0; t < ncomp; ++t) {
-                if (!PLANAR || t > 0) {
-                    wait_slot(sw, pw);
-                    if (++sw == NS) {
-                        sw = 0;
-                        pw ^= 1;
-                    }
+            if (mbar_try_wait(bar, parity)) return true;
+            const long long t0 = clock64();
+            while (!mbar_try_wait(bar, parity)) {
+                if (abort_flag || clock64() - t0 > L.wait_limit) {
+                    abort_flag = 1;
+                    return false;
                 }
-                if (HB) wait_bar(&fullb[sb], pb);  // the plane's own fibres, W-tilde sums, other variables
-                const int k = PLANAR ? 0 : pc.z + t;
-                const int yb = (PLANAR ? (pc.z + t) * TY : pc.y) + row0;  // y of this thread's first row
-                const unsigned char* stc = smem + (PLANAR ? sp : sc) * P::A_STAGE;
-                const unsigned char* stp = PLANAR ? stc : smem + sp * P::A_STAGE;
-                const unsigned char* stn = PLANAR ? stc : smem + sn * P::A_STAGE;
-                const unsigned char* stb = bstages + sb * P::B_STAGE;
-                const float* Up = reinterpret_cast<const float*>(stp + P::U_OFF);
-                const float* Uc = reinterpret_cast<const float*>(stc + P::U_OFF);
-                const float* Un = reinterpret_cast<const float*>(stn + P::U_OFF);
-                const float* Fb = reinterpret_cast<const float*>(stb + P::F_OFF);  // [3][TY][TX]
-                const float* Db = reinterpret_cast<const float*>(stb + P::D_OFF);  // [3][TY][TX]
-                const unsigned char* Mp = stp + P::M_OFF;
-                const unsigned char* Mc = stc + P::M_OFF;
-                const unsigned char* Mn = stn + P::M_OFF;
-                const float* Sv = reinterpret_cast<const float*>(stb + P::S_OFF);
-                const bool zn_ok = k + 1 < a.nz, zp_ok = k > 0;
-                const int c0 = (row0 + 1) * UW + (2 * tx + 4);   // stage index of node (x, yb), even
+            }
+            return true;
+        };
+        auto bar_a = [&](int off) { return reinterpret_cast<uint64_t*>(smem + off + P::A_BAR); };
+        // Wait for the next plane of ring A; its stage's byte offset.
+        auto next_plane = [&]() {
+            const int o = aw;
+            if (!timed_out && !wait_bar(bar_a(o), apar)) timed_out = true;
+            aw += P::A_STAGE;
+            if (aw == NS * P::A_STAGE) {
+                aw = 0;
+                apar ^= 1;
+            }
+            return o;
+        };
+        auto ld2 = [&](const float* U, int o) { return *reinterpret_cast<const float2*>(U + o); };
+        const int toff = row0 * UW + (2 * tx + 4);  // stage index of node (x, yb - 1), even
+        const int boff = row0 * TX + 2 * tx;        // ring-B index of node (x, yb)
+        const int n_walk = (P::FLOW ? L.n_steps : 1) * n_pieces;  // the pieces of every step in order
+        int n_left = 0;  // planes this warp has left
+        for (int pw = 0; pw < n_walk; ++pw) {
+            const bool last_step = pw >= n_walk - n_pieces;
+            int op = PLANAR ? 0 : next_plane();  // the piece's first load carries its context
+            int oc = next_plane();
+            const PieceSlot& a = ring[lr];
+            lr = lr + 1 == NS ? 0 : lr + 1;
+            const int ncomp = timed_out ? 0 : a.z1 - a.z0;  // (a context that never came is not read further)
+            Coef co;
+            co.c_perp = a.c_perp; co.c_d = a.c_d; co.c_dh = a.c_dh; co.c_s = a.c_s; co.c_iso = a.c_iso;
+            float mp[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) mp[i] = a.mp[i];
+            const float theta = a.theta, dt = a.dt;
+            const bool stim_on = a.stim_amp != 0.0f;
+            const int nx = a.nx, ny = a.ny, nz = a.nz, px = a.px;
+            const int x = a.x0 + 2 * tx;  // first node of this thread's pair
+            const bool x_in = x < nx, x1_in = x + 1 < nx;
+            // unmasked grids: minus the number of x neighbours, and psi(x+1) - psi(x-1), of the two nodes
+            const float px0 = x1_in ? 1.0f : 0.0f, mx0 = x > 0 ? 1.0f : 0.0f, px1 = x + 2 < nx ? 1.0f : 0.0f;
+            const float2 ncx = MASKED ? splat2(-2.0f) : make_float2(-(px0 + mx0), -(px1 + 1.0f));
+            const float2 ex = make_float2(px0 - mx0, px1 - 1.0f);
+            // marched upwards, or downwards (then the plane before the current one lies above it)
+            const int first = down ? a.z1 - 1 : a.z0, dir = down ? -1 : 1;
+            int yb = (PLANAR ? first * TY : a.y0) + row0;  // y of this thread's first row
+            int k = PLANAR ? 0 : first;
+            long long gi = (long long)k * a.plane + (long long)yb * px + x;  // node (x, yb) of plane k (even)
+            const long long gstep = (PLANAR ? (long long)TY * px : a.plane) * dir;
+            float* const dst = a.dst;
+            const long long vol = a.vol;
+            for (int t = 0; t < ncomp; ++t) {
+                const int on = PLANAR ? (t ? (oc = next_plane()) : oc) : next_plane();
+                uint64_t* barb = reinterpret_cast<uint64_t*>(bstages + bw + P::B_BAR);
+                if (HB && !timed_out && !wait_bar(barb, bpar)) timed_out = true;
+                if (timed_out) break;
+                const float* Uc = reinterpret_cast<const float*>(smem + oc + P::U_OFF) + toff;
+                const int ozm = down ? on : op, ozp = down ? op : on;  // planes k-1 and k+1
+                const float* Up = reinterpret_cast<const float*>(smem + ozm + P::U_OFF) + toff;
+                const float* Un = reinterpret_cast<const float*>(smem + ozp + P::U_OFF) + toff;
+                const unsigned char* stb = bstages + bw;
+                const float* Fb = reinterpret_cast<const float*>(stb + P::F_OFF) + boff;  // [3][TY][TX]
+                const float* Db = reinterpret_cast<const float*>(stb + P::D_OFF) + boff;  // [3][TY][TX]
+                const float* Sv = reinterpret_cast<const float*>(stb + P::S_OFF) + boff;
+                const unsigned char* Mp = smem + ozm + P::M_OFF;
+                const unsigned char* Mc = smem + oc + P::M_OFF;
+                const unsigned char* Mn = smem + ozp + P::M_OFF;
                 const int m0 = (row0 + 1) * MW + (2 * tx + 16);  // mask index of node (x, yb)
-    
-                {
-                    auto ld2 = [&](const float* U, int o) { return *reinterpret_cast<const float2*>(U + o); };
-                    const bool x1_in = x + 1 < a.nx;
-                    // psi of the x neighbours of the two nodes (unmasked grids)
-                    const float px0 = x1_in ? 1.0f : 0.0f, mx0 = (x > 0) ? 1.0f : 0.0f;
-                    const float px1 = (x + 2 < a.nx) ? 1.0f : 0.0f, mx1 = 1.0f;
-    
-                    // phase 1: the stencil for the 2 x CY nodes of this thread.
-                    // Sliding window down the rows: plane k at x-2..x+3 (three
-                    // float2), own pair of planes k+-1, own pair of fibres.
-                    float Lr[CY][2], u0r[CY][2];
-                    bool live[CY][2];
-                    float2 wA[3], wB[3], wC[3], wN[3], wP[3];
-    #pragma unroll
-                    for (int w = 0; w < 2; ++w) {
-                        const int o = c0 + (w - 1) * UW;
-                        wA[w] = ld2(Uc, o - 2); wB[w] = ld2(Uc, o); wC[w] = ld2(Uc, o + 2);
-                        wN[w] = ld2(Un, o); wP[w] = ld2(Up, o);
+                const bool zn_ok = k + 1 < nz, zp_ok = k > 0;
+                const int nrows = ny - yb;  // rows of this thread inside the array
+                const float ncz = MASKED || (zn_ok && zp_ok) ? -2.0f : (zn_ok || zp_ok ? -1.0f : 0.0f);
+                // unmasked: some cross difference misses a neighbour on one side only (a row or plane at
+                // the array's border)
+                const bool border = !MASKED && ANISO && (yb == 0 || nrows <= CY || (!PLANAR && !(zn_ok && zp_ok)));
+
+                // Sliding window down the rows: plane k at x-1..x+2, the own pair of planes k+-1.
+                float2 wB[CY + 2], wN[CY + 2], wP[CY + 2];
+                float wA[CY + 2], wC[CY + 2];
+                auto load_row = [&](int w) {  // row w - 1 of the window
+                    const int o = w * UW;
+                    wB[w] = ld2(Uc, o);
+                    if (ANISO || (w > 0 && w <= CY)) {
+                        wA[w] = Uc[o - 1];
+                        wC[w] = Uc[o + 2];
                     }
-    #pragma unroll
-                    for (int r = 0; r < CY; ++r) {
-                        const int y = yb + r;
-                        const int c = c0 + r * UW;
-                        const int m = m0 + r * MW;
-                        {
-                            const int o = c + UW;  // row r+1
-                            wA[2] = ld2(Uc, o - 2); wB[2] = ld2(Uc, o); wC[2] = ld2(Uc, o + 2);
-                            wN[2] = ld2(Un, o); wP[2] = ld2(Up, o);
+                    if (!PLANAR && (ANISO || (w > 0 && w <= CY))) {
+                        wN[w] = ld2(Un, o);
+                        wP[w] = ld2(Up, o);
+                    }
+                };
+                load_row(0);
+                load_row(1);
+#pragma unroll
+                for (int r = 0; r < CY; ++r) {
+                    load_row(r + 2);
+                    if (r >= nrows) continue;  // (warp-uniform)
+                    const int w = r + 1;
+                    const float2 u0 = wB[w];
+                    bool live[2] = {x_in, x1_in};
+                    float2 Lr;
+                    const float ncy = MASKED ? -2.0f : ((r == 0 && yb == 0) || r + 1 == nrows
+                                                            ? (r == 0 && yb == 0 && r + 1 == nrows ? 0.0f : -1.0f)
+                                                            : -2.0f);
+                    const float2 sx = make_float2(__fadd_rn(u0.y, wA[w]), __fadd_rn(wC[w], u0.x));
+                    if (!ANISO) {
+                        float2 sum = add2(sx, add2(wB[w + 1], wB[w - 1]));
+                        float2 nc = add2(ncx, splat2(ncy));
+                        if (!PLANAR) {
+                            sum = add2(sum, add2(wN[w], wP[w]));
+                            nc = add2(nc, splat2(ncz));
                         }
-                        bool tis[2] = {x_in && y < a.ny, x_in && y < a.ny && x1_in}, intr[2];
-                        if (MASKED) {
-                            const unsigned char mc0 = Mc[m], mc1 = Mc[m + 1];
-                            tis[0] = tis[0] && (mc0 & MASK_TISSUE);
-                            tis[1] = tis[1] && (mc1 & MASK_TISSUE);
-                            intr[0] = (mc0 & MASK_INTERIOR) != 0;
-                            intr[1] = (mc1 & MASK_INTERIOR) != 0;
-                        } else {
-                            intr[0] = intr[1] = (y > 0) && (y + 1 < a.ny) && (PLANAR || (zp_ok && zn_ok));  // warp-uniform
+                        Lr = mul2(splat2(co.c_iso), fma2(nc, u0, sum));
+                    } else {
+                        Diffs d;
+                        d.xx = fma2(ncx, u0, sx);
+                        d.yy = fma2(splat2(ncy), u0, add2(wB[w + 1], wB[w - 1]));
+                        d.y1 = sub2(wB[w + 1], wB[w - 1]);
+                        const float ya = __fsub_rn(wA[w + 1], wA[w - 1]), yc = __fsub_rn(wC[w + 1], wC[w - 1]);
+                        d.xy = make_float2(__fsub_rn(d.y1.y, ya), __fsub_rn(yc, d.y1.x));
+                        if (!PLANAR) {
+                            d.zz = fma2(splat2(ncz), u0, add2(wN[w], wP[w]));
+                            d.z1 = sub2(wN[w], wP[w]);
+                            const float za = __fsub_rn(Un[w * UW - 1], Up[w * UW - 1]);
+                            const float zc = __fsub_rn(Un[w * UW + 2], Up[w * UW + 2]);
+                            d.xz = make_float2(__fsub_rn(d.z1.y, za), __fsub_rn(zc, d.z1.x));
+                            d.yz = sub2(sub2(wN[w + 1], wP[w + 1]), sub2(wN[w - 1], wP[w - 1]));
                         }
-                        Nb n[2];
-                        F3 f[2], sd[2];
-                        n[0].u0 = wB[1].x; n[0].xp = wB[1].y; n[0].xm = wA[1].y;
-                        n[0].yp = wB[2].x; n[0].ym = wB[0].x; n[0].zp = wN[1].x; n[0].zm = wP[1].x;
-                        n[1].u0 = wB[1].y; n[1].xp = wC[1].x; n[1].xm = wB[1].x;
-                        n[1].yp = wB[2].y; n[1].ym = wB[0].y; n[1].zp = wN[1].y; n[1].zm = wP[1].y;
-                        if (ANISO) {
-                            const float2 nA = ld2(Un, c - 2), nC = ld2(Un, c + 2);
-                            const float2 pA = ld2(Up, c - 2), pC = ld2(Up, c + 2);
-                            n[0].pp = wB[2].y; n[0].mm = wA[0].y; n[0].pm = wB[0].y; n[0].mp = wA[2].y;
-                            n[0].xpzp = wN[1].y; n[0].xmzm = pA.y; n[0].xpzm = wP[1].y; n[0].xmzp = nA.y;
-                            n[0].ypzp = wN[2].x; n[0].ymzm = wP[0].x; n[0].ypzm = wP[2].x; n[0].ymzp = wN[0].x;
-                            n[1].pp = wC[2].x; n[1].mm = wB[0].x; n[1].pm = wC[0].x; n[1].mp = wB[2].x;
-                            n[1].xpzp = nC.x; n[1].xmzm = wP[1].x; n[1].xpzm = pC.x; n[1].xmzp = wN[1].x;
-                            n[1].ypzp = wN[2].y; n[1].ymzm = wP[0].y; n[1].ypzm = wP[2].y; n[1].ymzp = wN[0].y;
-                            // the pair's own fibres and W-tilde sums ([comp][row][x] in ring B)
-                            const int bo = (row0 + r) * TX + 2 * tx;
-                            const float2 fx = ld2(Fb, bo), fy = ld2(Fb + CB, bo), fz = ld2(Fb + 2 * CB, bo);
-                            f[0] = F3{fx.x, fy.x, fz.x};
-                            f[1] = F3{fx.y, fy.y, fz.y};
-                            if (ANISO == AN_SUMS) {
-                                const float2 dx = ld2(Db, bo), dy = ld2(Db + CB, bo), dz = ld2(Db + 2 * CB, bo);
-                                sd[0] = F3{dx.x, dy.x, dz.x};
-                                sd[1] = F3{dx.y, dy.y, dz.y};
-                            } else {
-                                sd[0] = sd[1] = F3{0.f, 0.f, 0.f};
+                        if (ANISO == AN_SUMS)
+                            d.x1 = make_float2(__fsub_rn(u0.y, wA[w]), __fsub_rn(wC[w], u0.x));
+                        if (border) {
+                            // psi = 0 on one side only leaves a cross difference short of u0 where both
+                            // axes end (the array's edges)
+                            const float ey = (r + 1 == nrows ? 0.0f : 1.0f) - (r == 0 && yb == 0 ? 0.0f : 1.0f);
+                            const float ez = (zn_ok ? 1.0f : 0.0f) - (zp_ok ? 1.0f : 0.0f);
+                            d.xy = fma2(mul2(ex, splat2(-ey)), u0, d.xy);
+                            if (!PLANAR) {
+                                d.xz = fma2(mul2(ex, splat2(-ez)), u0, d.xz);
+                                d.yz = fma2(splat2(-ey * ez), u0, d.yz);
                             }
-                        } else {
-    #pragma unroll
-                            for (int e = 0; e < 2; ++e) f[e] = sd[e] = F3{0.f, 0.f, 0.f};
                         }
-    #pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            live[r][e] = tis[e];
-                            u0r[r][e] = n[e].u0;
-                            // fast formula for every node (values of void or
-                            // out-of-array nodes are finite and never stored) ...
-                            if (MASKED)
-                                Lr[r][e] = lap_interior<ANISO>(a, n[e], f[e], sd[e]);
-                            else
-                                Lr[r][e] = lap_xbound<ANISO>(a, n[e], e ? px1 : px0, e ? mx1 : mx0, f[e], sd[e]);
+                        const float2 f[3] = {ld2(Fb, r * TX), ld2(Fb, r * TX + CB), ld2(Fb, r * TX + 2 * CB)};
+                        float2 sd[3];
+                        if (ANISO == AN_SUMS) {
+#pragma unroll
+                            for (int c = 0; c < 3; ++c) sd[c] = ld2(Db, r * TX + c * CB);
                         }
-                        // ... and the general one where a y/z neighbour (or, in a
-                        // masked grid, any neighbour) may be void: rare, and
-                        // warp-uniform on unmasked grids
-                        if (!((intr[0] || !tis[0]) && (intr[1] || !tis[1]))) {
-    #pragma unroll
+                        Lr = lap_pair<ANISO, PLANAR>(co, d, f, sd);
+                    }
+                    if (MASKED) {
+                        const int m = m0 + r * MW;
+                        const unsigned char mc0 = Mc[m], mc1 = Mc[m + 1];
+                        live[0] = live[0] && (mc0 & MASK_TISSUE);
+                        live[1] = live[1] && (mc1 & MASK_TISSUE);
+                        const bool intr[2] = {(mc0 & MASK_INTERIOR) != 0, (mc1 & MASK_INTERIOR) != 0};
+                        // the general formula where any neighbour may be void
+                        if ((live[0] && !intr[0]) || (live[1] && !intr[1])) {
+#pragma unroll
                             for (int e = 0; e < 2; ++e) {
-                                if (!tis[e] || intr[e]) continue;
-                                const int xe = x + e, me = m + e;
+                                if (!live[e] || intr[e]) continue;
+                                const int me = m + e, ue = w * UW + e;
                                 Psi q;
-                                if (MASKED) {
-                                    q.xp = Mc[me + 1] != 0; q.xm = Mc[me - 1] != 0;
-                                    q.yp = Mc[me + MW] != 0; q.ym = Mc[me - MW] != 0;
-                                    q.zp = zn_ok && Mn[me] != 0; q.zm = zp_ok && Mp[me] != 0;
+                                Nb n;
+                                n.u0 = Uc[ue];
+                                n.xp = Uc[ue + 1]; n.xm = Uc[ue - 1]; n.yp = Uc[ue + UW]; n.ym = Uc[ue - UW];
+                                n.zp = Un[ue]; n.zm = Up[ue];
+                                q.xp = Mc[me + 1] != 0; q.xm = Mc[me - 1] != 0;
+                                q.yp = Mc[me + MW] != 0; q.ym = Mc[me - MW] != 0;
+                                q.zp = zn_ok && Mn[me] != 0; q.zm = zp_ok && Mp[me] != 0;
+                                F3 f = {0.f, 0.f, 0.f}, sd = {0.f, 0.f, 0.f};
+                                if (ANISO) {
+                                    n.pp = Uc[ue + UW + 1]; n.mm = Uc[ue - UW - 1];
+                                    n.pm = Uc[ue - UW + 1]; n.mp = Uc[ue + UW - 1];
+                                    n.xpzp = Un[ue + 1]; n.xmzm = Up[ue - 1]; n.xpzm = Up[ue + 1]; n.xmzp = Un[ue - 1];
+                                    n.ypzp = Un[ue + UW]; n.ymzm = Up[ue - UW]; n.ypzm = Up[ue + UW]; n.ymzp = Un[ue - UW];
                                     q.pp = Mc[me + MW + 1] != 0; q.mm = Mc[me - MW - 1] != 0;
                                     q.pm = Mc[me - MW + 1] != 0; q.mp = Mc[me + MW - 1] != 0;
                                     q.xpzp = zn_ok && Mn[me + 1] != 0; q.xmzm = zp_ok && Mp[me - 1] != 0;
                                     q.xpzm = zp_ok && Mp[me + 1] != 0; q.xmzp = zn_ok && Mn[me - 1] != 0;
                                     q.ypzp = zn_ok && Mn[me + MW] != 0; q.ymzm = zp_ok && Mp[me - MW] != 0;
                                     q.ypzm = zp_ok && Mp[me + MW] != 0; q.ymzp = zn_ok && Mn[me - MW] != 0;
-                                } else {
-                                    const bool xp = xe + 1 < a.nx, xm = xe > 0, yp = y + 1 < a.ny, ym = y > 0;
-                                    q.xp = xp; q.xm = xm; q.yp = yp; q.ym = ym; q.zp = zn_ok; q.zm = zp_ok;
-                                    q.pp = xp && yp; q.mm = xm && ym; q.pm = xp && ym; q.mp = xm && yp;
-                                    q.xpzp = xp && zn_ok; q.xmzm = xm && zp_ok; q.xpzm = xp && zp_ok; q.xmzp = xm && zn_ok;
-                                    q.ypzp = yp && zn_ok; q.ymzm = ym && zp_ok; q.ypzm = yp && zp_ok; q.ymzp = ym && zn_ok;
+                                    const int be = r * TX + e;
+                                    f = F3{Fb[be], Fb[be + CB], Fb[be + 2 * CB]};
+                                    if (ANISO == AN_SUMS) sd = F3{Db[be], Db[be + CB], Db[be + 2 * CB]};
                                 }
-                                Lr[r][e] = lap_general<ANISO>(a, n[e], q, f[e], sd[e]);
+                                const float Lg = lap_general<ANISO>(co, n, q, f, sd);
+                                if (e) Lr.y = Lg; else Lr.x = Lg;
                             }
-                        }
-                        // slide the window down one row
-                        wA[0] = wA[1]; wA[1] = wA[2]; wB[0] = wB[1]; wB[1] = wB[2]; wC[0] = wC[1]; wC[1] = wC[2];
-                        wN[0] = wN[1]; wN[1] = wN[2]; wP[0] = wP[1]; wP[1] = wP[2];
-                    }
-    
-                    // phase 2: reaction, stores, activation, tissue sum (predicated)
-                    const bool stim_on = a.stim_amp != 0.0f;
-    #pragma unroll
-                    for (int r = 0; r < CY; ++r) {
-                        const int y = yb + r;
-                        const long long gi = (long long)k * a.plane + (long long)y * a.px + x;  // even
-                        float yv[2][S];
-    #pragma unroll
-                        for (int e = 0; e < 2; ++e) yv[e][0] = u0r[r][e];
-    #pragma unroll
-                        for (int v = 1; v < S32; ++v) {
-                            const float2 sv = *reinterpret_cast<const float2*>(Sv + (v - 1) * TX * TY + (row0 + r) * TX + 2 * tx);
-                            yv[0][v] = sv.x;
-                            yv[1][v] = sv.y;
-                        }
-    #pragma unroll
-                        for (int v = S32; v < S; ++v) {  // 16-bit gates, decoded to FP32
-                            const uint32_t w = *reinterpret_cast<const uint32_t*>(
-                                stb + P::G_OFF + 2 * ((v - S32) * TX * TY + (row0 + r) * TX + 2 * tx));
-                            const float2 gv = gate_decode2<GATES>(w);
-                            yv[0][v] = gv.x;
-                            yv[1][v] = gv.y;
-                        }
-                            float Isr[2];
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            Isr[e] = 0.0f;
-                            if (stim_on && live[r][e] && a.stim[gi + e]) Isr[e] = a.stim_amp;
-                        }
-                        if (GEN && a.split) {
-                            // Lie splitting: the diffusion substep on its own, then
-                            // the kinetics step from the half-step voltage
-#pragma unroll
-                            for (int e = 0; e < 2; ++e) {
-                                yv[e][0] += a.dt * Lr[r][e];
-                                Lr[r][e] = 0.0f;
-                            }
-                        }
-                        if constexpr (SURR && MODEL == BBX_BR) {
-                            // the surrogate where the state is inside the training
-                            // envelope and V below the upstroke threshold; the
-                            // exact model elsewhere
-                            const SurrogateData* W = a.surr;
-                            bool want[2] = {false, false};
-                            if (W) {
-#pragma unroll
-                                for (int e = 0; e < 2; ++e) {
-                                    bool in = live[r][e] && yv[e][0] < W->v_up;
-#pragma unroll
-                                    for (int v = 0; v < S; ++v)
-                                        in = in && yv[e][v] >= W->norm[32 + v] && yv[e][v] <= W->norm[40 + v];
-                                    want[e] = in;
-                                }
-                            }
-                            if (__any_sync(0xffffffffu, want[0] || want[1])) {
-                                float dsur[2][8];
-                                surrogate_warp64(W, wbufs + (tid >> 5) * 2048, yv, dsur);
-#pragma unroll
-                                for (int e = 0; e < 2; ++e) {
-                                    if (want[e]) {
-#pragma unroll
-                                        for (int v = 0; v < S; ++v) yv[e][v] += dsur[e][v];
-                                        yv[e][0] += a.dt * (Lr[r][e] + Isr[e]);
-                                    } else {
-                                        Model<MODEL>::update(mp, yv[e], Lr[r][e], Isr[e], a.dt);
-                                    }
-                                }
-                            } else {
-#pragma unroll
-                                for (int e = 0; e < 2; ++e) Model<MODEL>::update(mp, yv[e], Lr[r][e], Isr[e], a.dt);
-                            }
-                        } else if constexpr (MODEL != BBX_BR && GEN) {
-                            if (a.rk4) {
-#pragma unroll
-                                for (int e = 0; e < 2; ++e) rk4_update<MODEL>(mp, yv[e], Lr[r][e], Isr[e], a.dt);
-                            } else {
-#pragma unroll
-                                for (int e = 0; e < 2; ++e) Model<MODEL>::update(mp, yv[e], Lr[r][e], Isr[e], a.dt);
-                            }
-                        } else if constexpr (MODEL == BBX_BR_MRL || MODEL == BBX_BR_FCA) {
-#pragma unroll
-                            for (int e = 0; e < 2; ++e)
-                                Model<MODEL>::update_tab(mp, a.tab, yv[e], Lr[r][e], Isr[e], a.dt);
-                        } else if constexpr (MODEL == BBX_BR && GEN) {
-                            // tabulated Rush-Larsen coefficients (the general
-                            // variants only, so the default kernel is unchanged)
-                            if (a.tab) {
-#pragma unroll
-                                for (int e = 0; e < 2; ++e)
-                                    Model<MODEL>::update_tab(mp, a.tab, yv[e], Lr[r][e], Isr[e], a.dt);
-                            } else {
-#pragma unroll
-                                for (int e = 0; e < 2; ++e) Model<MODEL>::update(mp, yv[e], Lr[r][e], Isr[e], a.dt);
-                            }
-                        } else {
-#pragma unroll
-                            for (int e = 0; e < 2; ++e) Model<MODEL>::update(mp, yv[e], Lr[r][e], Isr[e], a.dt);
-                        }
-                        if (live[r][0] && live[r][1]) {
-    #pragma unroll
-                            for (int v = 0; v < S32; ++v)
-                                st_global(a.dst + (long long)v * a.vol + gi, make_float2(yv[0][v], yv[1][v]));
-    #pragma unroll
-                            for (int v = S32; v < S; ++v)
-                                st_global_u32(a.dst16 + (long long)(v - S32) * a.vol + gi,
-                                              gate_encode2<GATES>(yv[0][v], yv[1][v]));
-                        } else if (live[r][0] || live[r][1]) {
-    #pragma unroll
-                            for (int e = 0; e < 2; ++e)
-                                if (live[r][e]) {
-    #pragma unroll
-                                    for (int v = 0; v < S32; ++v) st_global(a.dst + (long long)v * a.vol + gi + e, yv[e][v]);
-    #pragma unroll
-                                    for (int v = S32; v < S; ++v)
-                                        st_global_u16(a.dst16 + (long long)(v - S32) * a.vol + gi + e,
-                                                      gate_encode<GATES>(yv[e][v]));
-                                }
-                        }
-    #pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            if (live[r][e] && u0r[r][e] < theta && theta <= yv[e][0]) {
-                                if (a.act[gi + e] == BBX_ACT_NONE) a.act[gi + e] = a.step_next;
-                            }
-                            two_sum_add(vsum, live[r][e] ? yv[e][0] : 0.0f);
                         }
                     }
+
+                    // reaction, stores, activation, tissue sum (predicated)
+                    const long long gr = gi + (long long)r * px;
+                    float2 y[S];
+                    y[0] = u0;
+#pragma unroll
+                    for (int v = 1; v < S32; ++v) y[v] = ld2(Sv, (v - 1) * CB + r * TX);
+#pragma unroll
+                    for (int v = S32; v < S; ++v) {  // 16-bit gates, decoded to FP32
+                        const uint32_t w16 = *reinterpret_cast<const uint32_t*>(
+                            stb + P::G_OFF + 2 * ((v - S32) * CB + boff + r * TX));
+                        y[v] = gate_decode2<GATES>(w16);
+                    }
+                    float2 Is = splat2(0.0f);
+                    if (stim_on) {
+                        if (live[0] && a.stim[gr]) Is.x = a.stim_amp;
+                        if (live[1] && a.stim[gr + 1]) Is.y = a.stim_amp;
+                    }
+                    if (GEN && a.split) {
+                        // Lie splitting: the diffusion substep on its own, then
+                        // the kinetics step from the half-step voltage
+                        y[0] = fma2(splat2(dt), Lr, y[0]);
+                        Lr = splat2(0.0f);
+                    }
+                    react_pair<MODEL, SURR, GEN>(a, mp, dt, wbufs, live, y, Lr, Is);
+                    if (live[0] && live[1]) {
+                        float* q = dst + gr;
+#pragma unroll
+                        for (int v = 0; v < S32; ++v) {
+                            st_global(q, y[v]);
+                            q += vol;
+                        }
+#pragma unroll
+                        for (int v = S32; v < S; ++v)
+                            st_global_u32(a.dst16 + (long long)(v - S32) * a.vol + gr, gate_encode2<GATES>(y[v].x, y[v].y));
+                    } else if (live[0] || live[1]) {
+#pragma unroll
+                        for (int e = 0; e < 2; ++e)
+                            if (live[e]) {
+#pragma unroll
+                                for (int v = 0; v < S32; ++v)
+                                    st_global(a.dst + (long long)v * a.vol + gr + e, e ? y[v].y : y[v].x);
+#pragma unroll
+                                for (int v = S32; v < S; ++v)
+                                    st_global_u16(a.dst16 + (long long)(v - S32) * a.vol + gr + e,
+                                                  gate_encode<GATES>(e ? y[v].y : y[v].x));
+                            }
+                    }
+                    const bool up0 = u0.x < theta && theta <= y[0].x, up1 = u0.y < theta && theta <= y[0].y;
+                    if (up0 || up1) {
+                        if (up0 && live[0] && a.act[gr] == BBX_ACT_NONE) a.act[gr] = a.step_next;
+                        if (up1 && live[1] && a.act[gr + 1] == BBX_ACT_NONE) a.act[gr + 1] = a.step_next;
+                    }
+                    // (columns outside an unmasked array are left out of the piece's sum)
+                    if (last_step) two_sum_add2(vhi, vlo, MASKED ? make_float2(live[0] ? y[0].x : 0.0f, live[1] ? y[0].y : 0.0f) : y[0]);
                 }
-    
-                    __syncwarp();
+
+                __syncwarp();
+                if (P::FLOW) ++n_left;
                 if (lane == 0) {
-                    mbar_arrive(&empty[sp]);
-                    if (HB) mbar_arrive(&emptyb[sb]);
+                    if (P::FLOW && !last_step) st_shared_release(&sync_done[warp], n_left);
+                    mbar_arrive(bar_a(PLANAR ? oc : op) + 1);
+                    if (HB) mbar_arrive(barb + 1);
                 }
-                if (HB && ++sb == NB) {
-                    sb = 0;
-                    pb ^= 1;
+                if (HB) {
+                    bw += P::B_STAGE;
+                    if (bw == NB * P::B_STAGE) {
+                        bw = 0;
+                        bpar ^= 1;
+                    }
                 }
-                sp = sc;
-                sc = sn;
-                sn = sn + 1 == NS ? 0 : sn + 1;
+                op = oc;
+                oc = on;
+                if (PLANAR) yb += dir * TY;
+                else k += dir;
+                gi += gstep;
             }
             __syncwarp();
-            if (!PLANAR && lane == 0) {
-                // release the piece's last two planes (or all of a piece cut short)
-                for (int j = jb + (ncomp > 0 ? ncomp : 0); j < jb + (ncomp > 0 ? ncomp + 2 : 2); ++j)
-                    mbar_arrive(&empty[j % NS]);
+            if (!PLANAR && lane == 0) {  // release the piece's last two planes
+                mbar_arrive(bar_a(op) + 1);
+                mbar_arrive(bar_a(oc) + 1);
             }
-            jb += (ncomp > 0 ? ncomp : 0) + (PLANAR ? 0 : 2);
+            if (!last_step) continue;
             // per-piece partial of the tissue sum, and a vote on timeouts
-            double v = (double)vsum.hi + (double)vsum.lo;
+            const int pi = down ? piece_end - 1 - (pw - (n_walk - n_pieces)) : piece_begin + (pw - (n_walk - n_pieces));
+            double v = (x_in ? (double)vhi.x + (double)vlo.x : 0.0) + (x1_in ? (double)vhi.y + (double)vlo.y : 0.0);
             for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
             if (lane == 0) red_scratch[warp] = v;
             const bool any_to = consumers_sync_or(timed_out, NCT);
@@ -1787,7 +2091,7 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
             }
             consumers_sync(NCT);
             if (!L.single && warp == 0 && !any_to) grid_piece_done(L, pi, lane);
-            vsum.hi = vsum.lo = 0.0f;
+            vhi = vlo = splat2(0.0f);
             if (any_to) break;
         }
         if (timed_out) abort_flag = 1;
@@ -1798,9 +2102,9 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
         // Give the loads that may still be in flight a bounded chance to land.
         atomicOr(L.err, ERRBIT_TIMEOUT);
         for (int j = issued > NS ? issued - NS : 0; j < issued; ++j)
-            (void)mbar_wait_bounded(&full[j % NS], (j / NS) & 1, L.wait_limit);
+            (void)mbar_wait_bounded(full(j % NS), (j / NS) & 1, L.wait_limit);
         for (int j = issuedb > NB ? issuedb - NB : 0; j < issuedb; ++j)
-            (void)mbar_wait_bounded(&fullb[j % NB], (j / NB) & 1, L.wait_limit);
+            (void)mbar_wait_bounded(fullb(j % NB), (j / NB) & 1, L.wait_limit);
     }
     step_finalize(L, red_scratch);
 }
@@ -1811,6 +2115,7 @@ struct StepKernel {
     int smem;
     int threads;
     int ty;
+    bool flow = false;  // may take several steps in one launch
 };
 
 }  // namespace bbx

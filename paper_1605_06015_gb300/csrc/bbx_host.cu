@@ -44,6 +44,7 @@ constexpr long long kWaitLimitCycles = 4000000000LL;  // about 2 s of SM clock
 constexpr long long kPoisonWaitLimit = 2000000LL;     // about 1 ms
 constexpr int kMaxPartials = 152 * 32;
 constexpr int kErrFibre = 4;
+constexpr int kFlowSteps = 64;  // time steps of one launch at most
 constexpr int kChunkX = 16;  // x granularity of a masked grid's piece origins (the mask copy's 16-byte rule)
 
 int model_nvars(int model) {
@@ -159,30 +160,28 @@ bool encode(CUtensorMap* m, CUtensorMapDataType dt, int rank, void* base, const 
 // set-up kernels
 // ------------------------------------------------------------------------
 
-// Normalise interleaved fibres into the SoA field [3][nz][ny][pxf] whose rows
-// are stored from x = -4 (storage column x + 4) with the x-padding filled by
-// the nearest in-array fibre (clamped); a zero vector at a tissue node sets
-// the error bit.  Void nodes get 0.
-__global__ void k_fibres(const float* __restrict__ in, int nx, int ny, int nz, int pxf, long long fplane,
-                         long long fvol, const uint8_t* __restrict__ mask, int px, long long plane,
-                         float* __restrict__ out, int* err) {
-    const long long n = (long long)pxf * ny * nz;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+// Normalise interleaved fibres into the SoA field [3][nz][ny][px], in the
+// state's layout: a step copies a tile's own fibres only, so rows need no
+// halo, and a 64-node row of a tile starts on a 128-byte line (stored from
+// x = -4 instead, each row touched a third line; the 512x512x256 slab's
+// copies alone, with no arithmetic, took 340 us a step against 296 us).  A
+// zero vector at a tissue node sets the error bit.  Void nodes and the row
+// padding get 0.
+__global__ void k_fibres(const float* __restrict__ in, int nx, int ny, int nz, const uint8_t* __restrict__ mask,
+                         int px, long long plane, long long vol, float* __restrict__ out, int* err) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < vol;
          i += (long long)gridDim.x * blockDim.x) {
-        const int xs = int(i % pxf);
-        const long long r = i / pxf;
+        const int x = int(i % px);
+        const long long r = i / px;
         const int y = int(r % ny);
         const int z = int(r / ny);
-        const int x = min(max(xs - 4, 0), nx - 1);
-        const bool real = (xs - 4) == x;
-        const long long src = (long long)x + (long long)nx * (y + (long long)ny * z);
-        const bool tissue = mask ? mask[z * plane + (long long)y * px + x] != 0 : true;
-        const float fx = in[3 * src], fy = in[3 * src + 1], fz = in[3 * src + 2];
-        const float n2 = fx * fx + fy * fy + fz * fz;
         float ox = 0.f, oy = 0.f, oz = 0.f;
-        if (tissue) {
+        if (x < nx && (!mask || mask[z * plane + (long long)y * px + x] != 0)) {
+            const long long src = (long long)x + (long long)nx * (y + (long long)ny * z);
+            const float fx = in[3 * src], fy = in[3 * src + 1], fz = in[3 * src + 2];
+            const float n2 = fx * fx + fy * fy + fz * fz;
             if (!(n2 > 0.0f) || !isfinite(n2)) {
-                if (real) atomicOr(err, kErrFibre);
+                atomicOr(err, kErrFibre);
             } else {
                 const float nr = __fsqrt_rn(n2);
                 ox = __fdiv_rn(fx, nr);
@@ -190,10 +189,9 @@ __global__ void k_fibres(const float* __restrict__ in, int nx, int ny, int nz, i
                 oz = __fdiv_rn(fz, nr);
             }
         }
-        const long long o = z * fplane + (long long)y * pxf + xs;
-        out[o] = ox;
-        out[fvol + o] = oy;
-        out[2 * fvol + o] = oz;
+        out[i] = ox;
+        out[vol + i] = oy;
+        out[2 * vol + i] = oz;
     }
 }
 
@@ -205,8 +203,8 @@ __global__ void k_fibres(const float* __restrict__ in, int nx, int ny, int nz, i
 // are computed once, in double precision, and read by every step.  Layout
 // [3][nz][ny][px]; 0 at void nodes.  *nonzero is set to 1 if any stored sum
 // differs from 0 (the step kernel skips loading sums that all vanish).
-__global__ void k_divergence(const float* __restrict__ fib, int nx, int ny, int nz, int pxf, long long fplane,
-                             long long fvol, const uint8_t* __restrict__ mask, int px, long long plane,
+__global__ void k_divergence(const float* __restrict__ fib, int nx, int ny, int nz,
+                             const uint8_t* __restrict__ mask, int px, long long plane,
                              long long vol, float* __restrict__ div, int* __restrict__ nonzero) {
     const long long n = (long long)nx * ny * nz;
     bool any = false;
@@ -222,10 +220,10 @@ __global__ void k_divergence(const float* __restrict__ fib, int nx, int ny, int 
             return mask ? (mask[zz * plane + (long long)yy * px + xx] & 1) != 0 : true;
         };
         auto fibre = [&](int xx, int yy, int zz, double* f) {
-            const long long q = zz * fplane + (long long)yy * pxf + (xx + 4);
+            const long long q = zz * plane + (long long)yy * px + xx;
             f[0] = fib[q];
-            f[1] = fib[fvol + q];
-            f[2] = fib[2 * fvol + q];
+            f[1] = fib[vol + q];
+            f[2] = fib[2 * vol + q];
         };
         double acc[3] = {0.0, 0.0, 0.0};
         if (tissue(x, y, z)) {
@@ -242,9 +240,11 @@ __global__ void k_divergence(const float* __restrict__ fib, int nx, int ny, int 
             }
         }
         const float s0 = (float)acc[0], s1 = (float)acc[1], s2 = (float)acc[2];
-        div[o] = s0;
-        div[vol + o] = s1;
-        div[2 * vol + o] = s2;
+        // a sum takes part only where both neighbours of its axis are tissue:
+        // stored as 0 elsewhere, so that the step needs no test for it
+        div[o] = tissue(x - 1, y, z) && tissue(x + 1, y, z) ? s0 : 0.0f;
+        div[vol + o] = tissue(x, y - 1, z) && tissue(x, y + 1, z) ? s1 : 0.0f;
+        div[2 * vol + o] = tissue(x, y, z - 1) && tissue(x, y, z + 1) ? s2 : 0.0f;
         any = any || s0 != 0.0f || s1 != 0.0f || s2 != 0.0f;
     }
     if (__any_sync(0xffffffffu, any) && (threadIdx.x & 31) == 0) atomicOr(nonzero, 1);
@@ -612,7 +612,14 @@ struct LaunchPlan {
     unsigned int* d_tissue_done = nullptr;  // per grid, zero between launches
     int* d_empty = nullptr;                 // grids without pieces
     int n_empty = 0;
-    size_t cap_pieces = 0, cap_cta = 0, cap_tis = 0, cap_tlist = 0, cap_done = 0, cap_empty = 0;
+    size_t cap_pieces = 0, cap_cta = 0, cap_tis = 0, cap_tlist = 0, cap_done = 0, cap_empty = 0, cap_flags = 0;
+    // Several steps in one launch (unmasked grids): the done flags of every
+    // column and computed plane, and the running step number they have reached
+    bool flow = false;
+    int* d_flags = nullptr;
+    PieceFlags* d_piece_flags = nullptr;
+    size_t cap_pflags = 0;
+    unsigned int epoch = 0;
     int cta_stride = 1, n_slots = 0;
 
     void release() {
@@ -625,6 +632,8 @@ struct LaunchPlan {
         cudaFree(d_ticket);
         cudaFree(d_tissue_done);
         cudaFree(d_empty);
+        cudaFree(d_flags);
+        cudaFree(d_piece_flags);
         *this = LaunchPlan();
     }
 };
@@ -690,7 +699,14 @@ int plan_shares(const std::vector<Seg>& segs, int ctas, std::vector<std::vector<
 
 // The launch plan of a list of segments (plan_shares), uploaded; per grid,
 // the pieces are listed for the fixed-order totals.
-int build_plan(LaunchPlan* lp, const std::vector<Seg>& segs, int n_tissues, int ctas) {
+// lattice: the grids' columns when their steps may share a launch (the CTAs
+// wait for one another then: a cooperative launch), or empty.
+struct Lattice {
+    int nbx, nby, len, z0;  // columns, computed planes of a column (a sheet: tile rows) from z0 on
+    bool planar;
+};
+int build_plan(LaunchPlan* lp, const std::vector<Seg>& segs, int n_tissues, int ctas, const std::vector<Lattice>& lattice,
+               int device) {
     long long T = 0;
     for (const Seg& sg : segs) T += sg.z1 - sg.z0;
     lp->n_planes = T;
@@ -738,6 +754,27 @@ int build_plan(LaunchPlan* lp, const std::vector<Seg>& segs, int n_tissues, int 
         if (toff[(size_t)t + 1] == toff[(size_t)t]) empty.push_back(t);
     if ((rc = upload(&lp->d_empty, &lp->cap_empty, empty))) return rc;
     lp->n_empty = (int)empty.size();
+    lp->flow = false;
+    int coop = 0;
+    if (lp->k.flow && !lattice.empty() && cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device) == cudaSuccess && coop) {
+        std::vector<long long> off((size_t)n_tissues + 1, 0);
+        for (int t = 0; t < n_tissues; ++t)
+            off[(size_t)t + 1] = off[(size_t)t] + (long long)lattice[(size_t)t].nbx * lattice[(size_t)t].nby * lattice[(size_t)t].len;
+        std::vector<PieceFlags> pf(nslot, PieceFlags{});
+        for (int c = 0; c < ctas; ++c)
+            for (int i = 0; i < cnt[(size_t)c]; ++i) {
+                const size_t k = (size_t)c * stride + i;
+                const Lattice& la = lattice[(size_t)ptis[k]];
+                const int bx = pieces[k].x / kTileX, by = la.planar ? 0 : pieces[k].y / lp->k.ty;
+                pf[k] = {off[(size_t)ptis[k]] + ((long long)by * la.nbx + bx) * la.len - la.z0, la.nbx * la.len, la.len, la.z0,
+                         (bx > 0 ? 1 : 0) | (bx + 1 < la.nbx ? 2 : 0) | (by > 0 ? 4 : 0) | (by + 1 < la.nby ? 8 : 0)};
+            }
+        std::vector<int> zero_flags((size_t)off[(size_t)n_tissues], 0);
+        if ((rc = upload(&lp->d_flags, &lp->cap_flags, zero_flags))) return rc;
+        if ((rc = upload(&lp->d_piece_flags, &lp->cap_pflags, pf))) return rc;
+        lp->epoch = 0;
+        lp->flow = true;
+    }
     lp->cta_stride = stride;
     lp->n_slots = (int)nslot;
     if (!lp->d_ticket) {
@@ -782,7 +819,32 @@ LaunchArgs launch_args(const LaunchPlan& lp, const TissueArgs* d_tissues, int* d
     L.poison_first_load = poison;
     L.cur_hint = -1;
     L.wait_limit = poison ? kPoisonWaitLimit : kWaitLimitCycles;
+    L.n_steps = 1;
+    L.flags = lp.d_flags;
+    L.piece_flags = lp.d_piece_flags;
     return L;
+}
+
+// Several steps of a plan in one cooperative launch (its CTAs wait for one
+// another between steps, plane by plane, so all of them must be resident).
+cudaError_t launch_flow(LaunchPlan* lp, LaunchArgs* L, int n_steps, cudaStream_t s) {
+    L->n_steps = n_steps;
+    L->epoch = (int)lp->epoch;
+    void* args[] = {(void*)L};
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(lp->ctas);
+    cfg.blockDim = dim3(lp->k.threads);
+    cfg.dynamicSmemBytes = (size_t)lp->k.smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, lp->k.fn, args);
+    if (e == cudaSuccess) lp->epoch += (unsigned int)n_steps;
+    L->n_steps = 1;
+    return e;
 }
 
 // A step launch, allowed to start while the previous kernel on the stream
@@ -848,12 +910,10 @@ struct bbx_grid {
 
     uint8_t* d_mask = nullptr;
     long long n_tissue = 0;
-    float* d_fib = nullptr;  // [3][nz][ny][pxf], x stored from -4 (clamped padding)
+    float* d_fib = nullptr;  // [3][nz][ny][px] unit fibres
     float* d_div = nullptr;  // [3][nz][ny][px]: the fixed W-tilde sums of every node (k_divergence)
     bool wsum_zero = false;  // every W-tilde sum is exactly 0 (the step need not load them)
     bool wsum_elide = true;  // skip loading vanishing sums (bbx_set_wsum_elision)
-    int pxf = 0;
-    long long fplane = 0, fvol = 0;
     bool aniso = false;
     double Dpar = 1.0, Dperp = 1.0;
 
@@ -1067,12 +1127,14 @@ void cover_chunks(const uint8_t* flags, int ncx, int nby, int nbz, int ty, int z
 }
 
 // Active columns (64 x ty nodes) of a grid with their active z-runs, for the
-// given tile rows (the brick list must have been built for g->ty).
-void grid_segments(const bbx_grid* g, int tissue, std::vector<Seg>* segs) {
+// the kernel's tile rows (those of a masked grid are g->ty, for which the brick
+// list must have been built).
+void grid_segments(const bbx_grid* g, int rows, int tissue, std::vector<Seg>* segs) {
+    const int nty = (g->ny + rows - 1) / rows;
     if (g->nz == 1) {
         // a sheet: runs of tiles down each column, (z0, z1) = tile range
         if (!g->d_mask) {
-            for (int bx = 0; bx < g->nbx; ++bx) segs->push_back({tissue, bx * kTileX, 0, 0, g->nby});
+            for (int bx = 0; bx < g->nbx; ++bx) segs->push_back({tissue, bx * kTileX, 0, 0, nty});
             return;
         }
         std::vector<std::vector<int>> col((size_t)g->nbx);
@@ -1092,8 +1154,8 @@ void grid_segments(const bbx_grid* g, int tissue, std::vector<Seg>* segs) {
     // a z-slab computes only the planes between its halo planes
     const int zlo = g->halo_lo, zhi = g->nz - g->halo_hi;
     if (!g->d_mask) {
-        for (int by = 0; by < g->nby; ++by)
-            for (int bx = 0; bx < g->nbx; ++bx) segs->push_back({tissue, bx * kTileX, by * g->ty, zlo, zhi});
+        for (int by = 0; by < nty; ++by)
+            for (int bx = 0; bx < g->nbx; ++bx) segs->push_back({tissue, bx * kTileX, by * rows, zlo, zhi});
         return;
     }
     std::vector<Seg> all;
@@ -1140,12 +1202,10 @@ int encode_targs(const bbx_grid* g, int ty, TissueArgs* t) {
         }
     }
     if (g->aniso) {
-        const cuuint64_t fd4[4] = {(cuuint64_t)g->pxf, (cuuint64_t)g->ny, (cuuint64_t)g->nz, 3};
-        const cuuint64_t fstr4[3] = {(cuuint64_t)g->pxf * 4, (cuuint64_t)g->fplane * 4, (cuuint64_t)g->fvol * 4};
+        const cuuint64_t fd4[4] = {(cuuint64_t)g->nx, (cuuint64_t)g->ny, (cuuint64_t)g->nz, 3};
         const cuuint32_t fbox[4] = {(cuuint32_t)kTileX, (cuuint32_t)ty, 1, 3};  // a tile's own fibres
-        if (!encode(&t->tm_f, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, g->d_fib, fd4, fstr4, fbox)) return BBX_ERR_CUDA;
-        const cuuint64_t dd4[4] = {(cuuint64_t)g->nx, (cuuint64_t)g->ny, (cuuint64_t)g->nz, 3};
-        if (!encode(&t->tm_d, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, g->d_div, dd4, str4, fbox)) return BBX_ERR_CUDA;
+        if (!encode(&t->tm_f, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, g->d_fib, fd4, str4, fbox)) return BBX_ERR_CUDA;
+        if (!encode(&t->tm_d, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, g->d_div, fd4, str4, fbox)) return BBX_ERR_CUDA;
     } else {
         t->tm_f = t->tm_u[0];
         t->tm_d = t->tm_u[0];
@@ -1189,6 +1249,13 @@ int encode_targs(const bbx_grid* g, int ty, TissueArgs* t) {
     t->tab = (g->model == BBX_BR_MRL || g->model == BBX_BR_FCA || (g->model == BBX_BR && g->tab_on)) ? g->d_tab
                                                                                                     : nullptr;
     return BBX_OK;
+}
+
+// The columns of an unmasked grid for tile rows `ty`.
+Lattice grid_lattice(const bbx_grid* g, int ty) {
+    const int nbx = (g->nx + kTileX - 1) / kTileX, nty = (g->ny + ty - 1) / ty;
+    if (g->nz == 1) return {nbx, 1, nty, 0, true};
+    return {nbx, nty, g->nz - g->halo_lo - g->halo_hi, g->halo_lo, false};
 }
 
 int finish_total(bbx_grid* g);
@@ -1261,12 +1328,14 @@ int prepare(bbx_grid* g) {
         rc = select_kernel(g->model, g->d_mask != nullptr, g->aniso ? AN_SUMS : AN_ISO, g->ty, g->device,
                            g->num_sms, &k, &ctas, surr, g->nz == 1, wants_general(g), g->gates);
     if (rc) return rc;
-    if ((rc = encode_targs(g, g->ty, &g->h_t))) return rc;
+    if ((rc = encode_targs(g, k.ty, &g->h_t))) return rc;
     BBX_CUDA(cudaMemcpyAsync(g->d_t, &g->h_t, sizeof(TissueArgs), cudaMemcpyHostToDevice, g->stream));
     std::vector<Seg> segs;
-    grid_segments(g, 0, &segs);
+    grid_segments(g, k.ty, 0, &segs);
     g->lp.k = k;
-    if ((rc = build_plan(&g->lp, segs, 1, ctas))) return rc;
+    std::vector<Lattice> lattice;
+    if (!g->d_mask) lattice.push_back(grid_lattice(g, k.ty));
+    if ((rc = build_plan(&g->lp, segs, 1, ctas, lattice, g->device))) return rc;
     BBX_CUDA(cudaStreamSynchronize(g->stream));
     g->ready = true;
     return BBX_OK;
@@ -1572,13 +1641,11 @@ int bbx_set_fibres(bbx_grid* g, const float* f, double D_par, double D_perp) {
     } else {
         float* tmp = nullptr;
         float* fib = nullptr;
-        const int pxf = (g->nx + 8 + 31) / 32 * 32;
-        const long long fplane = (long long)pxf * g->ny, fvol = fplane * g->nz;
         if (dmalloc(&tmp, sizeof(float) * 3 * g->ncell) != cudaSuccess) {
             cudaGetLastError();
             return BBX_ERR_NOMEM;
         }
-        if (dmalloc(&fib, sizeof(float) * 3 * fvol) != cudaSuccess) {
+        if (dmalloc(&fib, sizeof(float) * 3 * (size_t)g->vol) != cudaSuccess) {
             cudaGetLastError();
             cudaFree(tmp);
             return BBX_ERR_NOMEM;
@@ -1587,8 +1654,8 @@ int bbx_set_fibres(bbx_grid* g, const float* f, double D_par, double D_perp) {
         cudaError_t e = cudaMemcpyAsync(tmp, f, sizeof(float) * 3 * g->ncell, cudaMemcpyHostToDevice, g->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(g->d_err, 0, sizeof(int), g->stream);
         if (e == cudaSuccess) {
-            k_fibres<<<n_blocks_for(fvol, 256), 256, 0, g->stream>>>(tmp, g->nx, g->ny, g->nz, pxf, fplane, fvol,
-                                                                      g->d_mask, g->px, g->plane, fib, g->d_err);
+            k_fibres<<<n_blocks_for(g->vol, 256), 256, 0, g->stream>>>(tmp, g->nx, g->ny, g->nz, g->d_mask, g->px,
+                                                                        g->plane, g->vol, fib, g->d_err);
             e = cudaGetLastError();
         }
         if (e == cudaSuccess) e = cudaMemcpyAsync(&err, g->d_err, sizeof(int), cudaMemcpyDeviceToHost, g->stream);
@@ -1608,7 +1675,7 @@ int bbx_set_fibres(bbx_grid* g, const float* f, double D_par, double D_perp) {
                     // g->d_err is clear here (reset after the fibre check); it
                     // carries the "some sum is nonzero" word for this one call
                     k_divergence<<<n_blocks_for(g->ncell, 256), 256, 0, g->stream>>>(
-                        fib, g->nx, g->ny, g->nz, pxf, fplane, fvol, g->d_mask, g->px, g->plane, g->vol, div,
+                        fib, g->nx, g->ny, g->nz, g->d_mask, g->px, g->plane, g->vol, div,
                         g->d_err);
                     e = cudaGetLastError();
                 }
@@ -1631,9 +1698,6 @@ int bbx_set_fibres(bbx_grid* g, const float* f, double D_par, double D_perp) {
         cudaFree(g->d_div);
         g->d_fib = fib;
         g->d_div = div;
-        g->pxf = pxf;
-        g->fplane = fplane;
-        g->fvol = fvol;
         g->aniso = true;
         g->Dpar = D_par;
         g->Dperp = D_perp;
@@ -1947,12 +2011,23 @@ int bbx_step(bbx_grid* g, double dt, int n_steps) {
     if (!g->d_mask) {
         // unmasked grid: whole columns in order (nz planes, or a sheet's nby
         // tile rows), equal shares (build_plan)
-        L.reg_len = g->nz > 1 ? g->nz - g->halo_lo - g->halo_hi : g->nby;
+        L.reg_len = g->nz > 1 ? g->nz - g->halo_lo - g->halo_hi : (g->ny + g->lp.k.ty - 1) / g->lp.k.ty;
         L.reg_z0 = g->nz > 1 ? g->halo_lo : 0;
         L.reg_nbx = g->nbx;
-        L.reg_ty = g->ty;
+        L.reg_ty = g->lp.k.ty;
         L.reg_ctas = g->lp.ctas;
         L.reg_planes = g->lp.n_planes;
+    }
+    while (g->lp.flow && !g->poison && n_steps >= 2) {
+        const int m = std::min(n_steps, kFlowSteps);
+        L.cur_hint = g->h_cur;
+        if (launch_flow(&g->lp, &L, m, g->stream) != cudaSuccess) {
+            cudaGetLastError();  // not launchable as a whole: one launch per step from here on
+            g->lp.flow = false;
+            break;
+        }
+        g->h_cur ^= m & 1;
+        n_steps -= m;
     }
     for (int s = 0; s < n_steps; ++s) {
         L.cur_hint = g->h_cur;
@@ -2440,6 +2515,11 @@ int bbx_autotune(bbx_grid* g, double dt, double* best_ms) {
     int bty = g->ty, bzb = g->zb;
     rc = BBX_OK;
     for (int ty : tys) {
+        // 28 rows of an unmasked anisotropic light model leave one CTA per SM
+        // (256x256x64 slab 34 us a step against 22.8 with 14 rows, 512x512x256
+        // 400 against 345); on tissue at rest, which a grid often holds when it
+        // is tuned, the difference can vanish in the memory's own scatter
+        if (ty == 28 && !g->d_mask && g->aniso && g->S <= 2) continue;
         for (int zb : zbs) {
             if ((rc = bbx_set_tiling(g, ty, zb)) != BBX_OK) {
                 if (rc == BBX_ERR_UNSUPPORTED) {
@@ -2555,6 +2635,7 @@ struct bbx_batch {
     int graph_steps = 0;
     int* d_err = nullptr;
     bool built = false;
+    bool flow = false;  // several steps share a launch in every group
 };
 
 namespace {
@@ -2611,7 +2692,22 @@ int batch_build(bbx_batch* b, const std::vector<int>* tys) {
         if (tys && gi < tys->size()) gr.ty = (*tys)[gi];
         else if (gi < keep_ty.size()) gr.ty = keep_ty[gi];
     }
+    // Several steps share a launch where the batch is one group of unmasked
+    // light grids.  Cooperative launches of several groups are not sure to
+    // run side by side (two of them enqueued behind other work ran one after
+    // the other: 256 tissues 456 us a step against 340 by graphs of single
+    // steps).
+    b->flow = b->groups.size() == 1;
+    std::vector<int> full(b->groups.size(), 0);
+    for (size_t gi = 0; gi < b->groups.size(); ++gi) {
+        auto& gr = b->groups[gi];
+        int rc = select_kernel(gr.model, gr.masked, gr.aniso ? AN_SUMS : AN_ISO, gr.ty, b->device, b->num_sms, &gr.lp.k,
+                               &full[gi], gr.surr, gr.planar, gr.general);
+        if (rc) return rc;
+        b->flow = b->flow && gr.lp.k.flow;
+    }
     long long total_work = 0;
+    std::vector<std::vector<Lattice>> lattice(b->groups.size());
     std::vector<std::vector<Seg>> segs(b->groups.size());
     for (size_t gi = 0; gi < b->groups.size(); ++gi) {
         auto& gr = b->groups[gi];
@@ -2625,15 +2721,17 @@ int batch_build(bbx_batch* b, const std::vector<int>* tys) {
                 int rc = build_bricks(g);
                 if (rc) { g->ty = ty0; build_bricks(g); return rc; }
             }
-            grid_segments(g, (int)m, &segs[gi]);
-            int rc = encode_targs(g, gr.ty, &ta[m]);
+            grid_segments(g, gr.lp.k.ty, (int)m, &segs[gi]);
+            int rc = encode_targs(g, gr.lp.k.ty, &ta[m]);
+            lattice[gi].push_back(grid_lattice(g, gr.lp.k.ty));
             if (g->ty != ty0) {
                 g->ty = ty0;
                 build_bricks(g);
             }
             if (rc) return rc;
         }
-        for (const Seg& sg : segs[gi]) gr.work += (long long)(sg.z1 - sg.z0);
+        // (a group's cost goes with its nodes, whatever its tile height)
+        for (const Seg& sg : segs[gi]) gr.work += (long long)(sg.z1 - sg.z0) * gr.lp.k.ty;
         total_work += gr.work;
         if (dmalloc(&gr.d_t, sizeof(TissueArgs) * ta.size()) != cudaSuccess) {
             cudaGetLastError();
@@ -2645,48 +2743,52 @@ int batch_build(bbx_batch* b, const std::vector<int>* tys) {
     }
     for (size_t gi = 0; gi < b->groups.size(); ++gi) {
         auto& gr = b->groups[gi];
-        int ctas = 0;
-        int rc = select_kernel(gr.model, gr.masked, gr.aniso ? AN_SUMS : AN_ISO, gr.ty, b->device, b->num_sms, &gr.lp.k, &ctas, gr.surr,
-                               gr.planar, gr.general);
-        if (rc) return rc;
-        long long share = total_work > 0 ? (long long)((double)ctas * gr.work / total_work + 0.5) : 1;
+        const double part = total_work > 0 ? (double)full[gi] * gr.work / total_work : 1.0;
+        long long share = (long long)(b->flow ? part : part + 0.5);
         if (share < 1) share = 1;
-        if ((rc = build_plan(&gr.lp, segs[gi], (int)gr.members.size(), (int)share))) return rc;
+        int rc = build_plan(&gr.lp, segs[gi], (int)gr.members.size(), (int)share,
+                            b->flow ? lattice[gi] : std::vector<Lattice>(), b->device);
+        if (rc) return rc;
     }
+    for (auto& gr : b->groups) b->flow = b->flow && (gr.lp.flow || gr.lp.n_planes == 0);
     b->versions.clear();
     for (bbx_grid* g : b->grids) b->versions.push_back(g->version);
     b->built = true;
     return BBX_OK;
 }
 
-// One batch step of grids that hold no tissue (a group without pieces):
+// Batch steps of grids that hold no tissue (a group without pieces):
 // nothing moves, time, step count and parity advance as for the others.
-__global__ void k_advance_empty(const TissueArgs* __restrict__ T, int n) {
+__global__ void k_advance_empty(const TissueArgs* __restrict__ T, int n, int n_steps) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         TissueDyn* d = T[i].dyn;
         d->total = 0.0;
-        d->t = d->t + T[i].dt_d;
-        d->n = d->n + 1;
-        d->cur = d->cur ^ 1;
+        double t = d->t;
+        for (int s = 0; s < n_steps; ++s) t = t + T[i].dt_d;
+        d->t = t;
+        d->n = d->n + n_steps;
+        d->cur = d->cur ^ (n_steps & 1);
         d->total_pending = 0;
     }
 }
 
-int batch_launch_step(bbx_batch* b) {
+// n_steps steps of every group, side by side: one (the graph's node), or up
+// to kFlowSteps in one launch a group (b->flow).
+int batch_launch_step(bbx_batch* b, int n_steps = 1) {
     BBX_CUDA(cudaEventRecord(b->fork, b->ps));
     for (auto& gr : b->groups) {
         if (gr.lp.n_planes == 0) {
             if (gr.members.empty()) continue;
             BBX_CUDA(cudaStreamWaitEvent(gr.s, b->fork, 0));
-            k_advance_empty<<<1, 32, 0, gr.s>>>(gr.d_t, (int)gr.members.size());
+            k_advance_empty<<<1, 32, 0, gr.s>>>(gr.d_t, (int)gr.members.size(), n_steps);
             BBX_CUDA(cudaGetLastError());
             BBX_CUDA(cudaEventRecord(gr.done, gr.s));
             BBX_CUDA(cudaStreamWaitEvent(b->ps, gr.done, 0));
             continue;
         }
         BBX_CUDA(cudaStreamWaitEvent(gr.s, b->fork, 0));
-        const LaunchArgs L = launch_args(gr.lp, gr.d_t, b->d_err, 0);
-        BBX_CUDA(launch(gr.lp, L, gr.s));
+        LaunchArgs L = launch_args(gr.lp, gr.d_t, b->d_err, 0);
+        BBX_CUDA(n_steps > 1 ? launch_flow(&gr.lp, &L, n_steps, gr.s) : launch(gr.lp, L, gr.s));
         BBX_CUDA(cudaEventRecord(gr.done, gr.s));
         BBX_CUDA(cudaStreamWaitEvent(b->ps, gr.done, 0));
     }
@@ -2778,13 +2880,20 @@ int bbx_batch_step(bbx_batch* b, int n_steps) {
     }
     int rc;
     if (!b->built && (rc = batch_build(b, nullptr))) return rc;
-    const int chunk = n_steps < 16 ? n_steps : 16;
-    if (n_steps >= 2 && b->graph_steps != chunk && (rc = batch_capture(b, chunk))) return rc;
+    // without shared launches: graphs of up to 16 steps
+    const int chunk = b->flow ? 1 : (n_steps < 16 ? n_steps : 16);
+    if (chunk >= 2 && b->graph_steps != chunk && (rc = batch_capture(b, chunk))) return rc;
     // order the batch's stream after the members' stream, and back
     BBX_CUDA(cudaEventRecord(b->enter, b->stream));
     BBX_CUDA(cudaStreamWaitEvent(b->ps, b->enter, 0));
     int done = 0;
-    if (n_steps >= 2) {
+    if (b->flow) {
+        while (n_steps - done >= 2) {
+            const int m = std::min(n_steps - done, kFlowSteps);
+            if ((rc = batch_launch_step(b, m))) return rc;
+            done += m;
+        }
+    } else if (n_steps >= 2) {
         for (; done + chunk <= n_steps; done += chunk) BBX_CUDA(cudaGraphLaunch(b->gexec, b->ps));
     }
     for (; done < n_steps; ++done)
@@ -2851,9 +2960,10 @@ int bbx_batch_autotune(bbx_batch* b, double* best_ms) {
             if (r == BBX_ERR_UNSUPPORTED) continue;
             if (r) { rc = r; break; }
             cudaStreamSynchronize(b->stream);
-            for (int s = 0; s < 2 && rc == BBX_OK; ++s) rc = batch_launch_step(b);
+            const int per = b->flow ? 4 : 1;  // steps of a launch
+            for (int s = 0; s < 4 && rc == BBX_OK; s += per) rc = batch_launch_step(b, per);
             cudaEventRecord(e0, b->ps);
-            for (int s = 0; s < 4 && rc == BBX_OK; ++s) rc = batch_launch_step(b);
+            for (int s = 0; s < 4 && rc == BBX_OK; s += per) rc = batch_launch_step(b, per);
             cudaEventRecord(e1, b->ps);
             cudaEventSynchronize(e1);
             float ms = 0.f;

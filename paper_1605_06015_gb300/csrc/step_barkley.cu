@@ -7,7 +7,7 @@ template <bool MA, int AN, int TY, bool PL, bool GE>
 static StepKernel make_barkley() {
     using P = Plan<BBX_BARKLEY, MA, AN, TY>;
     return StepKernel{reinterpret_cast<const void*>(&step_kernel<BBX_BARKLEY, MA, AN, TY, false, PL, GE>), P::SMEM,
-                      P::THREADS, TY};
+                      P::THREADS, TY, P::FLOW};
 }
 
 // planar: grids with nz = 1 (tiles marched along y); general: the variant
