@@ -577,6 +577,54 @@ __device__ __forceinline__ float expm1_br(float x) {
     return __expf(x) - 1.0f;
 }
 
+// Powers of two, logarithm and reciprocal by the special-function unit, for
+// pairs; results below the normal range are 0.
+__device__ __forceinline__ float2 ex2_pair(float2 a) {
+    float2 r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(a.x));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(a.y));
+    return r;
+}
+__device__ __forceinline__ float2 lg2_pair(float2 a) {
+    float2 r;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(a.x));
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(a.y));
+    return r;
+}
+__device__ __forceinline__ float2 rcp_pair(float2 a) {
+    float2 r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(a.x));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(a.y));
+    return r;
+}
+// a e^{k (V + c)} with log2a = log2(a): one multiply-add and one power of two.
+__device__ __forceinline__ float2 exp_rate(float2 V, double k, double c, double log2a) {
+    constexpr double l2e = 1.4426950408889634;
+    return ex2_pair(fma2(V, splat2((float)(k * l2e)), splat2((float)(k * c * l2e + log2a))));
+}
+// 1 / a and 1 / b by one reciprocal.
+__device__ __forceinline__ void rcp_both(float2 a, float2 b, float2* ra, float2* rb) {
+    const float2 i = rcp_pair(mul2(a, b));
+    *ra = mul2(i, b);
+    *rb = mul2(i, a);
+}
+// (1 - e^{-z}) / z for |z| < 1/4: its Taylor series to z^5/720 (the first
+// omitted term is below 5e-8).
+__device__ __forceinline__ float2 phi_series(float2 z) {
+    float2 p = fma2(z, splat2(-1.0f / 720.0f), splat2(1.0f / 120.0f));
+    p = fma2(z, p, splat2(-1.0f / 24.0f));
+    p = fma2(z, p, splat2(1.0f / 6.0f));
+    p = fma2(z, p, splat2(-0.5f));
+    return fma2(z, p, splat2(1.0f));
+}
+// The same for any z >= 0: by the power of two where z >= 1/4 (1 - e^{-z} >= 0.22 there).
+__device__ __forceinline__ float2 phi_any(float2 z) {
+    const float2 q = phi_series(z);
+    const float2 e = ex2_pair(mul2(z, splat2(-1.44269504f)));
+    const float2 r = mul2(sub2(splat2(1.0f), e), rcp_pair(z));
+    return make_float2(z.x < 0.25f ? q.x : r.x, z.y < 0.25f ? q.y : r.y);
+}
+
 // Voltage tables of the Beeler-Reuter models: kTabN entries kTabDv mV apart
 // from kTabVmin (-120 to +80 mV), 16 floats (4 float4) each; V outside the
 // range takes the end entry.  Entry index and interpolation weight of V.
@@ -667,6 +715,102 @@ struct Model<BBX_BR> {
         increment(mp, y, L, Is, dt, d);
 #pragma unroll
         for (int v = 0; v < 8; ++v) y[v] = y[v] + d[v];
+    }
+
+    // The same for a pair of nodes (Is the stimulus).  What bounds it is the
+    // number of instructions: update() takes about 470 per node (each
+    // exponential, logarithm and division carries the scaling of its denormal
+    // range), this about 110.  Exponents are one multiply-add; exponentials
+    // that are powers of one another (0.02, 0.04, 0.06 and 0.1, 0.2 per mV)
+    // share one; the two rates of a gate share one reciprocal; and the
+    // Rush-Larsen increment (1 - e^{-s dt}) (alpha/s - y), s = alpha + beta,
+    // is taken as dt phi(s dt) (alpha - s y), phi(z) = (1 - e^{-z})/z, which
+    // needs no division.  For V in (-140, 120) mV and dt <= 0.19 ms, where no
+    // exponential leaves the range and s dt < 1/4 for x1, j, d, f; update()
+    // elsewhere.
+    __device__ static __forceinline__ void update2(const float* mp, float2* y, float2 L, float2 Is, float dt) {
+        const float2 V = y[0], Ca = y[1];
+        if (!(fminf(V.x, V.y) > -140.0f && fmaxf(V.x, V.y) < 120.0f && dt <= 0.19f)) {
+            float a[8], b[8];
+#pragma unroll
+            for (int v = 0; v < 8; ++v) {
+                a[v] = y[v].x;
+                b[v] = y[v].y;
+            }
+            update(mp, a, L.x, Is.x, dt);
+            update(mp, b, L.y, Is.y, dt);
+#pragma unroll
+            for (int v = 0; v < 8; ++v) y[v] = make_float2(a[v], b[v]);
+            return;
+        }
+        const float2 one = splat2(1.0f);
+        const float2 R = exp_rate(V, -0.02, 20.0, 0.0);  // e^{-0.02 (V + 20)}
+        const float2 R2 = mul2(R, R);                    // e^{-0.04 (V + 20)}
+        const float2 P = exp_rate(V, -0.1, 47.0, 0.0);   // e^{-0.1 (V + 47)}
+        const float2 P2 = mul2(P, P);                    // e^{-0.2 (V + 47)}
+
+        // the removable singularities w / (1 - e^{-z}), z = k w: alpha_m (w = V + 47, k = 0.1) and
+        // the linear part of I_K1 (w = V + 23, k = 0.04); 1 / (k phi(z)) near 0
+        float2 nm = add2(V, splat2(47.0f)), dm = sub2(one, P);
+        float2 nl = add2(V, splat2(23.0f)), dl = fma2(R2, splat2(-0.8869204367f), one);  // e^{-0.12}
+        if (fminf(fabsf(nm.x), fabsf(nm.y)) < 2.5f) {
+            const float2 q = phi_series(mul2(nm, splat2(0.1f)));
+            if (fabsf(nm.x) < 2.5f) { nm.x = 10.0f; dm.x = q.x; }
+            if (fabsf(nm.y) < 2.5f) { nm.y = 10.0f; dm.y = q.y; }
+        }
+        if (fminf(fabsf(nl.x), fabsf(nl.y)) < 6.25f) {
+            const float2 q = phi_series(mul2(nl, splat2(0.04f)));
+            if (fabsf(nl.x) < 6.25f) { nl.x = 25.0f; dl.x = q.x; }
+            if (fabsf(nl.y) < 6.25f) { nl.y = 25.0f; dl.y = q.y; }
+        }
+        float2 im, il;
+        rcp_both(dm, dl, &im, &il);
+        const float2 a_m = mul2(nm, im);
+        const float2 lin = mul2(nl, il);  // (0.2 w / (1 - e^{-z}) = 0.2 lin)
+
+        // membrane currents
+        const float2 V_ENa = add2(V, splat2(-mp[2]));
+        const float2 m3hj = mul2(mul2(mul2(y[3], y[3]), y[3]), mul2(y[4], y[5]));
+        const float2 INa = mul2(fma2(m3hj, splat2(mp[0]), splat2(mp[1])), V_ENa);
+        // V - E_s = V + 82.3 + 13.0287 ln Ca
+        const float2 V_Es = fma2(lg2_pair(Ca), splat2(9.03080667f), add2(V, splat2(82.3f)));
+        const float2 Is_ = mul2(mul2(mul2(y[6], y[7]), splat2(mp[3])), V_Es);
+        // 0.8 (e^{0.04 (V + 77)} - 1) e^{-0.04 (V + 35)}
+        const float2 Ix1 = mul2(y[2], fma2(R2, splat2(-0.439049309f), splat2(4.29244478f)));
+        // 4 (e^{0.04 (V + 85)} - 1) / (e^{0.08 (V + 53)} + e^{0.04 (V + 53)}), r = e^{-0.04 (V + 53)}
+        const float2 r = mul2(R2, splat2(0.267135302f));
+        const float2 Eh = exp_rate(V, -0.082, 22.5, 0.0);
+        float2 ik, bh;
+        rcp_both(add2(one, r), add2(one, Eh), &ik, &bh);
+        const float2 k1 = mul2(mul2(r, sub2(splat2(3.59663973f), r)), ik);
+        const float2 IK1 = fma2(k1, splat2(1.4f), mul2(lin, splat2(0.07f)));
+        const float2 Iion = add2(add2(INa, Is_), add2(Ix1, IK1));
+        const float2 dCa = fma2(Is_, splat2(-1e-7f), fma2(Ca, splat2(-0.07f), splat2(7e-9f)));
+
+        // the gates: alpha and beta, 1/ms
+        auto gate = [&](int v, float2 al, float2 be, bool any) {
+            const float2 s = add2(al, be), z = mul2(s, splat2(dt));
+            const float2 t = fma2(s, make_float2(-y[v].x, -y[v].y), al);
+            y[v] = fma2(mul2(any ? phi_any(z) : phi_series(z), t), splat2(dt), y[v]);
+        };
+        auto gate2 = [&](int v, float2 n1, float2 d1, float2 n2, float2 d2) {
+            float2 i1, i2;
+            rcp_both(d1, d2, &i1, &i2);
+            gate(v, mul2(n1, i1), mul2(n2, i2), false);
+        };
+        const float2 a_h = exp_rate(V, -0.25, 77.0, -2.9885043611621702);
+        gate2(2, exp_rate(V, 0.026, 50.0, -10.965784284662087), add2(one, exp_rate(V, -0.057, 50.0, 0.0)),
+              mul2(mul2(R2, R), splat2(0.0013f)), add2(R2, one));
+        gate(3, a_m, exp_rate(V, -0.056, 72.0, 5.321928094887363), true);
+        gate(4, a_h, mul2(bh, splat2(1.7f)), true);
+        gate2(5, mul2(a_h, splat2(0.339952723f)), fma2(P2, splat2(0.00202943064f), one), splat2(0.3f),
+              fma2(P, splat2(4.48168907f), one));
+        gate2(6, exp_rate(V, -0.01, -5.0, -3.3959286763311392), add2(one, exp_rate(V, -0.072, -5.0, 0.0)),
+              exp_rate(V, -0.017, 44.0, -3.8365012677171206), add2(one, exp_rate(V, 0.05, 44.0, 0.0)));
+        gate2(7, exp_rate(V, -0.008, 28.0, -6.380821783940931), add2(one, exp_rate(V, 0.15, 28.0, 0.0)),
+              mul2(R, splat2(0.00532174991f)), fma2(P2, splat2(29.9641000f), one));
+        y[0] = fma2(splat2(dt), add2(sub2(Is, Iion), L), V);  // Cm = 1
+        y[1] = fma2(splat2(dt), dCa, Ca);
     }
 
     // The same step with the Rush-Larsen coefficients tabulated in V (the
@@ -1281,62 +1425,59 @@ template <int MODEL, bool SURR, bool GEN>
 __device__ __forceinline__ void react_pair(const PieceSlot& a, const float* mp, float dt, unsigned char* wbufs,
                                            const bool* live, float2* y, float2 L, float2 Is) {
     constexpr int S = Model<MODEL>::S;
-    if constexpr (MODEL == BBX_BR || MODEL == BBX_BR_MRL || MODEL == BBX_BR_FCA) {
+    if constexpr (MODEL == BBX_BR && SURR) {
+        // the surrogate where the state is inside the training envelope and V
+        // below the upstroke threshold; the exact model elsewhere
+        const SurrogateData* W = a.surr;
         float ys[2][S];
-        const float Ls[2] = {L.x, L.y}, Iss[2] = {Is.x, Is.y};
 #pragma unroll
         for (int v = 0; v < S; ++v) {
             ys[0][v] = y[v].x;
             ys[1][v] = y[v].y;
         }
-        if constexpr (SURR && MODEL == BBX_BR) {
-            // the surrogate where the state is inside the training envelope and V
-            // below the upstroke threshold; the exact model elsewhere
-            const SurrogateData* W = a.surr;
-            bool want[2] = {false, false};
-            if (W) {
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    bool in = live[e] && ys[e][0] < W->v_up;
-#pragma unroll
-                    for (int v = 0; v < S; ++v) in = in && ys[e][v] >= W->norm[32 + v] && ys[e][v] <= W->norm[40 + v];
-                    want[e] = in;
-                }
-            }
-            if (__any_sync(0xffffffffu, want[0] || want[1])) {
-                float dsur[2][8];
-                surrogate_warp64(W, wbufs + (threadIdx.x >> 5) * 2048, ys, dsur);
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    if (want[e]) {
-#pragma unroll
-                        for (int v = 0; v < S; ++v) ys[e][v] += dsur[e][v];
-                        ys[e][0] += dt * (Ls[e] + Iss[e]);
-                    } else {
-                        Model<MODEL>::update(mp, ys[e], Ls[e], Iss[e], dt);
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int e = 0; e < 2; ++e) Model<MODEL>::update(mp, ys[e], Ls[e], Iss[e], dt);
-            }
-        } else {
-            // tabulated Rush-Larsen coefficients (of BBX_BR in the general
-            // variants only, so the default kernel carries no code for them)
+        bool want[2] = {false, false};
+        if (W) {
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-                if constexpr (MODEL != BBX_BR) {
-                    Model<MODEL>::update_tab(mp, a.tab, ys[e], Ls[e], Iss[e], dt);
-                } else {
-                    if (GEN && a.tab)
-                        Model<MODEL>::update_tab(mp, a.tab, ys[e], Ls[e], Iss[e], dt);
-                    else
-                        Model<MODEL>::update(mp, ys[e], Ls[e], Iss[e], dt);
-                }
+                bool in = live[e] && ys[e][0] < W->v_up;
+#pragma unroll
+                for (int v = 0; v < S; ++v) in = in && ys[e][v] >= W->norm[32 + v] && ys[e][v] <= W->norm[40 + v];
+                want[e] = in;
             }
         }
+        const bool some = __any_sync(0xffffffffu, want[0] || want[1]);
+        if (!(want[0] && want[1])) Model<MODEL>::update2(mp, y, L, Is, dt);
+        if (some) {
+            float dsur[2][8];
+            surrogate_warp64(W, wbufs + (threadIdx.x >> 5) * 2048, ys, dsur);
+            if (want[0]) {
 #pragma unroll
-        for (int v = 0; v < S; ++v) y[v] = make_float2(ys[0][v], ys[1][v]);
+                for (int v = 0; v < S; ++v) y[v].x = ys[0][v] + dsur[0][v];
+                y[0].x += dt * (L.x + Is.x);
+            }
+            if (want[1]) {
+#pragma unroll
+                for (int v = 0; v < S; ++v) y[v].y = ys[1][v] + dsur[1][v];
+                y[0].y += dt * (L.y + Is.y);
+            }
+        }
+    } else if constexpr (MODEL == BBX_BR || MODEL == BBX_BR_MRL || MODEL == BBX_BR_FCA) {
+        // tabulated Rush-Larsen coefficients (of BBX_BR in the general
+        // variants only, so the default kernel carries no code for them)
+        if (MODEL != BBX_BR || (GEN && a.tab)) {
+            float ys[2][S];
+#pragma unroll
+            for (int v = 0; v < S; ++v) {
+                ys[0][v] = y[v].x;
+                ys[1][v] = y[v].y;
+            }
+            Model<MODEL>::update_tab(mp, a.tab, ys[0], L.x, Is.x, dt);
+            Model<MODEL>::update_tab(mp, a.tab, ys[1], L.y, Is.y, dt);
+#pragma unroll
+            for (int v = 0; v < S; ++v) y[v] = make_float2(ys[0][v], ys[1][v]);
+        } else if constexpr (MODEL == BBX_BR) {
+            Model<MODEL>::update2(mp, y, L, Is, dt);
+        }
     } else {
         const float2 src = add2(L, Is);
         if (GEN && a.rk4) {
