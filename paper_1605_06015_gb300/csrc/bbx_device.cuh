@@ -60,7 +60,7 @@ struct TissueArgs {  // (CUtensorMap members impose its alignment)
     CUtensorMap tm_g[2];  // 16-bit gates of buffer b (box TX x TY x 6 uint16), when stored so
     CUtensorMap tm_f;     // unit fibres (box TX x TY x 3, no halo)
     CUtensorMap tm_d;     // the W-tilde sums of every node (box TX x TY x 3)
-    CUtensorMap tm_m;     // tissue mask bytes
+    CUtensorMap tm_m;     // neighbour words of a masked grid (box TX x TY, no halo)
     float* state[2];      // the ping-pong buffers, var v at state[b] + v*vol (32-bit variables)
     uint16_t* gate16[2];  // 16-bit gates: gate g (variable 2 + g) at gate16[b] + g*vol, or nullptr
     int32_t* act;         // activation steps
@@ -75,8 +75,7 @@ struct TissueArgs {  // (CUtensorMap members impose its alignment)
     int rk4;    // kinetics solver: 1 classical RK4 (right-hand-side models), 0 forward Euler / Rush-Larsen
     int wsum_zero;  // 1: every W-tilde sum of the grid is exactly 0 (a single-grid launch then skips their copies)
     // diffusion constants over h^2: anisotropic D = Dperp I + (Dpar-Dperp) f f^T
-    // gives c_perp = Dperp/h^2, c_d = (Dpar-Dperp)/h^2, c_dh = c_d/2 (edge
-    // weights), c_s = c_d/4 (Wtilde); isotropic D gives c_iso = D/h^2.
+    // gives c_perp = Dperp/h^2, c_d = (Dpar-Dperp)/h^2, c_s = c_d/4 (Wtilde); isotropic D gives c_iso = D/h^2.
     float c_perp, c_d, c_dh, c_s, c_iso;
     float mp[8];  // model parameters in kernel form
     const struct SurrogateData* surr;  // reaction surrogate (Beeler-Reuter), or nullptr
@@ -1088,6 +1087,18 @@ constexpr int align128(int b) { return (b + 127) & ~127; }
 // 18 stencil neighbours are all tissue inside the array ("interior").
 enum : uint8_t { MASK_TISSUE = 1, MASK_INTERIOR = 2 };
 
+// Per-node word of a masked grid, as the step reads it (a tile's own words,
+// 4 B a node, instead of three planes of mask bytes with their halo and a
+// byte load and a test for each neighbour): the grid indicator psi of the 18
+// stencil neighbours, then the node's own two mask bits.
+enum : uint32_t {
+    PSI_XP = 1u << 0, PSI_XM = 1u << 1, PSI_YP = 1u << 2, PSI_YM = 1u << 3, PSI_ZP = 1u << 4, PSI_ZM = 1u << 5,
+    PSI_XPYP = 1u << 6, PSI_XMYM = 1u << 7, PSI_XPYM = 1u << 8, PSI_XMYP = 1u << 9,
+    PSI_XPZP = 1u << 10, PSI_XMZM = 1u << 11, PSI_XPZM = 1u << 12, PSI_XMZP = 1u << 13,
+    PSI_YPZP = 1u << 14, PSI_YMZM = 1u << 15, PSI_YPZM = 1u << 16, PSI_YMZP = 1u << 17,
+    PSI_TISSUE = 1u << 18, PSI_INTERIOR = 1u << 19
+};
+
 // Storage of the Beeler-Reuter gates (variables 2..7) between steps: FP32
 // (default), IEEE binary16, or 16-bit unsigned fixed point y = u / 65535
 // (uniform steps of 1.5e-5 over [0, 1]); arithmetic is FP32 in every case,
@@ -1134,19 +1145,17 @@ struct Plan {
     static constexpr int THREADS = step_threads(TY, MASKED, S);  // consumer warps + producer warp (+ sync warp)
     static constexpr int UW = TX + 8;   // x from x0-4 to x0+TX+3 (16-byte aligned start)
     static constexpr int UH = TY + 2;   // y from y0-1 to y0+TY
-    static constexpr int MW = TX + 32;  // mask bytes: x from x0-16 (16-byte aligned start)
     // ring A, one stage per loaded plane (the computed planes and the z-halo
-    // planes): V with its one-node halo, the mask with its halo
+    // planes): V with its one-node halo
     static constexpr int U_RAW = UW * UH * 4;
-    static constexpr int M_RAW = MASKED ? MW * UH : 0;
     static constexpr int U_OFF = 0;
-    static constexpr int M_OFF = U_OFF + align128(U_RAW);
     // (each stage ends with its two mbarriers, so a stage's address gives them)
-    static constexpr int A_BAR = M_OFF + align128(M_RAW);
+    static constexpr int A_BAR = U_OFF + align128(U_RAW);
     static constexpr int A_STAGE = A_BAR + 128;
-    static constexpr uint32_t A_BYTES = U_RAW + M_RAW;
+    static constexpr uint32_t A_BYTES = U_RAW;
     // ring B, one stage per computed plane: the node's own unit fibre and
-    // W-tilde sums (3 x TX x TY floats each), the other variables
+    // W-tilde sums (3 x TX x TY floats each), the other variables, the
+    // neighbour words of a masked grid
     static constexpr int F_RAW = ANISO ? 3 * TX * TY * 4 : 0;
     static constexpr int D_RAW = ANISO == AN_SUMS ? 3 * TX * TY * 4 : 0;
     static constexpr int S32_RAW = (S > 1) ? (S - 1 - NG) * TX * TY * 4 : 0;  // 32-bit non-diffusing variables
@@ -1156,9 +1165,11 @@ struct Plan {
     static constexpr int D_OFF = F_OFF + F_RAW;    // (each part a multiple of 128 bytes)
     static constexpr int S_OFF = D_OFF + D_RAW;
     static constexpr int G_OFF = S_OFF + S32_RAW;
-    static constexpr int B_BAR = align128(F_RAW + D_RAW + S_RAW);
+    static constexpr int M_RAW = MASKED ? TX * TY * 4 : 0;
+    static constexpr int M_OFF = G_OFF + G_RAW;
+    static constexpr int B_BAR = align128(F_RAW + D_RAW + S_RAW + M_RAW);
     static constexpr int B_STAGE = B_BAR + 128;
-    static constexpr uint32_t B_BYTES = F_RAW + D_RAW + S_RAW;
+    static constexpr uint32_t B_BYTES = F_RAW + D_RAW + S_RAW + M_RAW;
     static constexpr bool HAS_B = B_BYTES > 0;
     static constexpr int BUDGET = (CTAS == 1 ? 200 : (CTAS == 2 ? 112 : (CTAS == 3 ? 72 : 54))) * 1024;  // dynamic shared memory per CTA
     static constexpr int NB_FIT = HAS_B ? (BUDGET - 5 * A_STAGE) / B_STAGE : 0;
@@ -1170,20 +1181,7 @@ struct Plan {
     // stages with their barriers, warp buffers, piece contexts
     static constexpr int SMEM = 128 + RING_OFF + NA * 176;
     static_assert(TY % RY == 0 && CY >= 1, "tile rows must be a multiple of the thread rows");
-    static_assert(U_RAW % 16 == 0 && F_RAW % 128 == 0 && D_RAW % 128 == 0 && S32_RAW % 128 == 0, "stage layout");
-};
-
-struct F3 {
-    float x, y, z;
-};
-
-// Neighbour values of one node: faces, then the 12 edges of the 19-point
-// stencil ("pm" = x+1,y-1 etc.).
-struct Nb {
-    float u0, xp, xm, yp, ym, zp, zm;
-    float pp, mm, pm, mp;          // (x,y) edges
-    float xpzp, xmzm, xpzm, xmzp;  // (x,z) edges
-    float ypzp, ymzm, ypzm, ymzp;  // (y,z) edges
+    static_assert(U_RAW % 16 == 0 && F_RAW % 128 == 0 && D_RAW % 128 == 0 && S32_RAW % 128 == 0 && G_RAW % 128 == 0, "stage layout");
 };
 
 // The precomputed ingredients of Eq. (Lu) at a node: the unit fibre f (D =
@@ -1232,47 +1230,6 @@ __device__ __forceinline__ float2 lap_pair(const Coef& a, const Diffs& d, const 
     }
     return L;
 }
-
-// Grid indicator psi of the 18 neighbours (bit order: xp xm yp ym zp zm, then
-// pp mm pm mp, xpzp xmzm xpzm xmzp, ypzp ymzm ypzm ymzp).
-struct Psi {
-    bool xp, xm, yp, ym, zp, zm;
-    bool pp, mm, pm, mp;
-    bool xpzp, xmzm, xpzm, xmzp;
-    bool ypzp, ymzm, ypzm, ymzp;
-};
-
-// (L u)_p for any tissue node: every weight carries its psi (a void or
-// out-of-array neighbour contributes nothing); the W-tilde sums already hold
-// a void neighbour's tensor replaced by D^p.
-template <int ANISO>
-__device__ __forceinline__ float lap_general(const Coef& a, const Nb& n, const Psi& q, F3 f, F3 sd) {
-    auto d = [&](bool ps, float uq) { return ps ? (uq - n.u0) : 0.0f; };
-    const float exp_ = d(q.xp, n.xp), exm = d(q.xm, n.xm), eyp = d(q.yp, n.yp), eym = d(q.ym, n.ym);
-    const float ezp = d(q.zp, n.zp), ezm = d(q.zm, n.zm);
-    if (!ANISO) {
-        return a.c_iso * (((exp_ + exm) + (eyp + eym)) + (ezp + ezm));
-    }
-    const float Dxx = fmaf(a.c_d, f.x * f.x, a.c_perp);
-    const float Dyy = fmaf(a.c_d, f.y * f.y, a.c_perp);
-    const float Dzz = fmaf(a.c_d, f.z * f.z, a.c_perp);
-    const float hx = a.c_dh * f.x;
-    const float Dxy = hx * f.y, Dxz = hx * f.z, Dyz = a.c_dh * f.y * f.z;
-    float L = Dxx * (exp_ + exm);
-    L = fmaf(Dyy, eyp + eym, L);
-    L = fmaf(Dzz, ezp + ezm, L);
-    if (ANISO == AN_SUMS) {
-        float dv = (q.xp && q.xm) ? sd.x * (n.xp - n.xm) : 0.0f;
-        if (q.yp && q.ym) dv = fmaf(sd.y, n.yp - n.ym, dv);
-        if (q.zp && q.zm) dv = fmaf(sd.z, n.zp - n.zm, dv);
-        L = fmaf(a.c_s, dv, L);
-    }
-    L = fmaf(Dxy, (d(q.pp, n.pp) + d(q.mm, n.mm)) - (d(q.pm, n.pm) + d(q.mp, n.mp)), L);
-    L = fmaf(Dxz, (d(q.xpzp, n.xpzp) + d(q.xmzm, n.xmzm)) - (d(q.xpzm, n.xpzm) + d(q.xmzp, n.xmzp)), L);
-    L = fmaf(Dyz, (d(q.ypzp, n.ypzp) + d(q.ymzm, n.ymzm)) - (d(q.ypzm, n.ypzm) + d(q.ymzp, n.ymzp)), L);
-    return L;
-}
-
 
 // ---------------------------------------------------------------------------
 // the fused step kernel
@@ -1548,7 +1505,7 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
     using P = Plan<MODEL, MASKED, ANISO, TY, SURR, GATES>;
     static_assert(GATES == GATES_F32 || (MODEL == BBX_BR && !SURR), "16-bit gates: Beeler-Reuter without surrogate");
     constexpr int NG = P::NG, S32 = P::S - NG;  // 16-bit variables last
-    constexpr int S = P::S, TX = P::TX, UW = P::UW, MW = P::MW, CY = P::CY;
+    constexpr int S = P::S, TX = P::TX, UW = P::UW, CY = P::CY;
     constexpr int NS = P::NA;            // ring A: loaded planes
     constexpr int NB = P::NB;            // ring B: computed planes (0: nothing beyond V and the mask)
     constexpr bool HB = P::HAS_B;
@@ -1652,6 +1609,7 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
             }
             if (S > 1 && S32 > 1) tma_load_4d(sb + P::S_OFF, &T->tm_s[src], x0, y0, z, 1, bar);
             if (NG) tma_load_4d(sb + P::G_OFF, &T->tm_g[src], x0, y0, z, 0, bar);
+            if (MASKED) tma_load_3d(sb + P::M_OFF, &T->tm_m, x0, y0, z, bar);
         };
         // Single-grid launch of an unmasked grid with a known parity: the
         // first piece from the schedule's shape and its first plane copies
@@ -1684,7 +1642,6 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
                         const bool halo = !PLANAR && ((off == 0) || (off == nl - 1));
                         mbar_expect_tx(bar, P::A_BYTES);
                         tma_load_3d(st + P::U_OFF, &T->tm_u[src], pc_early.x - 4, y0 - 1, z, bar);
-                        if (MASKED) tma_load_3d(st + P::M_OFF, &T->tm_m, pc_early.x - 16, y0 - 1, z, bar);
                         if (HB && !halo) {  // computed plane b = off - 1 (3D) or off (sheet): slot b
                             const int b = PLANAR ? off : off - 1;
                             mbar_expect_tx(fullb(b), b_bytes);
@@ -1792,7 +1749,6 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
                             // (an unmasked grid's plane outside the array: the copy fills zeros)
                             mbar_arrive_expect_tx(bar, P::A_BYTES);
                             tma_load_3d(st + P::U_OFF, &T->tm_u[src], pc.x - 4, y0 - 1, z, bar);
-                            if (MASKED) tma_load_3d(st + P::M_OFF, &T->tm_m, pc.x - 16, y0 - 1, z, bar);
                             if (HB && comp) {
                                 mbar_arrive_expect_tx(fullb(bs), b_bytes);
                                 load_b(T, src, pc.x, y0, z, bs, fullb(bs));
@@ -2010,10 +1966,7 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
                 const float* Fb = reinterpret_cast<const float*>(stb + P::F_OFF) + boff;  // [3][TY][TX]
                 const float* Db = reinterpret_cast<const float*>(stb + P::D_OFF) + boff;  // [3][TY][TX]
                 const float* Sv = reinterpret_cast<const float*>(stb + P::S_OFF) + boff;
-                const unsigned char* Mp = smem + ozm + P::M_OFF;
-                const unsigned char* Mc = smem + oc + P::M_OFF;
-                const unsigned char* Mn = smem + ozp + P::M_OFF;
-                const int m0 = (row0 + 1) * MW + (2 * tx + 16);  // mask index of node (x, yb)
+                const uint32_t* Mb = reinterpret_cast<const uint32_t*>(stb + P::M_OFF) + boff;
                 const bool zn_ok = k + 1 < nz, zp_ok = k > 0;
                 const int nrows = ny - yb;  // rows of this thread inside the array
                 const float ncz = MASKED || (zn_ok && zp_ok) ? -2.0f : (zn_ok || zp_ok ? -1.0f : 0.0f);
@@ -2045,36 +1998,71 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
                     const int w = r + 1;
                     const float2 u0 = wB[w];
                     bool live[2] = {x_in, x1_in};
+                    uint2 psi = make_uint2(0u, 0u);
+                    bool edge = false;  // a tissue node of the pair has a void neighbour
+                    if (MASKED) {
+                        psi = *reinterpret_cast<const uint2*>(Mb + r * TX);
+                        live[0] = (psi.x & PSI_TISSUE) != 0;
+                        live[1] = (psi.y & PSI_TISSUE) != 0;
+                        edge = (live[0] && !(psi.x & PSI_INTERIOR)) || (live[1] && !(psi.y & PSI_INTERIOR));
+                    }
                     float2 Lr;
                     const float ncy = MASKED ? -2.0f : ((r == 0 && yb == 0) || r + 1 == nrows
                                                             ? (r == 0 && yb == 0 && r + 1 == nrows ? 0.0f : -1.0f)
                                                             : -2.0f);
-                    const float2 sx = make_float2(__fadd_rn(u0.y, wA[w]), __fadd_rn(wC[w], u0.x));
+                    // a neighbour's value, u0 in place of a void one (every difference with it then vanishes)
+                    auto nb = [&](uint32_t bit, float a0, float a1) {
+                        return make_float2(psi.x & bit ? a0 : u0.x, psi.y & bit ? a1 : u0.y);
+                    };
+                    float2 sx = make_float2(__fadd_rn(u0.y, wA[w]), __fadd_rn(wC[w], u0.x));
+                    float2 sy = add2(wB[w + 1], wB[w - 1]), sz;
+                    if (!PLANAR) sz = add2(wN[w], wP[w]);
+                    if (MASKED && edge) {
+                        sx = add2(nb(PSI_XP, u0.y, wC[w]), nb(PSI_XM, wA[w], u0.x));
+                        sy = add2(nb(PSI_YP, wB[w + 1].x, wB[w + 1].y), nb(PSI_YM, wB[w - 1].x, wB[w - 1].y));
+                        if (!PLANAR) sz = add2(nb(PSI_ZP, wN[w].x, wN[w].y), nb(PSI_ZM, wP[w].x, wP[w].y));
+                    }
                     if (!ANISO) {
-                        float2 sum = add2(sx, add2(wB[w + 1], wB[w - 1]));
+                        float2 sum = add2(sx, sy);
                         float2 nc = add2(ncx, splat2(ncy));
                         if (!PLANAR) {
-                            sum = add2(sum, add2(wN[w], wP[w]));
+                            sum = add2(sum, sz);
                             nc = add2(nc, splat2(ncz));
                         }
                         Lr = mul2(splat2(co.c_iso), fma2(nc, u0, sum));
                     } else {
                         Diffs d;
                         d.xx = fma2(ncx, u0, sx);
-                        d.yy = fma2(splat2(ncy), u0, add2(wB[w + 1], wB[w - 1]));
+                        d.yy = fma2(splat2(ncy), u0, sy);
                         d.y1 = sub2(wB[w + 1], wB[w - 1]);
                         const float ya = __fsub_rn(wA[w + 1], wA[w - 1]), yc = __fsub_rn(wC[w + 1], wC[w - 1]);
                         d.xy = make_float2(__fsub_rn(d.y1.y, ya), __fsub_rn(yc, d.y1.x));
+                        float nA, nC, pA, pC;
                         if (!PLANAR) {
-                            d.zz = fma2(splat2(ncz), u0, add2(wN[w], wP[w]));
+                            nA = Un[w * UW - 1], nC = Un[w * UW + 2], pA = Up[w * UW - 1], pC = Up[w * UW + 2];
+                            d.zz = fma2(splat2(ncz), u0, sz);
                             d.z1 = sub2(wN[w], wP[w]);
-                            const float za = __fsub_rn(Un[w * UW - 1], Up[w * UW - 1]);
-                            const float zc = __fsub_rn(Un[w * UW + 2], Up[w * UW + 2]);
-                            d.xz = make_float2(__fsub_rn(d.z1.y, za), __fsub_rn(zc, d.z1.x));
+                            d.xz = make_float2(__fsub_rn(d.z1.y, __fsub_rn(nA, pA)), __fsub_rn(__fsub_rn(nC, pC), d.z1.x));
                             d.yz = sub2(sub2(wN[w + 1], wP[w + 1]), sub2(wN[w - 1], wP[w - 1]));
                         }
                         if (ANISO == AN_SUMS)
                             d.x1 = make_float2(__fsub_rn(u0.y, wA[w]), __fsub_rn(wC[w], u0.x));
+                        if (MASKED && edge) {
+                            d.xy = sub2(sub2(nb(PSI_XPYP, wB[w + 1].y, wC[w + 1]), nb(PSI_XPYM, wB[w - 1].y, wC[w - 1])),
+                                        sub2(nb(PSI_XMYP, wA[w + 1], wB[w + 1].x), nb(PSI_XMYM, wA[w - 1], wB[w - 1].x)));
+                            if (!PLANAR) {
+                                d.xz = sub2(sub2(nb(PSI_XPZP, wN[w].y, nC), nb(PSI_XPZM, wP[w].y, pC)),
+                                            sub2(nb(PSI_XMZP, nA, wN[w].x), nb(PSI_XMZM, pA, wP[w].x)));
+                                d.yz = sub2(sub2(nb(PSI_YPZP, wN[w + 1].x, wN[w + 1].y), nb(PSI_YPZM, wP[w + 1].x, wP[w + 1].y)),
+                                            sub2(nb(PSI_YMZP, wN[w - 1].x, wN[w - 1].y), nb(PSI_YMZM, wP[w - 1].x, wP[w - 1].y)));
+                            }
+                            // (a W-tilde sum is 0 where its axis misses a neighbour, whose value may be anything)
+                            if (ANISO == AN_SUMS) {
+                                d.x1 = sub2(nb(PSI_XP, u0.y, wC[w]), nb(PSI_XM, wA[w], u0.x));
+                                d.y1 = sub2(nb(PSI_YP, wB[w + 1].x, wB[w + 1].y), nb(PSI_YM, wB[w - 1].x, wB[w - 1].y));
+                                if (!PLANAR) d.z1 = sub2(nb(PSI_ZP, wN[w].x, wN[w].y), nb(PSI_ZM, wP[w].x, wP[w].y));
+                            }
+                        }
                         if (border) {
                             // psi = 0 on one side only leaves a cross difference short of u0 where both
                             // axes end (the array's edges)
@@ -2093,47 +2081,6 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
                             for (int c = 0; c < 3; ++c) sd[c] = ld2(Db, r * TX + c * CB);
                         }
                         Lr = lap_pair<ANISO, PLANAR>(co, d, f, sd);
-                    }
-                    if (MASKED) {
-                        const int m = m0 + r * MW;
-                        const unsigned char mc0 = Mc[m], mc1 = Mc[m + 1];
-                        live[0] = live[0] && (mc0 & MASK_TISSUE);
-                        live[1] = live[1] && (mc1 & MASK_TISSUE);
-                        const bool intr[2] = {(mc0 & MASK_INTERIOR) != 0, (mc1 & MASK_INTERIOR) != 0};
-                        // the general formula where any neighbour may be void
-                        if ((live[0] && !intr[0]) || (live[1] && !intr[1])) {
-#pragma unroll
-                            for (int e = 0; e < 2; ++e) {
-                                if (!live[e] || intr[e]) continue;
-                                const int me = m + e, ue = w * UW + e;
-                                Psi q;
-                                Nb n;
-                                n.u0 = Uc[ue];
-                                n.xp = Uc[ue + 1]; n.xm = Uc[ue - 1]; n.yp = Uc[ue + UW]; n.ym = Uc[ue - UW];
-                                n.zp = Un[ue]; n.zm = Up[ue];
-                                q.xp = Mc[me + 1] != 0; q.xm = Mc[me - 1] != 0;
-                                q.yp = Mc[me + MW] != 0; q.ym = Mc[me - MW] != 0;
-                                q.zp = zn_ok && Mn[me] != 0; q.zm = zp_ok && Mp[me] != 0;
-                                F3 f = {0.f, 0.f, 0.f}, sd = {0.f, 0.f, 0.f};
-                                if (ANISO) {
-                                    n.pp = Uc[ue + UW + 1]; n.mm = Uc[ue - UW - 1];
-                                    n.pm = Uc[ue - UW + 1]; n.mp = Uc[ue + UW - 1];
-                                    n.xpzp = Un[ue + 1]; n.xmzm = Up[ue - 1]; n.xpzm = Up[ue + 1]; n.xmzp = Un[ue - 1];
-                                    n.ypzp = Un[ue + UW]; n.ymzm = Up[ue - UW]; n.ypzm = Up[ue + UW]; n.ymzp = Un[ue - UW];
-                                    q.pp = Mc[me + MW + 1] != 0; q.mm = Mc[me - MW - 1] != 0;
-                                    q.pm = Mc[me - MW + 1] != 0; q.mp = Mc[me + MW - 1] != 0;
-                                    q.xpzp = zn_ok && Mn[me + 1] != 0; q.xmzm = zp_ok && Mp[me - 1] != 0;
-                                    q.xpzm = zp_ok && Mp[me + 1] != 0; q.xmzp = zn_ok && Mn[me - 1] != 0;
-                                    q.ypzp = zn_ok && Mn[me + MW] != 0; q.ymzm = zp_ok && Mp[me - MW] != 0;
-                                    q.ypzm = zp_ok && Mp[me + MW] != 0; q.ymzp = zn_ok && Mn[me - MW] != 0;
-                                    const int be = r * TX + e;
-                                    f = F3{Fb[be], Fb[be + CB], Fb[be + 2 * CB]};
-                                    if (ANISO == AN_SUMS) sd = F3{Db[be], Db[be + CB], Db[be + 2 * CB]};
-                                }
-                                const float Lg = lap_general<ANISO>(co, n, q, f, sd);
-                                if (e) Lr.y = Lg; else Lr.x = Lg;
-                            }
-                        }
                     }
 
                     // reaction, stores, activation, tissue sum (predicated)

@@ -281,6 +281,36 @@ __global__ void k_mask_interior(const uint8_t* __restrict__ in, uint8_t* __restr
     }
 }
 
+// The step's per-node words of a masked grid (PSI_*) from its mask bytes.
+__global__ void k_psi(const uint8_t* __restrict__ m, uint32_t* __restrict__ out, int nx, int ny, int nz, int px,
+                      long long plane) {
+    const long long n = (long long)nx * ny * nz;
+    constexpr int off[18][3] = {{1, 0, 0}, {-1, 0, 0}, {0, 1, 0}, {0, -1, 0}, {0, 0, 1}, {0, 0, -1},
+                                {1, 1, 0}, {-1, -1, 0}, {1, -1, 0}, {-1, 1, 0},
+                                {1, 0, 1}, {-1, 0, -1}, {1, 0, -1}, {-1, 0, 1},
+                                {0, 1, 1}, {0, -1, -1}, {0, 1, -1}, {0, -1, 1}};  // in the order of PSI_*
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+         i += (long long)gridDim.x * blockDim.x) {
+        const int x = int(i % nx);
+        const long long r = i / nx;
+        const int y = int(r % ny);
+        const int z = int(r / ny);
+        const long long gi = z * plane + (long long)y * px + x;
+        uint32_t w = 0;
+        if (m[gi] & MASK_TISSUE) {
+            w = PSI_TISSUE | (m[gi] & MASK_INTERIOR ? (uint32_t)PSI_INTERIOR : 0u);
+#pragma unroll
+            for (int b = 0; b < 18; ++b) {
+                const int X = x + off[b][0], Y = y + off[b][1], Z = z + off[b][2];
+                if (X >= 0 && Y >= 0 && Z >= 0 && X < nx && Y < ny && Z < nz &&
+                    (m[Z * plane + (long long)Y * px + X] & MASK_TISSUE))
+                    w |= 1u << b;
+            }
+        }
+        out[gi] = w;
+    }
+}
+
 // One block per brick: does the brick hold any tissue node?
 __global__ void k_brick_flags(const uint8_t* __restrict__ mask, int nx, int ny, int nz, int px, long long plane,
                               int ty, int zb, int nbx, int nby, uint8_t* flags) {
@@ -909,6 +939,7 @@ struct bbx_grid {
     int device = 0, num_sms = 0;
 
     uint8_t* d_mask = nullptr;
+    uint32_t* d_psi = nullptr;  // masked grids: the step's per-node words (PSI_*), laid out as the mask
     long long n_tissue = 0;
     float* d_fib = nullptr;  // [3][nz][ny][px] unit fibres
     float* d_div = nullptr;  // [3][nz][ny][px]: the fixed W-tilde sums of every node (k_divergence)
@@ -1211,9 +1242,8 @@ int encode_targs(const bbx_grid* g, int ty, TissueArgs* t) {
         t->tm_d = t->tm_u[0];
     }
     if (g->d_mask) {
-        const cuuint64_t mstr[2] = {(cuuint64_t)g->px, (cuuint64_t)g->plane};
-        const cuuint32_t mbox[3] = {(cuuint32_t)(kTileX + 32), (cuuint32_t)(ty + 2), 1};
-        if (!encode(&t->tm_m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, g->d_mask, dims3, mstr, mbox)) return BBX_ERR_CUDA;
+        const cuuint32_t mbox[3] = {(cuuint32_t)kTileX, (cuuint32_t)ty, 1};
+        if (!encode(&t->tm_m, CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, g->d_psi, dims3, str3, mbox)) return BBX_ERR_CUDA;
     } else {
         t->tm_m = t->tm_u[0];
     }
@@ -1496,6 +1526,7 @@ void bbx_destroy_grid(bbx_grid* g) {
     if (g->ev_halo) cudaEventDestroy(g->ev_halo);
     cudaFree(g->d_stage);
     cudaFree(g->d_mask);
+    cudaFree(g->d_psi);
     cudaFree(g->d_fib);
     cudaFree(g->d_div);
     if (!g->bound) {
@@ -1606,6 +1637,14 @@ int bbx_create_grid(bbx_grid** out, int nx, int ny, int nz, double h, const uint
             }
             k_mask_interior<<<n_blocks_for(ncell, 256), 256, 0, g->stream>>>(tmp, g->d_mask, nx, ny, nz, g->px,
                                                                              g->plane);
+            if (dmalloc(&g->d_psi, sizeof(uint32_t) * (size_t)g->vol) != cudaSuccess) {
+                cudaGetLastError();
+                cudaStreamSynchronize(g->stream);
+                cudaFree(tmp);
+                rc = BBX_ERR_NOMEM;
+                break;
+            }
+            k_psi<<<n_blocks_for(ncell, 256), 256, 0, g->stream>>>(g->d_mask, g->d_psi, nx, ny, nz, g->px, g->plane);
             const cudaError_t e1 = cudaGetLastError();
             const cudaError_t e2 = cudaStreamSynchronize(g->stream);
             cudaFree(tmp);
