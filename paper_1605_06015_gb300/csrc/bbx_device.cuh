@@ -1053,9 +1053,12 @@ struct Model<BBX_BR_FCA> {
 // ---------------------------------------------------------------------------
 
 constexpr int kTileX = 64;  // nodes per brick along x: 32 threads x 2 nodes
-// Several steps in one launch: unmasked grids of the light models (the
-// others' steps are long next to a launch, and the further warp it takes would
-// cost the registers their consumers need).
+// Several steps in one launch (FLOW variants): unmasked grids of the light
+// models (the others' steps are long next to a launch, and the further warp it
+// takes would cost the registers their consumers need).  The same grids in a
+// batch of several kernel types run the variants without the sync warp, one
+// launch a step: four CTAs per SM instead of three when isotropic (192 sheets
+// and 64 blocks 337 us a step against 365).
 __host__ __device__ constexpr bool has_flow(bool masked, int s) { return !masked && s <= 2; }
 // Consumer warps per CTA (plus the producer warp, plus the sync warp) for a
 // tile of TY rows: 7 warps of 1 or 2 rows each for TY = 7, 14; for 28 rows 7
@@ -1064,8 +1067,8 @@ __host__ __device__ constexpr bool has_flow(bool masked, int s) { return !masked
 // (8 warps and 16 rows with the sync warp, which load the four schedulers
 // evenly, were slower: 256x256x64 slab 24.9 -> 29.5 us, sheets 60 -> 73 us.)
 __host__ __device__ constexpr int rows_of_threads(int ty, bool flow) { return ty == 28 && !flow ? 14 : 7; }
-__host__ __device__ constexpr int step_threads(int ty, bool masked, int s) {
-    return 32 * rows_of_threads(ty, has_flow(masked, s)) + 32 + (has_flow(masked, s) ? 32 : 0);
+__host__ __device__ constexpr int step_threads(int ty, bool flow) {
+    return 32 * rows_of_threads(ty, flow) + 32 + (flow ? 32 : 0);
 }
 
 // Anisotropy of a step kernel variant: isotropic (c_iso only), anisotropic
@@ -1077,8 +1080,8 @@ enum : int { AN_ISO = 0, AN_SUMS = 1, AN_NO_SUMS = 2 };
 // two CTAs of 256 threads allow 128 registers a thread; the masked
 // anisotropic stencil with 2 rows a thread and the surrogate need more; the
 // unmasked isotropic variants fit in 64, so four CTAs hide more latency).
-__host__ __device__ constexpr int ctas_per_sm(bool masked, bool aniso, int ty, bool surr, int s) {
-    if (has_flow(masked, s)) return aniso ? (ty == 28 ? 1 : 2) : 3;
+__host__ __device__ constexpr int ctas_per_sm(bool masked, bool aniso, int ty, bool surr, bool flow) {
+    if (flow) return aniso ? (ty == 28 ? 1 : 2) : 3;
     return (masked && aniso && ty != 7) || ty == 28 || (surr && ty != 7) ? 1 : (!masked && !aniso && !surr ? 4 : 2);
 }
 constexpr int align128(int b) { return (b + 127) & ~127; }
@@ -1133,16 +1136,17 @@ __device__ __forceinline__ void st_global_u16(uint16_t* p, uint16_t v) {
     asm volatile("st.global.u16 [%0], %1;" ::"l"(p), "h"(v));
 }
 
-template <int MODEL, bool MASKED, int ANISO, int TY, bool SURR = false, int GATES = GATES_F32>
+template <int MODEL, bool MASKED, int ANISO, int TY, bool SURR = false, int GATES = GATES_F32,
+          bool FL = has_flow(MASKED, Model<MODEL>::S)>
 struct Plan {
     static constexpr int S = Model<MODEL>::S;
     static constexpr int NG = GATES ? 6 : 0;  // variables stored in 16 bits (the gates, last in the state)
     static constexpr int TX = kTileX;
-    static constexpr int RY = rows_of_threads(TY, has_flow(MASKED, S));
-    static constexpr int CTAS = ctas_per_sm(MASKED, ANISO != AN_ISO, TY, SURR, S);
+    static constexpr int RY = rows_of_threads(TY, FL);
+    static constexpr int CTAS = ctas_per_sm(MASKED, ANISO != AN_ISO, TY, SURR, FL);
     static constexpr int CY = TY / RY;  // nodes per thread along y (each a pair in x)
-    static constexpr bool FLOW = has_flow(MASKED, S);
-    static constexpr int THREADS = step_threads(TY, MASKED, S);  // consumer warps + producer warp (+ sync warp)
+    static constexpr bool FLOW = FL;
+    static constexpr int THREADS = step_threads(TY, FL);  // consumer warps + producer warp (+ sync warp)
     static constexpr int UW = TX + 8;   // x from x0-4 to x0+TX+3 (16-byte aligned start)
     static constexpr int UH = TY + 2;   // y from y0-1 to y0+TY
     // ring A, one stage per loaded plane (the computed planes and the z-halo
@@ -1499,10 +1503,10 @@ __device__ __forceinline__ int tile_row_of(int4 pc, int off) {
 // when all RY consumer warps are done with the plane.  No CTA-wide barrier is
 // taken per plane.
 template <int MODEL, bool MASKED, int ANISO, int TY, bool SURR = false, bool PLANAR = false, bool GEN = false,
-          int GATES = GATES_F32>
-__global__ void __launch_bounds__(step_threads(TY, MASKED, Model<MODEL>::S), ctas_per_sm(MASKED, ANISO != AN_ISO, TY, SURR, Model<MODEL>::S))
+          int GATES = GATES_F32, bool FL = has_flow(MASKED, Model<MODEL>::S)>
+__global__ void __launch_bounds__(step_threads(TY, FL), ctas_per_sm(MASKED, ANISO != AN_ISO, TY, SURR, FL))
 step_kernel(const __grid_constant__ LaunchArgs L) {
-    using P = Plan<MODEL, MASKED, ANISO, TY, SURR, GATES>;
+    using P = Plan<MODEL, MASKED, ANISO, TY, SURR, GATES, FL>;
     static_assert(GATES == GATES_F32 || (MODEL == BBX_BR && !SURR), "16-bit gates: Beeler-Reuter without surrogate");
     constexpr int NG = P::NG, S32 = P::S - NG;  // 16-bit variables last
     constexpr int S = P::S, TX = P::TX, UW = P::UW, CY = P::CY;
@@ -1949,7 +1953,7 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
             const int first = down ? a.z1 - 1 : a.z0, dir = down ? -1 : 1;
             int yb = (PLANAR ? first * TY : a.y0) + row0;  // y of this thread's first row
             int k = PLANAR ? 0 : first;
-            long long gi = (long long)k * a.plane + (long long)yb * px + x;  // node (x, yb) of plane k (even)
+            float* pd = a.dst + (long long)k * a.plane + (long long)yb * px + x;  // node (x, yb) of plane k (even)
             const long long gstep = (PLANAR ? (long long)TY * px : a.plane) * dir;
             float* const dst = a.dst;
             const long long vol = a.vol;
@@ -1972,7 +1976,10 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
                 const float ncz = MASKED || (zn_ok && zp_ok) ? -2.0f : (zn_ok || zp_ok ? -1.0f : 0.0f);
                 // unmasked: some cross difference misses a neighbour on one side only (a row or plane at
                 // the array's border)
-                const bool border = !MASKED && ANISO && (yb == 0 || nrows <= CY || (!PLANAR && !(zn_ok && zp_ok)));
+                // unmasked: this thread's rows touch the array's border in y
+                const bool yborder = !MASKED && (yb == 0 || nrows <= CY);
+                const float2 ncp = add2(ncx, splat2(-2.0f + (PLANAR ? 0.0f : ncz)));  // (isotropic: all axes)
+                const bool border = !MASKED && ANISO && (yborder || (!PLANAR && !(zn_ok && zp_ok)));
 
                 // Sliding window down the rows: plane k at x-1..x+2, the own pair of planes k+-1.
                 float2 wB[CY + 2], wN[CY + 2], wP[CY + 2];
@@ -2007,9 +2014,8 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
                         edge = (live[0] && !(psi.x & PSI_INTERIOR)) || (live[1] && !(psi.y & PSI_INTERIOR));
                     }
                     float2 Lr;
-                    const float ncy = MASKED ? -2.0f : ((r == 0 && yb == 0) || r + 1 == nrows
-                                                            ? (r == 0 && yb == 0 && r + 1 == nrows ? 0.0f : -1.0f)
-                                                            : -2.0f);
+                    float miss = 0.0f;  // y neighbours outside the array
+                    if (!MASKED && yborder) miss = (r == 0 && yb == 0 ? 1.0f : 0.0f) + (r + 1 == nrows ? 1.0f : 0.0f);
                     // a neighbour's value, u0 in place of a void one (every difference with it then vanishes)
                     auto nb = [&](uint32_t bit, float a0, float a1) {
                         return make_float2(psi.x & bit ? a0 : u0.x, psi.y & bit ? a1 : u0.y);
@@ -2024,16 +2030,14 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
                     }
                     if (!ANISO) {
                         float2 sum = add2(sx, sy);
-                        float2 nc = add2(ncx, splat2(ncy));
-                        if (!PLANAR) {
-                            sum = add2(sum, sz);
-                            nc = add2(nc, splat2(ncz));
-                        }
+                        if (!PLANAR) sum = add2(sum, sz);
+                        float2 nc = ncp;
+                        if (!MASKED && yborder) nc = add2(nc, splat2(miss));
                         Lr = mul2(splat2(co.c_iso), fma2(nc, u0, sum));
                     } else {
                         Diffs d;
                         d.xx = fma2(ncx, u0, sx);
-                        d.yy = fma2(splat2(ncy), u0, sy);
+                        d.yy = fma2(splat2(miss - 2.0f), u0, sy);
                         d.y1 = sub2(wB[w + 1], wB[w - 1]);
                         const float ya = __fsub_rn(wA[w + 1], wA[w - 1]), yc = __fsub_rn(wC[w + 1], wC[w - 1]);
                         d.xy = make_float2(__fsub_rn(d.y1.y, ya), __fsub_rn(yc, d.y1.x));
@@ -2084,7 +2088,7 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
                     }
 
                     // reaction, stores, activation, tissue sum (predicated)
-                    const long long gr = gi + (long long)r * px;
+                    float* const pr = pd + r * px;
                     float2 y[S];
                     y[0] = u0;
 #pragma unroll
@@ -2097,6 +2101,7 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
                     }
                     float2 Is = splat2(0.0f);
                     if (stim_on) {
+                        const long long gr = pr - dst;
                         if (live[0] && a.stim[gr]) Is.x = a.stim_amp;
                         if (live[1] && a.stim[gr + 1]) Is.y = a.stim_amp;
                     }
@@ -2108,7 +2113,7 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
                     }
                     react_pair<MODEL, SURR, GEN>(a, mp, dt, wbufs, live, y, Lr, Is);
                     if (live[0] && live[1]) {
-                        float* q = dst + gr;
+                        float* q = pr;
 #pragma unroll
                         for (int v = 0; v < S32; ++v) {
                             st_global(q, y[v]);
@@ -2116,22 +2121,23 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
                         }
 #pragma unroll
                         for (int v = S32; v < S; ++v)
-                            st_global_u32(a.dst16 + (long long)(v - S32) * a.vol + gr, gate_encode2<GATES>(y[v].x, y[v].y));
+                            st_global_u32(a.dst16 + (long long)(v - S32) * vol + (pr - dst), gate_encode2<GATES>(y[v].x, y[v].y));
                     } else if (live[0] || live[1]) {
 #pragma unroll
                         for (int e = 0; e < 2; ++e)
                             if (live[e]) {
 #pragma unroll
                                 for (int v = 0; v < S32; ++v)
-                                    st_global(a.dst + (long long)v * a.vol + gr + e, e ? y[v].y : y[v].x);
+                                    st_global(pr + (long long)v * vol + e, e ? y[v].y : y[v].x);
 #pragma unroll
                                 for (int v = S32; v < S; ++v)
-                                    st_global_u16(a.dst16 + (long long)(v - S32) * a.vol + gr + e,
+                                    st_global_u16(a.dst16 + (long long)(v - S32) * vol + (pr - dst) + e,
                                                   gate_encode<GATES>(e ? y[v].y : y[v].x));
                             }
                     }
                     const bool up0 = u0.x < theta && theta <= y[0].x, up1 = u0.y < theta && theta <= y[0].y;
                     if (up0 || up1) {
+                        const long long gr = pr - dst;
                         if (up0 && live[0] && a.act[gr] == BBX_ACT_NONE) a.act[gr] = a.step_next;
                         if (up1 && live[1] && a.act[gr + 1] == BBX_ACT_NONE) a.act[gr + 1] = a.step_next;
                     }
@@ -2157,7 +2163,7 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
                 oc = on;
                 if (PLANAR) yb += dir * TY;
                 else k += dir;
-                gi += gstep;
+                pd += gstep;
             }
             __syncwarp();
             if (!PLANAR && lane == 0) {  // release the piece's last two planes

@@ -15,11 +15,11 @@
 #include "bbx_mlp.cuh"
 
 namespace bbx {
-StepKernel step_kernel_fhn(bool masked, int aniso, int ty, bool planar, bool general);
-StepKernel step_kernel_barkley(bool masked, int aniso, int ty, bool planar, bool general);
+StepKernel step_kernel_fhn(bool masked, int aniso, int ty, bool planar, bool general, bool flow);
+StepKernel step_kernel_barkley(bool masked, int aniso, int ty, bool planar, bool general, bool flow);
 StepKernel step_kernel_br(bool masked, int aniso, int ty, bool planar, bool general);
-StepKernel step_kernel_zfk(bool masked, int aniso, int ty, bool planar, bool general);
-StepKernel step_kernel_diffusion(bool masked, int aniso, int ty, bool planar, bool general);
+StepKernel step_kernel_zfk(bool masked, int aniso, int ty, bool planar, bool general, bool flow);
+StepKernel step_kernel_diffusion(bool masked, int aniso, int ty, bool planar, bool general, bool flow);
 StepKernel step_kernel_br_mrl(bool masked, int aniso, int ty, bool planar, bool general);
 StepKernel step_kernel_br_fca(bool masked, int aniso, int ty, bool planar, bool general);
 cudaError_t mrl_build_table(float4* tab, double dt, cudaStream_t s);
@@ -111,7 +111,7 @@ void model_kernel_params(int model, const double* p, float* mp) {
 // aniso: AN_ISO, AN_SUMS or AN_NO_SUMS (the last only for the plain kernels of
 // unmasked grids; the 16-bit-gate and surrogate variants read the sums)
 StepKernel lookup_kernel(int model, bool masked, int aniso, int ty, bool surrogate, bool planar, bool general,
-                         int gates = GATES_F32) {
+                         int gates, bool flow) {
     if (gates != GATES_F32)  // 16-bit gates: Beeler-Reuter without surrogate
         return model == BBX_BR && !surrogate && aniso != AN_NO_SUMS
                    ? step_kernel_br16(masked, aniso != AN_ISO, ty, planar, general, gates)
@@ -121,11 +121,11 @@ StepKernel lookup_kernel(int model, bool masked, int aniso, int ty, bool surroga
                    ? step_kernel_br_surrogate(masked, aniso != AN_ISO, ty)
                    : StepKernel{nullptr, 0, 0, 0};
     switch (model) {
-        case BBX_FHN: return step_kernel_fhn(masked, aniso, ty, planar, general);
-        case BBX_BARKLEY: return step_kernel_barkley(masked, aniso, ty, planar, general);
+        case BBX_FHN: return step_kernel_fhn(masked, aniso, ty, planar, general, flow);
+        case BBX_BARKLEY: return step_kernel_barkley(masked, aniso, ty, planar, general, flow);
         case BBX_BR: return step_kernel_br(masked, aniso, ty, planar, general);
-        case BBX_ZFK: return step_kernel_zfk(masked, aniso, ty, planar, general);
-        case BBX_DIFFUSION: return step_kernel_diffusion(masked, aniso, ty, planar, general);
+        case BBX_ZFK: return step_kernel_zfk(masked, aniso, ty, planar, general, flow);
+        case BBX_DIFFUSION: return step_kernel_diffusion(masked, aniso, ty, planar, general, flow);
         case BBX_BR_MRL: return step_kernel_br_mrl(masked, aniso, ty, planar, general);
         case BBX_BR_FCA: return step_kernel_br_fca(masked, aniso, ty, planar, general);
     }
@@ -901,8 +901,8 @@ cudaError_t launch(const LaunchPlan& lp, const LaunchArgs& L, cudaStream_t s) {
 // Select the kernel for a configuration, check it fits, and return the CTA
 // budget (resident CTAs on the whole GPU).
 int select_kernel(int model, bool masked, int aniso, int ty, int device, int num_sms, StepKernel* out,
-                  int* ctas, bool surrogate, bool planar, bool general, int gates = GATES_F32) {
-    StepKernel k = lookup_kernel(model, masked, aniso, ty, surrogate, planar, general, gates);
+                  int* ctas, bool surrogate, bool planar, bool general, int gates = GATES_F32, bool flow = true) {
+    StepKernel k = lookup_kernel(model, masked, aniso, ty, surrogate, planar, general, gates, flow);
     if (!k.fn) return BBX_ERR_UNSUPPORTED;
     int smem_optin = 0;
     if (cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess) {
@@ -2732,16 +2732,15 @@ int batch_build(bbx_batch* b, const std::vector<int>* tys) {
         else if (gi < keep_ty.size()) gr.ty = keep_ty[gi];
     }
     // Several steps share a launch where the batch is one group of unmasked
-    // light grids.  Cooperative launches of several groups are not sure to
-    // run side by side (two of them enqueued behind other work ran one after
-    // the other: 256 tissues 456 us a step against 340 by graphs of single
-    // steps).
+    // light grids; several groups step side by side, one launch each a step
+    // (cooperative launches of several groups gained nothing: 343 to 366 us a
+    // step for 192 sheets and 64 blocks, against 337).
     b->flow = b->groups.size() == 1;
     std::vector<int> full(b->groups.size(), 0);
     for (size_t gi = 0; gi < b->groups.size(); ++gi) {
         auto& gr = b->groups[gi];
         int rc = select_kernel(gr.model, gr.masked, gr.aniso ? AN_SUMS : AN_ISO, gr.ty, b->device, b->num_sms, &gr.lp.k,
-                               &full[gi], gr.surr, gr.planar, gr.general);
+                               &full[gi], gr.surr, gr.planar, gr.general, GATES_F32, b->groups.size() == 1);
         if (rc) return rc;
         b->flow = b->flow && gr.lp.k.flow;
     }
