@@ -31,6 +31,8 @@ cudaError_t launch_ppm(const float* s0, const float* s1, const int* cur, const u
                        const float hi[3], uint8_t* out, int num_sms, cudaStream_t s);
 cudaError_t resident_sheet_steps(int model, const TissueArgs* d_t, int nx, int ny, int n_steps, int* d_err,
                                  cudaStream_t s, bool check_only, bool* ok);
+cudaError_t resident_pair_steps(int model, const TissueArgs* d_t, int nx, int ny, int n_steps, int* d_err,
+                                cudaStream_t s, bool check_only, bool* ok);
 cudaError_t launch_singz(const float* s0, const float* s1, const int* cur, long long off_a, long long off_b,
                          float iso_a, float iso_b, const uint8_t* mask, int nx, int ny, int nz, int px,
                          long long plane, float* xyz, int max_points, int* d_count, int num_sms, cudaStream_t s);
@@ -110,6 +112,7 @@ void model_kernel_params(int model, const double* p, float* mp) {
 // scheme or the RK4 solver (kernels for 7- and 14-row tiles).
 // aniso: AN_ISO, AN_SUMS or AN_NO_SUMS (the last only for the plain kernels of
 // unmasked grids; the 16-bit-gate and surrogate variants read the sums)
+// flow: the variant that may take several steps in one launch, where there is one
 StepKernel lookup_kernel(int model, bool masked, int aniso, int ty, bool surrogate, bool planar, bool general,
                          int gates, bool flow) {
     if (gates != GATES_F32)  // 16-bit gates: Beeler-Reuter without surrogate
@@ -999,6 +1002,7 @@ struct bbx_grid {
     int split = 0;  // time-stepping scheme (bbx_set_scheme)
     int rk4 = 0;    // kinetics solver (bbx_set_solver)
     int resident = 0;  // multi-step resident kernel requested (bbx_set_resident)
+    bool pairs_ok = false;  // the grid's shape runs in the register-resident kernel (looked up with the plan)
 
     // z-slab of a decomposed grid: the first halo_lo and last halo_hi planes
     // are halo planes (a neighbour slab's boundary V, read by the stencil,
@@ -1339,6 +1343,13 @@ int tab_refresh(bbx_grid* g) {
     return BBX_OK;
 }
 
+// The resident multi-step kernels serve small unmasked isotropic sheets of the
+// models given by a right-hand side, with the default scheme and solver.
+bool resident_shape(const bbx_grid* g) {
+    return g->nz == 1 && !g->d_mask && !g->aniso && !g->split && !g->rk4 && !g->surr_on &&
+           (g->model == BBX_FHN || g->model == BBX_BARKLEY || g->model == BBX_ZFK || g->model == BBX_DIFFUSION);
+}
+
 // Bring h_t, d_t and the single-grid launch plan in line with the settings.
 int prepare(bbx_grid* g) {
     g->ready = false;
@@ -1366,6 +1377,14 @@ int prepare(bbx_grid* g) {
     std::vector<Lattice> lattice;
     if (!g->d_mask) lattice.push_back(grid_lattice(g, k.ty));
     if ((rc = build_plan(&g->lp, segs, 1, ctas, lattice, g->device))) return rc;
+    g->pairs_ok = false;
+    if (resident_shape(g)) {
+        bool ok = false;
+        if (resident_pair_steps(g->model, nullptr, g->nx, g->ny, 0, nullptr, g->stream, true, &ok) != cudaSuccess)
+            cudaGetLastError();
+        else
+            g->pairs_ok = ok;
+    }
     BBX_CUDA(cudaStreamSynchronize(g->stream));
     g->ready = true;
     return BBX_OK;
@@ -1925,12 +1944,7 @@ int bbx_set_threshold(bbx_grid* g, double theta) {
     return g->model ? refresh_targs(g) : BBX_OK;
 }
 
-// The resident multi-step kernel serves small unmasked isotropic sheets of the
-// models given by a right-hand side, with the default scheme and solver.
-static bool resident_eligible(const bbx_grid* g) {
-    return g->nz == 1 && !g->d_mask && !g->aniso && !g->split && !g->rk4 && !g->surr_on && !g->poison &&
-           (g->model == BBX_FHN || g->model == BBX_BARKLEY || g->model == BBX_ZFK || g->model == BBX_DIFFUSION);
-}
+static bool resident_eligible(const bbx_grid* g) { return resident_shape(g) && !g->poison; }
 
 static int apply_kinetics_setting(bbx_grid* g);
 
@@ -2027,6 +2041,20 @@ int bbx_step(bbx_grid* g, double dt, int n_steps) {
         d.total = 0.0;
         d.total_pending = 0;
         if ((rc = write_dyn(g, d))) return rc;
+        g->stepped = true;
+        return BBX_OK;
+    }
+    if (n_steps >= 2 && g->pairs_ok && resident_eligible(g)) {
+        // a sheet that fits: all its steps in one cluster's registers and shared
+        // memory (200^2: 0.7 us a step against 4.7 by tiles), the same results
+        while (n_steps > 0) {
+            const int chunk = std::min(n_steps, 1 << 16);
+            bool ok = false;
+            BBX_CUDA(resident_pair_steps(g->model, g->d_t, g->nx, g->ny, chunk, g->d_err, g->stream, false, &ok));
+            if (!ok) return BBX_ERR_STATE;
+            n_steps -= chunk;
+            g->h_cur ^= chunk & 1;
+        }
         g->stepped = true;
         return BBX_OK;
     }
