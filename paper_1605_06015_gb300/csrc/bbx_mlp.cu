@@ -15,7 +15,7 @@ using namespace bbx;
 
 namespace {
 
-constexpr int kSB = 32;        // samples per training block (static shared memory < 48 KB)
+constexpr int kSB = 32;        // samples per training block
 constexpr int kThreads = 256;  // threads per training block
 
 __device__ __forceinline__ unsigned long long splitmix64(unsigned long long z) {
@@ -35,125 +35,207 @@ __device__ __forceinline__ long long sample_row(long long i, long long n, unsign
 
 // Forward and backward for kSB samples of the minibatch: per-block partial
 // gradients (float, [gridDim.x][kMlpParams]) and partial loss (double).
+//
+// Every product is a tile of outputs per thread with its operands read from
+// shared memory as float4: 32 multiply-adds for six 16-byte loads, where one
+// output at a time took two 4-byte loads a multiply-add, the weights' at a
+// stride of 64 floats (32 lanes on one bank).  Weight rows are padded to 68
+// (12) floats, so that eight lanes' float4 of eight rows touch every bank once.  Each
+// sum keeps its order (over inputs, outputs or samples ascending, from the
+// bias or 0), so results are bitwise those of one output at a time.
+// A step of 4096 samples: 84 us before.
+constexpr int kW1P = 12, kW2P = 68;  // padded row lengths
+constexpr int kSmW1 = 0, kSmW2 = kSmW1 + 64 * kW1P, kSmW3 = kSmW2 + 64 * kW2P, kSmB1 = kSmW3 + 8 * kW2P,
+              kSmB2 = kSmB1 + 64, kSmB3 = kSmB2 + 64, kSmX = kSmB3 + 8, kSmDy = kSmX + kSB * 8,
+              kSmH1 = kSmDy + kSB * 8, kSmH2 = kSmH1 + kSB * 64, kSmD2 = kSmH2 + kSB * 64,
+              kSmFloats = kSmD2 + kSB * 64;
+
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float dot4(float4 a, float4 b, float z) {  // in order x, y, z, w
+    return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, z))));
+}
+
+// Outputs of a layer with K inputs for rows j = jt + 16 i of the weights and
+// samples s = st + 16 e (i < 4, e < 2): relu(b + W in).
+template <int K, int WP>
+__device__ __forceinline__ void layer_tile(const float* W, const float* bias, const float* in, float* out, int jt, int st) {
+    float z[2][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) z[0][i] = z[1][i] = bias[jt + 16 * i];
+#pragma unroll 4
+    for (int k = 0; k < K; k += 4) {
+        const float4 a0 = ld4(in + st * K + k), a1 = ld4(in + (st + 16) * K + k);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float4 w = ld4(W + (jt + 16 * i) * WP + k);
+            z[0][i] = dot4(w, a0, z[0][i]);
+            z[1][i] = dot4(w, a1, z[1][i]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        out[st * 64 + jt + 16 * i] = fmaxf(z[0][i], 0.0f);
+        out[(st + 16) * 64 + jt + 16 * i] = fmaxf(z[1][i], 0.0f);
+    }
+}
+
 __global__ void __launch_bounds__(kThreads) k_mlp_fwd_bwd(const float* __restrict__ P, const float* __restrict__ X,
                                                            const float* __restrict__ T, long long n, int batch,
                                                            unsigned long long seed, unsigned long long step,
                                                            const float* __restrict__ norm, float* __restrict__ gpart,
                                                            double* __restrict__ lpart) {
-    __shared__ float W[kMlpParams];
-    __shared__ float xs[kSB][8], h1[kSB][64], h2[kSB][64], dy[kSB][8], d2[kSB][64];
+    extern __shared__ float4 sm4[];
+    float* sm = reinterpret_cast<float*>(sm4);
+    float *W1 = sm + kSmW1, *W2 = sm + kSmW2, *W3 = sm + kSmW3, *b1 = sm + kSmB1, *b2 = sm + kSmB2, *b3 = sm + kSmB3;
+    float *xs = sm + kSmX, *dy = sm + kSmDy, *h1 = sm + kSmH1, *h2 = sm + kSmH2, *d2 = sm + kSmD2;
     __shared__ double lsum[kThreads / 32];
+    static_assert(kSB == 32 && kThreads == 256, "thread tiles");
     const int tid = threadIdx.x;
-    for (int i = tid; i < kMlpParams; i += kThreads) W[i] = P[i];
-    const float* W1 = W + kOffW1;
-    const float* b1 = W + kOffB1;
-    const float* W2 = W + kOffW2;
-    const float* b2 = W + kOffB2;
-    const float* W3 = W + kOffW3;
-    const float* b3 = W + kOffB3;
+    const int jt = tid & 15, st = tid >> 4;
     const int s0 = blockIdx.x * kSB;
     const int ns = min(kSB, batch - s0);
-    // normalised inputs
-    for (int e = tid; e < kSB * 8; e += kThreads) {
-        const int s = e / 8, k = e % 8;
-        float v = 0.0f;
-        if (s < ns) {
-            const long long r = sample_row(s0 + s, n, seed, step);
-            v = (X[r * 8 + k] - norm[kNormMuIn + k]) / norm[kNormSdIn + k];
-        }
-        xs[s][k] = v;
+    // normalised inputs and targets: one value of each per thread (sample tid / 8, variable tid % 8)
+    const int ts = tid >> 3, tv = tid & 7;
+    float xv = 0.0f, tgt = 0.0f;
+    if (ts < ns) {
+        const long long r = sample_row(s0 + ts, n, seed, step);
+        xv = (X[r * 8 + tv] - norm[kNormMuIn + tv]) / norm[kNormSdIn + tv];
+        tgt = (T[r * 8 + tv] - norm[kNormMuOut + tv]) / norm[kNormSdOut + tv];
     }
+    for (int i = tid; i < 64 * 8; i += kThreads) W1[(i >> 3) * kW1P + (i & 7)] = P[kOffW1 + i];
+    for (int i = tid; i < 64 * 64; i += kThreads) W2[(i >> 6) * kW2P + (i & 63)] = P[kOffW2 + i];
+    for (int i = tid; i < 8 * 64; i += kThreads) W3[(i >> 6) * kW2P + (i & 63)] = P[kOffW3 + i];
+    if (tid < 64) {
+        b1[tid] = P[kOffB1 + tid];
+        b2[tid] = P[kOffB2 + tid];
+    }
+    if (tid < 8) b3[tid] = P[kOffB3 + tid];
+    xs[tid] = xv;
     __syncthreads();
-    for (int e = tid; e < kSB * 64; e += kThreads) {
-        const int s = e / 64, j = e % 64;
-        float z = b1[j];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) z = fmaf(W1[j * 8 + k], xs[s][k], z);
-        h1[s][j] = fmaxf(z, 0.0f);
-    }
+    layer_tile<8, kW1P>(W1, b1, xs, h1, jt, st);
     __syncthreads();
-    for (int e = tid; e < kSB * 64; e += kThreads) {
-        const int s = e / 64, j = e % 64;
-        float z = b2[j];
-#pragma unroll 16
-        for (int k = 0; k < 64; ++k) z = fmaf(W2[j * 64 + k], h1[s][k], z);
-        h2[s][j] = fmaxf(z, 0.0f);
-    }
+    layer_tile<64, kW2P>(W2, b2, h1, h2, jt, st);
     __syncthreads();
     // output, loss and dL/dy = 2 (y - t) / (batch * 8)
     double lacc = 0.0;
-    const float scale = 2.0f / (float)(batch * 8);
-    for (int e = tid; e < kSB * 8; e += kThreads) {
-        const int s = e / 8, o = e % 8;
+    {
         float g = 0.0f;
-        if (s < ns) {
-            float y = b3[o];
-#pragma unroll 16
-            for (int k = 0; k < 64; ++k) y = fmaf(W3[o * 64 + k], h2[s][k], y);
-            const long long r = sample_row(s0 + s, n, seed, step);
-            const float t = (T[r * 8 + o] - norm[kNormMuOut + o]) / norm[kNormSdOut + o];
-            const float d = y - t;
-            lacc += (double)d * (double)d;
-            g = scale * d;
+        if (ts < ns) {
+            float y = b3[tv];
+#pragma unroll 4
+            for (int k = 0; k < 64; k += 4) y = dot4(ld4(W3 + tv * kW2P + k), ld4(h2 + ts * 64 + k), y);
+            const float d = y - tgt;
+            lacc = (double)d * (double)d;
+            g = 2.0f / (float)(batch * 8) * d;
         }
-        dy[s][o] = g;
+        dy[tid] = g;
     }
     for (int off = 16; off > 0; off >>= 1) lacc += __shfl_xor_sync(0xffffffffu, lacc, off);
     if ((tid & 31) == 0) lsum[tid >> 5] = lacc;
     __syncthreads();
-    // dL/dz2 = (dy W3) * relu'(z2)
-    for (int e = tid; e < kSB * 64; e += kThreads) {
-        const int s = e / 64, k = e % 64;
-        float g = 0.0f;
+    // dL/dz2 = (dy W3) * relu'(z2): column k of samples s = tid / 64 + 4 i
+    const int kc = tid & 63, sq = tid >> 6;
+    {
+        float w[8];
 #pragma unroll
-        for (int o = 0; o < 8; ++o) g = fmaf(dy[s][o], W3[o * 64 + k], g);
-        d2[s][k] = h2[s][k] > 0.0f ? g : 0.0f;
+        for (int o = 0; o < 8; ++o) w[o] = W3[o * kW2P + kc];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int s = sq + 4 * i;
+            const float4 a = ld4(dy + s * 8), b = ld4(dy + s * 8 + 4);
+            float g = fmaf(a.x, w[0], 0.0f);
+            g = fmaf(a.y, w[1], g);
+            g = fmaf(a.z, w[2], g);
+            g = fmaf(a.w, w[3], g);
+            g = fmaf(b.x, w[4], g);
+            g = fmaf(b.y, w[5], g);
+            g = fmaf(b.z, w[6], g);
+            g = fmaf(b.w, w[7], g);
+            d2[s * 64 + kc] = h2[s * 64 + kc] > 0.0f ? g : 0.0f;
+        }
     }
     __syncthreads();
     float* gp = gpart + (size_t)blockIdx.x * kMlpParams;
-    // gradients of layer 3 and layer 2 (h2 no longer needed after dW3)
-    for (int e = tid; e < 8 * 64; e += kThreads) {
-        const int o = e / 64, k = e % 64;
-        float g = 0.0f;
-        for (int s = 0; s < kSB; ++s) g = fmaf(dy[s][o], h2[s][k], g);
-        gp[kOffW3 + e] = g;
+    // gradients of layer 3 (rows o = sq, sq + 4) and of the biases
+    {
+        float g0 = 0.0f, g1 = 0.0f;
+#pragma unroll 8
+        for (int s = 0; s < kSB; ++s) {
+            const float h = h2[s * 64 + kc];
+            g0 = fmaf(dy[s * 8 + sq], h, g0);
+            g1 = fmaf(dy[s * 8 + sq + 4], h, g1);
+        }
+        gp[kOffW3 + sq * 64 + kc] = g0;
+        gp[kOffW3 + (sq + 4) * 64 + kc] = g1;
     }
-    for (int o = tid; o < 8; o += kThreads) {
+    if (tid < 64) {
         float g = 0.0f;
-        for (int s = 0; s < kSB; ++s) g += dy[s][o];
-        gp[kOffB3 + o] = g;
+#pragma unroll 8
+        for (int s = 0; s < kSB; ++s) g += d2[s * 64 + tid];
+        gp[kOffB2 + tid] = g;
+    } else if (tid < 72) {
+        float g = 0.0f;
+        for (int s = 0; s < kSB; ++s) g += dy[s * 8 + tid - 64];
+        gp[kOffB3 + tid - 64] = g;
     }
-    for (int e = tid; e < 64 * 64; e += kThreads) {
-        const int j = e / 64, k = e % 64;
-        float g = 0.0f;
-        for (int s = 0; s < kSB; ++s) g = fmaf(d2[s][j], h1[s][k], g);
-        gp[kOffW2 + e] = g;
-    }
-    for (int j = tid; j < 64; j += kThreads) {
-        float g = 0.0f;
-        for (int s = 0; s < kSB; ++s) g += d2[s][j];
-        gp[kOffB2 + j] = g;
+    // gradients of layer 2: a 4 x 4 tile of (j, k) per thread
+    {
+        float g[4][4] = {};
+#pragma unroll 4
+        for (int s = 0; s < kSB; ++s) {
+            const float4 a = ld4(d2 + s * 64 + 4 * st), h = ld4(h1 + s * 64 + 4 * jt);
+            const float av[4] = {a.x, a.y, a.z, a.w}, hv[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) g[i][q] = fmaf(av[i], hv[q], g[i][q]);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) gp[kOffW2 + (4 * st + i) * 64 + 4 * jt + q] = g[i][q];
     }
     __syncthreads();
-    // dL/dz1 = (d2 W2) * relu'(z1), written over h2
-    for (int e = tid; e < kSB * 64; e += kThreads) {
-        const int s = e / 64, k = e % 64;
-        float g = 0.0f;
-#pragma unroll 16
-        for (int j = 0; j < 64; ++j) g = fmaf(d2[s][j], W2[j * 64 + k], g);
-        h2[s][k] = h1[s][k] > 0.0f ? g : 0.0f;
+    // dL/dz1 = (d2 W2) * relu'(z1), written over h2: columns 4 jt .. 4 jt + 3 of samples st, st + 16
+    {
+        float g[2][4] = {};
+#pragma unroll 4
+        for (int j = 0; j < 64; j += 4) {
+            const float4 a0 = ld4(d2 + st * 64 + j), a1 = ld4(d2 + (st + 16) * 64 + j);
+            const float av[2][4] = {{a0.x, a0.y, a0.z, a0.w}, {a1.x, a1.y, a1.z, a1.w}};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float4 w = ld4(W2 + (j + i) * kW2P + 4 * jt);
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    g[e][0] = fmaf(av[e][i], w.x, g[e][0]);
+                    g[e][1] = fmaf(av[e][i], w.y, g[e][1]);
+                    g[e][2] = fmaf(av[e][i], w.z, g[e][2]);
+                    g[e][3] = fmaf(av[e][i], w.w, g[e][3]);
+                }
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int i = (st + 16 * e) * 64 + 4 * jt + q;
+                h2[i] = h1[i] > 0.0f ? g[e][q] : 0.0f;
+            }
     }
     __syncthreads();
     for (int e = tid; e < 64 * 8; e += kThreads) {
         const int j = e / 8, k = e % 8;
         float g = 0.0f;
-        for (int s = 0; s < kSB; ++s) g = fmaf(h2[s][j], xs[s][k], g);
+#pragma unroll 8
+        for (int s = 0; s < kSB; ++s) g = fmaf(h2[s * 64 + j], xs[s * 8 + k], g);
         gp[kOffW1 + e] = g;
     }
-    for (int j = tid; j < 64; j += kThreads) {
+    if (tid < 64) {
         float g = 0.0f;
-        for (int s = 0; s < kSB; ++s) g += h2[s][j];
-        gp[kOffB1 + j] = g;
+#pragma unroll 8
+        for (int s = 0; s < kSB; ++s) g += h2[s * 64 + tid];
+        gp[kOffB1 + tid] = g;
     }
     if (tid == 0) {
         double l = 0.0;
@@ -162,33 +244,55 @@ __global__ void __launch_bounds__(kThreads) k_mlp_fwd_bwd(const float* __restric
     }
 }
 
-// Sum the per-block gradients in block order (double accumulation), write
-// the gradient, and (if lr > 0) apply one Adam step.  Block 0 also sums the
-// loss partials: loss = sum / (batch * 8).
-__global__ void k_mlp_reduce_adam(const float* __restrict__ gpart, int nblk, const double* __restrict__ lpart,
-                                  int batch, float* __restrict__ P, float* __restrict__ M, float* __restrict__ V,
-                                  float* __restrict__ G, double* __restrict__ loss, int step, float lr, float beta1,
-                                  float beta2, float eps) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < kMlpParams) {
-        double g = 0.0;
-        for (int b = 0; b < nblk; ++b) g += gpart[(size_t)b * kMlpParams + i];
-        G[i] = (float)g;
-        if (lr > 0.0f) {
-            const float gf = (float)g;
-            const float m = beta1 * M[i] + (1.0f - beta1) * gf;
-            const float v = beta2 * V[i] + (1.0f - beta2) * gf * gf;
-            M[i] = m;
-            V[i] = v;
-            const float mh = m / (1.0f - powf(beta1, (float)step));
-            const float vh = v / (1.0f - powf(beta2, (float)step));
-            P[i] = P[i] - lr * mh / (sqrtf(vh) + eps);
-        }
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+// Sum the per-block gradients in a fixed order (double accumulation: eight
+// segments of the blocks, each in block order, then the segments in order),
+// write the gradient, and (if lr > 0) apply one Adam step.  A block takes 32
+// parameters; one more block sums the loss partials: loss = sum / (batch * 8).
+// (One thread a parameter over all blocks' partials took 30 us for 128 of
+// them: a chain of loads on 21 SMs.)
+constexpr int kRedSeg = 8;
+__global__ void __launch_bounds__(32 * kRedSeg) k_mlp_reduce_adam(
+    const float* __restrict__ gpart, int nblk, const double* __restrict__ lpart, int batch, float* __restrict__ P,
+    float* __restrict__ M, float* __restrict__ V, float* __restrict__ G, double* __restrict__ loss, int step, float lr,
+    float beta1, float beta2, float eps) {
+    __shared__ double part[kRedSeg][32];
+    const int lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
+    if (blockIdx.x == gridDim.x - 1) {  // the loss
         double l = 0.0;
-        for (int b = 0; b < nblk; ++b) l += lpart[b];
-        *loss = l / ((double)batch * 8.0);
+        for (int b = threadIdx.x; b < nblk; b += 32 * kRedSeg) l += lpart[b];
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (lane == 0) part[seg][0] = l;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double s = 0.0;
+            for (int w = 0; w < kRedSeg; ++w) s += part[w][0];
+            *loss = s / ((double)batch * 8.0);
+        }
+        return;
+    }
+    const int i = blockIdx.x * 32 + lane;
+    const int per = (nblk + kRedSeg - 1) / kRedSeg, b0 = seg * per, b1 = min(nblk, b0 + per);
+    double g = 0.0;
+    if (i < kMlpParams) {
+#pragma unroll 8
+        for (int b = b0; b < b1; ++b) g += gpart[(size_t)b * kMlpParams + i];
+    }
+    part[seg][lane] = g;
+    __syncthreads();
+    if (seg != 0 || i >= kMlpParams) return;
+    g = 0.0;
+#pragma unroll
+    for (int w = 0; w < kRedSeg; ++w) g += part[w][lane];
+    G[i] = (float)g;
+    if (lr > 0.0f) {
+        const float gf = (float)g;
+        const float m = beta1 * M[i] + (1.0f - beta1) * gf;
+        const float v = beta2 * V[i] + (1.0f - beta2) * gf * gf;
+        M[i] = m;
+        V[i] = v;
+        const float mh = m / (1.0f - powf(beta1, (float)step));
+        const float vh = v / (1.0f - powf(beta2, (float)step));
+        P[i] = P[i] - lr * mh / (sqrtf(vh) + eps);
     }
 }
 
@@ -283,9 +387,9 @@ int run_batch(bbx_mlp* m, const float* X, const float* T, long long n, int batch
     int rc = ensure_blocks(m, nblk);
     if (rc) return rc;
     if (lr > 0.0f) ++m->step;
-    k_mlp_fwd_bwd<<<nblk, kThreads, 0, m->stream>>>(m->d_P, X, T, n, batch, seed, (unsigned long long)m->step,
+    k_mlp_fwd_bwd<<<nblk, kThreads, sizeof(float) * kSmFloats, m->stream>>>(m->d_P, X, T, n, batch, seed, (unsigned long long)m->step,
                                                     m->d_norm, m->d_gpart, m->d_lpart);
-    k_mlp_reduce_adam<<<(kMlpParams + 255) / 256, 256, 0, m->stream>>>(m->d_gpart, nblk, m->d_lpart, batch, m->d_P,
+    k_mlp_reduce_adam<<<(kMlpParams + 31) / 32 + 1, 32 * kRedSeg, 0, m->stream>>>(m->d_gpart, nblk, m->d_lpart, batch, m->d_P,
                                                                        m->d_M, m->d_V, m->d_G, m->d_loss, m->step,
                                                                        lr, 0.9f, 0.999f, 1e-8f);
     if (cudaGetLastError() != cudaSuccess) return BBX_ERR_CUDA;
@@ -310,7 +414,9 @@ int bbx_mlp_create(bbx_mlp** out, unsigned long long seed, void* cuda_stream) {
         cudaMalloc(&m->d_V, sizeof(float) * kMlpParams) != cudaSuccess ||
         cudaMalloc(&m->d_G, sizeof(float) * kMlpParams) != cudaSuccess ||
         cudaMalloc(&m->d_loss, sizeof(double)) != cudaSuccess ||
-        cudaMalloc(&m->d_norm, sizeof(float) * kNormSize) != cudaSuccess) {
+        cudaMalloc(&m->d_norm, sizeof(float) * kNormSize) != cudaSuccess ||
+        cudaFuncSetAttribute(k_mlp_fwd_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(float) * kSmFloats) !=
+            cudaSuccess) {
         cudaGetLastError();
         bbx_mlp_destroy(m);
         return BBX_ERR_NOMEM;
