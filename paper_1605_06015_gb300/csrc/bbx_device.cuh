@@ -4,15 +4,17 @@
 // The step kernel is one pass of the paper's unsplit scheme (section
 // "Computation of intermediate expressions": diff followed by euler /
 // rushlarsen) for every tissue node of a brick list:
-//   - 2.5D z-marching over bricks of 64 x TY x ZB nodes; each z-plane of V
-//     (with a one-node halo, widened in x to the 16-byte TMA rule), of the
-//     fibres (with halo), of the tissue mask (with halo) and of the
-//     non-diffusing variables is staged into shared memory by
-//     cp.async.bulk.tensor on an mbarrier ring of NS planes, loads running up
-//     to NS-3 planes ahead of the plane being computed;
-//   - the weights W = Wbar + Wtilde of Eq. (Lu) are rebuilt per node from the
-//     unit fibre vectors of the node and of its six face neighbours, Eq.
-//     (sigma); nothing per-weight is stored in HBM;
+//   - 2.5D z-marching over columns of 64 x TY nodes; a producer warp stages each
+//     z-plane of V (with a one-node halo, widened in x to the 16-byte TMA rule)
+//     in one ring of shared memory and each computed plane's own fibres, W-tilde
+//     sums, other variables and (masked grids) neighbour words in a second one,
+//     by cp.async.bulk.tensor on mbarriers, ahead of the consumer warps;
+//   - the operator of Eq. (Lu) is formed from differences of V, the node's unit
+//     fibre, Eq. (sigma), and the W-tilde sums, computed once per grid; its
+//     weights are not stored;
+//   - the arithmetic runs on pairs of x-adjacent nodes (packed FP32: one issue
+//     slot a pair), every operation with its rounding named, so that a node's
+//     result does not depend on the tile shape or the kernel variant;
 //   - the reaction update (Eq. (Euler) for V and non-gates, Eq. (RL) for
 //     gates) is fused, the new state is stored straight from registers;
 //   - the activation map is written on the first upward crossing only;
@@ -40,7 +42,7 @@ namespace bbx {
 
 enum : int { ERRBIT_TIMEOUT = 1, ERRBIT_NAN = 2, ERRBIT_HINT = 4 };
 
-// Device-updated state of one grid: written once per step, by the CTA that
+// Device-updated state of one grid: written once per launch, by the CTA that
 // takes the last start ticket (single-grid launch) or by the last CTA to
 // finish (batch launch), and by the on-demand sum of a pending total.
 struct TissueDyn {
@@ -76,7 +78,7 @@ struct TissueArgs {  // (CUtensorMap members impose its alignment)
     int wsum_zero;  // 1: every W-tilde sum of the grid is exactly 0 (a single-grid launch then skips their copies)
     // diffusion constants over h^2: anisotropic D = Dperp I + (Dpar-Dperp) f f^T
     // gives c_perp = Dperp/h^2, c_d = (Dpar-Dperp)/h^2, c_s = c_d/4 (Wtilde); isotropic D gives c_iso = D/h^2.
-    float c_perp, c_d, c_dh, c_s, c_iso;
+    float c_perp, c_d, c_s, c_iso;
     float mp[8];  // model parameters in kernel form
     const struct SurrogateData* surr;  // reaction surrogate (Beeler-Reuter), or nullptr
     const float4* tab;                 // V-table of the model (kTabN x 4 float4), or nullptr
@@ -138,7 +140,7 @@ struct LaunchArgs {
 };
 
 struct Coef {
-    float c_perp, c_d, c_dh, c_s, c_iso;
+    float c_perp, c_d, c_s, c_iso;
 };
 
 // ---------------------------------------------------------------------------
@@ -1079,7 +1081,8 @@ enum : int { AN_ISO = 0, AN_SUMS = 1, AN_NO_SUMS = 2 };
 // Resident CTAs per SM a kernel variant is built for (the register budget:
 // two CTAs of 256 threads allow 128 registers a thread; the masked
 // anisotropic stencil with 2 rows a thread and the surrogate need more; the
-// unmasked isotropic variants fit in 64, so four CTAs hide more latency).
+// unmasked isotropic variants fit in 64, so four CTAs hide more latency; with
+// a sync warp, 288 threads: 96 registers at two CTAs, 72 at three).
 __host__ __device__ constexpr int ctas_per_sm(bool masked, bool aniso, int ty, bool surr, bool flow) {
     if (flow) return aniso ? (ty == 28 ? 1 : 2) : 3;
     return (masked && aniso && ty != 7) || ty == 28 || (surr && ty != 7) ? 1 : (!masked && !aniso && !surr ? 4 : 2);
@@ -1486,7 +1489,8 @@ __device__ __forceinline__ int tile_row_of(int4 pc, int off) {
 }
 
 // Warp-specialised step kernel: warps 0..RY-1 compute (2 x CY nodes per
-// thread), warp RY is the producer.
+// thread), warp RY is the producer, warp RY + 1 (FL) tells the producer which
+// planes of the neighbouring columns have finished the step before.
 //
 // GEN: the variant that honours the per-grid scheme and solver settings (Lie
 // splitting, RK4 kinetics); the default variant (unsplit, Euler/Rush-Larsen)
@@ -1495,13 +1499,10 @@ __device__ __forceinline__ int tile_row_of(int4 pc, int off) {
 // PLANAR (grids with nz = 1): a piece is a run of tiles down one column of
 // the sheet, pieces[i] = (x0, -, first tile, end tile); each stage holds one
 // tile with its one-row halo and the consumers march along y.  The z
-// neighbours of a plane are the plane itself (the previous and next stage
-// pointers alias the current one): every z term of the stencil is then zero
-// (faces and edges exactly, the W-tilde divergence up to rounding), which is
-// the 5-point (isotropic) or 9-point (anisotropic) sheet operator.  Stage slots cycle through two mbarrier
-// rings: full[s] completes when the plane's bulk copies have landed, empty[s]
-// when all RY consumer warps are done with the plane.  No CTA-wide barrier is
-// taken per plane.
+// terms of the stencil are left out, which is the 5-point (isotropic) or
+// 9-point (anisotropic) sheet operator.  A stage's full barrier completes when
+// the plane's bulk copies have landed, its empty barrier when all RY consumer
+// warps are done with the plane.  No CTA-wide barrier is taken per plane.
 template <int MODEL, bool MASKED, int ANISO, int TY, bool SURR = false, bool PLANAR = false, bool GEN = false,
           int GATES = GATES_F32, bool FL = has_flow(MASKED, Model<MODEL>::S)>
 __global__ void __launch_bounds__(step_threads(TY, FL), ctas_per_sm(MASKED, ANISO != AN_ISO, TY, SURR, FL))
@@ -1511,7 +1512,7 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
     constexpr int NG = P::NG, S32 = P::S - NG;  // 16-bit variables last
     constexpr int S = P::S, TX = P::TX, UW = P::UW, CY = P::CY;
     constexpr int NS = P::NA;            // ring A: loaded planes
-    constexpr int NB = P::NB;            // ring B: computed planes (0: nothing beyond V and the mask)
+    constexpr int NB = P::NB;            // ring B: computed planes (0: nothing beyond V)
     constexpr bool HB = P::HAS_B;
     constexpr int NCW = P::RY;  // consumer warps
     constexpr int NCT = 32 * NCW;        // consumer threads
@@ -1733,7 +1734,7 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
                                 r.theta = T->theta;
                                 r.split = T->split;
                                 r.rk4 = T->rk4;
-                                r.c_perp = T->c_perp; r.c_d = T->c_d; r.c_dh = T->c_dh; r.c_s = T->c_s; r.c_iso = T->c_iso;
+                                r.c_perp = T->c_perp; r.c_d = T->c_d; r.c_s = T->c_s; r.c_iso = T->c_iso;
                                 r.surr = T->surr;
                                 r.tab = T->tab;
 #pragma unroll
@@ -1936,7 +1937,7 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
             lr = lr + 1 == NS ? 0 : lr + 1;
             const int ncomp = timed_out ? 0 : a.z1 - a.z0;  // (a context that never came is not read further)
             Coef co;
-            co.c_perp = a.c_perp; co.c_d = a.c_d; co.c_dh = a.c_dh; co.c_s = a.c_s; co.c_iso = a.c_iso;
+            co.c_perp = a.c_perp; co.c_d = a.c_d; co.c_s = a.c_s; co.c_iso = a.c_iso;
             float mp[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) mp[i] = a.mp[i];

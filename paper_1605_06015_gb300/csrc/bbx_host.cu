@@ -47,7 +47,7 @@ constexpr long long kPoisonWaitLimit = 2000000LL;     // about 1 ms
 constexpr int kMaxPartials = 152 * 32;
 constexpr int kErrFibre = 4;
 constexpr int kFlowSteps = 64;  // time steps of one launch at most
-constexpr int kChunkX = 16;  // x granularity of a masked grid's piece origins (the mask copy's 16-byte rule)
+constexpr int kChunkX = 16;  // x granularity of a masked grid's piece origins (every copy's 16-byte rule holds)
 
 int model_nvars(int model) {
     switch (model) {
@@ -858,6 +858,18 @@ LaunchArgs launch_args(const LaunchPlan& lp, const TissueArgs* d_tissues, int* d
     return L;
 }
 
+// Is the stream being captured into a graph?  A launch of several steps holds
+// the running step number in its parameters, which a replay would not advance:
+// captured steps are launched one by one.
+bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
 // Several steps of a plan in one cooperative launch (its CTAs wait for one
 // another between steps, plane by plane, so all of them must be resident).
 cudaError_t launch_flow(LaunchPlan* lp, LaunchArgs* L, int n_steps, cudaStream_t s) {
@@ -1275,7 +1287,6 @@ int encode_targs(const bbx_grid* g, int ty, TissueArgs* t) {
     const double cd = (g->Dpar - g->Dperp) * ih2;
     t->c_perp = (float)(g->Dperp * ih2);
     t->c_d = (float)cd;
-    t->c_dh = (float)(0.5 * cd);
     t->c_s = (float)(0.25 * cd);
     t->c_iso = (float)(g->Dpar * ih2);
     model_kernel_params(g->model, g->par, t->mp);
@@ -2046,7 +2057,8 @@ int bbx_step(bbx_grid* g, double dt, int n_steps) {
     }
     if (n_steps >= 2 && g->pairs_ok && resident_eligible(g)) {
         // a sheet that fits: all its steps in one cluster's registers and shared
-        // memory (200^2: 0.7 us a step against 4.7 by tiles), the same results
+        // memory (200^2, 20 steps a call: 1.8 us a step against 4.7 by tiles; 200
+        // steps: 1.1 us), the same results
         while (n_steps > 0) {
             const int chunk = std::min(n_steps, 1 << 16);
             bool ok = false;
@@ -2085,7 +2097,8 @@ int bbx_step(bbx_grid* g, double dt, int n_steps) {
         L.reg_ctas = g->lp.ctas;
         L.reg_planes = g->lp.n_planes;
     }
-    while (g->lp.flow && !g->poison && n_steps >= 2) {
+    const bool flow = n_steps >= 2 && g->lp.flow && !g->poison && !capturing(g->stream);
+    while (flow && g->lp.flow && n_steps >= 2) {
         const int m = std::min(n_steps, kFlowSteps);
         L.cur_hint = g->h_cur;
         if (launch_flow(&g->lp, &L, m, g->stream) != cudaSuccess) {
@@ -2947,19 +2960,20 @@ int bbx_batch_step(bbx_batch* b, int n_steps) {
     int rc;
     if (!b->built && (rc = batch_build(b, nullptr))) return rc;
     // without shared launches: graphs of up to 16 steps
+    const bool flow = b->flow && n_steps >= 2 && !capturing(b->stream);
     const int chunk = b->flow ? 1 : (n_steps < 16 ? n_steps : 16);
     if (chunk >= 2 && b->graph_steps != chunk && (rc = batch_capture(b, chunk))) return rc;
     // order the batch's stream after the members' stream, and back
     BBX_CUDA(cudaEventRecord(b->enter, b->stream));
     BBX_CUDA(cudaStreamWaitEvent(b->ps, b->enter, 0));
     int done = 0;
-    if (b->flow) {
+    if (flow) {
         while (n_steps - done >= 2) {
             const int m = std::min(n_steps - done, kFlowSteps);
             if ((rc = batch_launch_step(b, m))) return rc;
             done += m;
         }
-    } else if (n_steps >= 2) {
+    } else if (chunk >= 2) {
         for (; done + chunk <= n_steps; done += chunk) BBX_CUDA(cudaGraphLaunch(b->gexec, b->ps));
     }
     for (; done < n_steps; ++done)

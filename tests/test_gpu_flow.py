@@ -126,3 +126,26 @@ def test_batch_steps_of_one_launch_equal_single_steps_bitwise(bbx, n, planar):
         assert a.step_total() == b.step_total()
     A.close()
     B.close()
+
+
+@pytest.mark.parametrize("model,shape", [("barkley", (9, 30, 70)), ("fhn", (1, 64, 96)), ("fhn", (1, 900, 700))])
+def test_captured_steps_replay(bbx, model, shape):
+    """A call captured into a CUDA graph replays as the same call made again."""
+    torch = pytest.importorskip("torch")
+    mid = bbx.BBX_BARKLEY if model == "barkley" else bbx.BBX_FHN
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        A, dt = _grid(bbx, mid, shape, "none", 14)
+        A.step(dt, 4)
+        s.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            A.step(dt, 4)
+        for _ in range(3):
+            g.replay()
+        s.synchronize()
+    B, _ = _grid(bbx, mid, shape, "none", 14)
+    for _ in range(16):
+        B.step(dt, 1)
+    assert np.array_equal(A.read_all(), B.read_all())
+    assert A.get_time() == B.get_time()
