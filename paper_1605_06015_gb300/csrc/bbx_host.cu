@@ -150,11 +150,17 @@ bool get_encoder() {
     return g_encode != nullptr;
 }
 
+// Copies fetch whole 64-byte parts of a line into L2, not more: a box's rows
+// (256 bytes; V's 288 with the halo, from 16 bytes before) rarely start on the
+// 256-byte boundary that a larger promotion rounds them to, so it read up to
+// twice the bytes (256^3 Beeler-Reuter shell, whose pieces start at any 64
+// bytes: 128 us a step with 256 B, 122 with 128 B or none, 115.6 with 64 B;
+// 512x512x256 slab 337 -> 314, 8192^2 sheet 225 -> 194, small slabs the same).
 bool encode(CUtensorMap* m, CUtensorMapDataType dt, int rank, void* base, const cuuint64_t* dims,
             const cuuint64_t* strides, const cuuint32_t* box) {
     cuuint32_t es[4] = {1, 1, 1, 1};
     CUresult r = g_encode(m, dt, rank, base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                          CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                          CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_64B,
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
 }
