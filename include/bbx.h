@@ -220,15 +220,17 @@ int bbx_ppm_frame(bbx_grid* g, const int* layers, const double* lo, const double
 int bbx_phase_singularities(bbx_grid* g, int var_a, double iso_a, int var_b, double iso_b, float* xyz_dev,
                             int max_points, int* n_found);
 
-/* Resident multi-step mode for small sheets.  With on = 1, bbx_step calls of
- * two or more steps on this grid run as one launch of a cluster of 16 CTAs
- * (8 where the GPU offers no 16-CTA clusters) that keeps the whole sheet in
- * their shared memory (each CTA a band of
- * rows, the rows next to its band read from the neighbours' shared memory),
- * so a step costs neither a kernel launch nor a trip through DRAM.  Serves
- * unmasked isotropic sheets (nz = 1) of FHN, Barkley, ZFK or pure diffusion
- * with the unsplit scheme and Euler solver, up to about 200 KB of state per
- * CTA (for two variables, nx * ny up to ~260 000 with 16 CTAs).  Results agree with the
+/* Resident multi-step mode for small sheets.  A call of bbx_step with two or
+ * more steps on an unmasked isotropic sheet (nz = 1) of FHN, Barkley, ZFK or
+ * pure diffusion with the unsplit scheme and Euler solver that fits the
+ * registers and shared memory of one cluster of 16 CTAs runs all its
+ * steps there by itself, with the tiled kernel's results bitwise and without
+ * this switch.  With on = 1, larger sheets of that kind run in the shared
+ * memory of such a cluster (8 CTAs where the GPU offers no 16-CTA clusters),
+ * each CTA a band of rows, the rows next to its band read from the
+ * neighbours' shared memory, so a step costs neither a kernel launch nor a
+ * trip through DRAM: up to about 200 KB of state per CTA (for two variables,
+ * nx * ny up to ~260 000 with 16 CTAs).  The results of these agree with the
  * tiled kernel to rounding, not bitwise.  The fused total, time, step count
  * and activation map are kept as by the tiled kernel.  When the grid stops
  * qualifying (fibres, a mask, another scheme), steps go back to the tiled
@@ -285,9 +287,12 @@ int bbx_set_scheme(bbx_grid* g, int scheme);
 int bbx_set_solver(bbx_grid* g, int solver);
 
 /* Advance n_steps explicit steps of size dt (asynchronous on the grid's
- * stream).  Each step also reduces the new V over tissue nodes into one
- * double-precision partial per piece of its schedule (the total is summed
- * from them, in a fixed order, by bbx_step_total).  Errors: BBX_ERR_STATE (no
+ * stream).  Unmasked grids of at most two variables take up to 64 steps in one
+ * cooperative launch (one launch a step while the stream is being captured
+ * into a graph); results are bitwise those of calls with one step.  Each step
+ * also reduces the new V over tissue nodes into one double-precision partial
+ * per piece of its schedule (the total is summed from them, in a fixed order,
+ * by bbx_step_total).  Errors: BBX_ERR_STATE (no
  * model), BBX_ERR_ARG (dt <= 0, n_steps < 0), BBX_ERR_CUDA (launch),
  * BBX_ERR_UNSTABLE when dt (4 tr D + 2 |D_par - D_perp|) > 2 h^2, tr D =
  * D_par + 2 D_perp (3 D_par when isotropic): a Gershgorin bound on the
@@ -443,7 +448,8 @@ int bbx_halo_plane(bbx_grid* g, int side, int halo, void** dev_ptr, size_t* byte
  * advanced together.  Grids of one kernel type (model, masked, anisotropic)
  * share one persistent launch with a balanced schedule over all their
  * columns; the launches of the different types of a step run side by side,
- * each on a share of the GPU proportional to its work.  Steps are replayed
+ * each on a share of the GPU proportional to its work.  A batch of one type
+ * of unmasked light grids takes several steps a launch; others are replayed
  * from a CUDA graph captured on first use.  Not part of the paper: its
  * parameter studies ran one job per simulation. */
 typedef struct bbx_batch bbx_batch;

@@ -640,6 +640,63 @@ __device__ __forceinline__ int tab_index(float V, float* w) {
     return i;
 }
 
+// The interpolated table entry c at V.
+__device__ __forceinline__ void tab_entry(const float4* __restrict__ tab, float V, float* c) {
+    float w;
+    const int i = tab_index(V, &w);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const float4 a = __ldg(tab + 4 * i + q), b = __ldg(tab + 4 * i + 4 + q);
+        c[4 * q + 0] = fmaf(w, b.x - a.x, a.x);
+        c[4 * q + 1] = fmaf(w, b.y - a.y, a.y);
+        c[4 * q + 2] = fmaf(w, b.z - a.z, a.z);
+        c[4 * q + 3] = fmaf(w, b.w - a.w, a.w);
+    }
+}
+
+// The same for every lane's V, the 32 lanes of a warp together: four lanes
+// read one node's two entries as 2 x 64 consecutive bytes, interpolate four
+// coefficients each and hand them to the node's lane through shared memory
+// (buf: 32 nodes x 64 bytes, the 16-byte parts swapped so that eight lanes
+// touch every bank once).  What bounds a tabulated step is the wavefronts of
+// these loads: where V differs from node to node, a lane reading its own
+// node's entries takes eight loads of 32 separate lines, this eight loads of
+// eight 64-byte segments, and half as many wavefronts again for the exchange.
+// In waves (V different everywhere): 256x256x64 slab 113 -> 78 us a step, with
+// 16-bit gates 110 -> 75, 256^3 shell 129 -> 110, with 16-bit gates 129 -> 104.
+__device__ __forceinline__ void tab_entry_warp(const float4* __restrict__ tab, float V, float4* buf, float* c) {
+    const int lane = threadIdx.x & 31, p = lane & 3;
+    float w;
+    const int i = tab_index(V, &w);
+    float4 a[4], b[4];
+    float wn[4];
+#pragma unroll
+    for (int it = 0; it < 4; ++it) {
+        const int n = 8 * it + (lane >> 2);
+        const float4* e = tab + 4 * __shfl_sync(0xffffffffu, i, n) + p;
+        wn[it] = __shfl_sync(0xffffffffu, w, n);
+        a[it] = __ldg(e);
+        b[it] = __ldg(e + 4);
+    }
+    __syncwarp();  // the entries handed over before have been read
+#pragma unroll
+    for (int it = 0; it < 4; ++it) {
+        const int n = 8 * it + (lane >> 2);
+        buf[4 * n + (p ^ ((n >> 1) & 3))] =
+            make_float4(fmaf(wn[it], b[it].x - a[it].x, a[it].x), fmaf(wn[it], b[it].y - a[it].y, a[it].y),
+                        fmaf(wn[it], b[it].z - a[it].z, a[it].z), fmaf(wn[it], b[it].w - a[it].w, a[it].w));
+    }
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const float4 v = buf[4 * lane + (q ^ ((lane >> 1) & 3))];
+        c[4 * q + 0] = v.x;
+        c[4 * q + 1] = v.y;
+        c[4 * q + 2] = v.z;
+        c[4 * q + 3] = v.w;
+    }
+}
+
 template <>
 struct Model<BBX_BR> {
     static constexpr int S = 8;
@@ -818,21 +875,14 @@ struct Model<BBX_BR> {
     // rushlarsen device's tabulation, section "Exponential solvers"): per
     // entry A and B of Eq. (RL) for x1, m, h, j, d, f, then the V factors of
     // I_x1 (I_x1 = x1 K(V)) and I_K1, interpolated linearly; gates by
-    // y' = A y + B.  The table is built for the grid's dt.
-    __device__ static __forceinline__ void update_tab(const float* mp, const float4* __restrict__ tab, float* y,
-                                                      float L, float Is, float dt) {
+    // y' = A y + B.  The table is built for the grid's dt; entry(k, V, c): the
+    // interpolated entry c of the model's table k at V.
+    template <typename E>
+    __device__ static __forceinline__ void update_tab(const float* mp, E entry, float* y, float L, float Is,
+                                                      float dt) {
         const float V = y[0], Ca = y[1];
-        float w;
-        const int i = tab_index(V, &w);
         float c[16];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float4 a = __ldg(tab + 4 * i + q), b = __ldg(tab + 4 * i + 4 + q);
-            c[4 * q + 0] = fmaf(w, b.x - a.x, a.x);
-            c[4 * q + 1] = fmaf(w, b.y - a.y, a.y);
-            c[4 * q + 2] = fmaf(w, b.z - a.z, a.z);
-            c[4 * q + 3] = fmaf(w, b.w - a.w, a.w);
-        }
+        entry(0, V, c);
         const float m = y[3];
         const float INa = (mp[0] * m * m * m * y[4] * y[5] + mp[1]) * (V - mp[2]);
         const float Es = -82.3f - 13.0287f * __logf(Ca);
@@ -862,32 +912,20 @@ template <>
 struct Model<BBX_BR_MRL> {
     static constexpr int S = 11;
 
-    // tab: the Rush-Larsen table of Model<BBX_BR>::update_tab (kTabN x 4
-    // float4), followed by the chain's transition matrices (kTabN x 4 float4).
-    __device__ static __forceinline__ void update_tab(const float* mp, const float4* __restrict__ tab, float* y,
-                                                      float L, float Is, float dt) {
+    // Table 0: the Rush-Larsen table of Model<BBX_BR>::update_tab (kTabN x 4
+    // float4), followed by table 1, the chain's transition matrices (kTabN x 4
+    // float4).
+    template <typename E>
+    __device__ static __forceinline__ void update_tab(const float* mp, E entry, float* y, float L, float Is,
+                                                      float dt) {
         const float V = y[0], Ca = y[1];
-        float w;
-        const int i = tab_index(V, &w);
-        float c[16];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float4 a = __ldg(tab + 4 * i + q), b = __ldg(tab + 4 * i + 4 + q);
-            c[4 * q + 0] = fmaf(w, b.x - a.x, a.x);
-            c[4 * q + 1] = fmaf(w, b.y - a.y, a.y);
-            c[4 * q + 2] = fmaf(w, b.z - a.z, a.z);
-            c[4 * q + 3] = fmaf(w, b.w - a.w, a.w);
-        }
         // the chain, from V at the start of the step
-        const float4* t0 = tab + 4 * kTabN + 4 * i;
-        float pn[4];
+        float c[16], pn[4];
+        entry(1, V, c);
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const float4 a = __ldg(t0 + r), b = __ldg(t0 + 4 + r);
-            const float qa = fmaf(a.x, y[7], fmaf(a.y, y[8], fmaf(a.z, y[9], a.w * y[10])));
-            const float qb = fmaf(b.x, y[7], fmaf(b.y, y[8], fmaf(b.z, y[9], b.w * y[10])));
-            pn[r] = fmaf(w, qb - qa, qa);
-        }
+        for (int r = 0; r < 4; ++r)
+            pn[r] = fmaf(c[4 * r], y[7], fmaf(c[4 * r + 1], y[8], fmaf(c[4 * r + 2], y[9], c[4 * r + 3] * y[10])));
+        entry(0, V, c);
         // currents with P3 in place of m^3; x1, h, j, d, f by y' = A y + B
         const float INa = (mp[0] * y[10] * y[3] * y[4] + mp[1]) * (V - mp[2]);
         const float Es = -82.3f - 13.0287f * __logf(Ca);
@@ -998,22 +1036,14 @@ struct Model<BBX_BR_FCA> {
         }
     }
 
-    // tab: the Rush-Larsen table of Model<BBX_BR>::update_tab (kTabN x 4
+    // Table 0: the Rush-Larsen table of Model<BBX_BR>::update_tab (kTabN x 4
     // float4) with entry 14 = alpha_f(V) and entry 15 = 1 - e^{-dt/tau_c}.
-    __device__ static __forceinline__ void update_tab(const float* mp, const float4* __restrict__ tab, float* y,
-                                                      float L, float Is, float dt) {
+    template <typename E>
+    __device__ static __forceinline__ void update_tab(const float* mp, E entry, float* y, float L, float Is,
+                                                      float dt) {
         const float V = y[0], Ca = y[1];
-        float w;
-        const int i = tab_index(V, &w);
         float c[16];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float4 a = __ldg(tab + 4 * i + q), b = __ldg(tab + 4 * i + 4 + q);
-            c[4 * q + 0] = fmaf(w, b.x - a.x, a.x);
-            c[4 * q + 1] = fmaf(w, b.y - a.y, a.y);
-            c[4 * q + 2] = fmaf(w, b.z - a.z, a.z);
-            c[4 * q + 3] = fmaf(w, b.w - a.w, a.w);
-        }
+        entry(0, V, c);
         const float m = y[3];
         const float INa = (mp[0] * m * m * m * y[4] * y[5] + mp[1]) * (V - mp[2]);
         const float Es = -82.3f - 13.0287f * __logf(Ca);
@@ -1081,11 +1111,13 @@ enum : int { AN_ISO = 0, AN_SUMS = 1, AN_NO_SUMS = 2 };
 // Resident CTAs per SM a kernel variant is built for (the register budget:
 // two CTAs of 256 threads allow 128 registers a thread; the masked
 // anisotropic stencil with 2 rows a thread and the surrogate need more; the
-// unmasked isotropic variants fit in 64, so four CTAs hide more latency; with
+// unmasked isotropic variants of the light models fit in 64, so four CTAs hide
+// more latency (Beeler-Reuter spilled 216 bytes there: 83 us a step of a
+// 256x256x64 slab, 54 with two CTAs); with
 // a sync warp, 288 threads: 96 registers at two CTAs, 72 at three).
-__host__ __device__ constexpr int ctas_per_sm(bool masked, bool aniso, int ty, bool surr, bool flow) {
+__host__ __device__ constexpr int ctas_per_sm(bool masked, bool aniso, int ty, bool surr, bool flow, int s) {
     if (flow) return aniso ? (ty == 28 ? 1 : 2) : 3;
-    return (masked && aniso && ty != 7) || ty == 28 || (surr && ty != 7) ? 1 : (!masked && !aniso && !surr ? 4 : 2);
+    return (masked && aniso && ty != 7) || ty == 28 || (surr && ty != 7) ? 1 : (!masked && !aniso && s <= 2 ? 4 : 2);
 }
 constexpr int align128(int b) { return (b + 127) & ~127; }
 
@@ -1140,13 +1172,13 @@ __device__ __forceinline__ void st_global_u16(uint16_t* p, uint16_t v) {
 }
 
 template <int MODEL, bool MASKED, int ANISO, int TY, bool SURR = false, int GATES = GATES_F32,
-          bool FL = has_flow(MASKED, Model<MODEL>::S)>
+          bool FL = has_flow(MASKED, Model<MODEL>::S), bool GEN = false>
 struct Plan {
     static constexpr int S = Model<MODEL>::S;
     static constexpr int NG = GATES ? 6 : 0;  // variables stored in 16 bits (the gates, last in the state)
     static constexpr int TX = kTileX;
     static constexpr int RY = rows_of_threads(TY, FL);
-    static constexpr int CTAS = ctas_per_sm(MASKED, ANISO != AN_ISO, TY, SURR, FL);
+    static constexpr int CTAS = ctas_per_sm(MASKED, ANISO != AN_ISO, TY, SURR, FL, Model<MODEL>::S);
     static constexpr int CY = TY / RY;  // nodes per thread along y (each a pair in x)
     static constexpr bool FLOW = FL;
     static constexpr int THREADS = step_threads(TY, FL);  // consumer warps + producer warp (+ sync warp)
@@ -1178,12 +1210,27 @@ struct Plan {
     static constexpr int B_STAGE = B_BAR + 128;
     static constexpr uint32_t B_BYTES = F_RAW + D_RAW + S_RAW + M_RAW;
     static constexpr bool HAS_B = B_BYTES > 0;
-    static constexpr int BUDGET = (CTAS == 1 ? 200 : (CTAS == 2 ? 112 : (CTAS == 3 ? 72 : 54))) * 1024;  // dynamic shared memory per CTA
+    static constexpr int ROOM = (CTAS == 1 ? 200 : (CTAS == 2 ? 112 : (CTAS == 3 ? 72 : 54))) * 1024;  // dynamic shared memory per CTA
+    // A kernel that gathers from a V-table (TAB) takes at most three stages of
+    // ring B and leaves the rest to the L1 cache (Markov model, 181x428x43
+    // slab: 204 us a step with four, 155 with three); its warps gather
+    // together (tab_entry_warp) where their buffers cost none of these stages
+    // (256^3 tabulated shell: 110 us, 132 with two, 129 without the buffers
+    // and four).
+    static constexpr bool TAB = MODEL == BBX_BR_MRL || MODEL == BBX_BR_FCA || (MODEL == BBX_BR && GEN && !SURR);
+    static constexpr int NB_TAB = ROOM >= 3 * B_STAGE + 5 * A_STAGE ? 3 : 2;
+    static constexpr int TABW_BYTES = RY * 2048 + 2048;  // (2 KB: barriers and piece contexts)
+    static constexpr bool TABW = TAB && TABW_BYTES + NB_TAB * B_STAGE + 4 * A_STAGE <= ROOM;
+    // per consumer warp: the surrogate's 64 rows of 32 bytes, or 32 table entries of 64 bytes
+    static constexpr int WBUF = SURR || TABW ? RY * 2048 : 0;
+    static constexpr int BUDGET = ROOM - (TABW ? TABW_BYTES : 0);
     static constexpr int NB_FIT = HAS_B ? (BUDGET - 5 * A_STAGE) / B_STAGE : 0;
-    static constexpr int NB = !HAS_B ? 0 : (NB_FIT > 5 ? 5 : (NB_FIT < 2 ? 2 : NB_FIT));
-    static constexpr int NA_FIT = (BUDGET - NB * B_STAGE) / A_STAGE;
+    static constexpr int NB_MAX = TAB ? NB_TAB : 5;
+    static constexpr int NB = !HAS_B ? 0 : (TABW ? NB_TAB : (NB_FIT > NB_MAX ? NB_MAX : (NB_FIT < 2 ? 2 : NB_FIT)));
+    // (two CTAs: 228 KB an SM, 1 KB of it per CTA the system's)
+    static constexpr int NA_TWO = CTAS == 2 ? (114 * 1024 - 1024 - 128 - WBUF - NB * B_STAGE) / (A_STAGE + 176) : 8;
+    static constexpr int NA_ROOM = (BUDGET - NB * B_STAGE) / A_STAGE, NA_FIT = NA_ROOM < NA_TWO ? NA_ROOM : NA_TWO;
     static constexpr int NA = NA_FIT > 8 ? 8 : (NA_FIT < 4 ? 4 : NA_FIT);
-    static constexpr int WBUF = SURR ? RY * 2048 : 0;  // per consumer warp: 64 rows of 32 bytes
     static constexpr int RING_OFF = NA * A_STAGE + NB * B_STAGE + WBUF;
     // stages with their barriers, warp buffers, piece contexts
     static constexpr int SMEM = 128 + RING_OFF + NA * 176;
@@ -1385,7 +1432,7 @@ static_assert(sizeof(PieceSlot) <= 176, "piece ring slot size");
 // The kinetics step of a pair of nodes: y the state at the start of the step
 // (the half-step voltage under Lie splitting), L the diffusion term (0 then),
 // Is the stimulus.  All 32 lanes of a warp call it.
-template <int MODEL, bool SURR, bool GEN>
+template <int MODEL, bool SURR, bool GEN, bool TABW>
 __device__ __forceinline__ void react_pair(const PieceSlot& a, const float* mp, float dt, unsigned char* wbufs,
                                            const bool* live, float2* y, float2 L, float2 Is) {
     constexpr int S = Model<MODEL>::S;
@@ -1435,8 +1482,15 @@ __device__ __forceinline__ void react_pair(const PieceSlot& a, const float* mp, 
                 ys[0][v] = y[v].x;
                 ys[1][v] = y[v].y;
             }
-            Model<MODEL>::update_tab(mp, a.tab, ys[0], L.x, Is.x, dt);
-            Model<MODEL>::update_tab(mp, a.tab, ys[1], L.y, Is.y, dt);
+            auto entry = [&](int k, float V, float* c) {
+                const float4* t = a.tab + 4 * kTabN * k;
+                if constexpr (TABW)
+                    tab_entry_warp(t, V, reinterpret_cast<float4*>(wbufs + (threadIdx.x >> 5) * 2048), c);
+                else
+                    tab_entry(t, V, c);
+            };
+            Model<MODEL>::update_tab(mp, entry, ys[0], L.x, Is.x, dt);
+            Model<MODEL>::update_tab(mp, entry, ys[1], L.y, Is.y, dt);
 #pragma unroll
             for (int v = 0; v < S; ++v) y[v] = make_float2(ys[0][v], ys[1][v]);
         } else if constexpr (MODEL == BBX_BR) {
@@ -1505,9 +1559,9 @@ __device__ __forceinline__ int tile_row_of(int4 pc, int off) {
 // warps are done with the plane.  No CTA-wide barrier is taken per plane.
 template <int MODEL, bool MASKED, int ANISO, int TY, bool SURR = false, bool PLANAR = false, bool GEN = false,
           int GATES = GATES_F32, bool FL = has_flow(MASKED, Model<MODEL>::S)>
-__global__ void __launch_bounds__(step_threads(TY, FL), ctas_per_sm(MASKED, ANISO != AN_ISO, TY, SURR, FL))
+__global__ void __launch_bounds__(step_threads(TY, FL), ctas_per_sm(MASKED, ANISO != AN_ISO, TY, SURR, FL, Model<MODEL>::S))
 step_kernel(const __grid_constant__ LaunchArgs L) {
-    using P = Plan<MODEL, MASKED, ANISO, TY, SURR, GATES, FL>;
+    using P = Plan<MODEL, MASKED, ANISO, TY, SURR, GATES, FL, GEN>;
     static_assert(GATES == GATES_F32 || (MODEL == BBX_BR && !SURR), "16-bit gates: Beeler-Reuter without surrogate");
     constexpr int NG = P::NG, S32 = P::S - NG;  // 16-bit variables last
     constexpr int S = P::S, TX = P::TX, UW = P::UW, CY = P::CY;
@@ -2112,7 +2166,7 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
                         y[0] = fma2(splat2(dt), Lr, y[0]);
                         Lr = splat2(0.0f);
                     }
-                    react_pair<MODEL, SURR, GEN>(a, mp, dt, wbufs, live, y, Lr, Is);
+                    react_pair<MODEL, SURR, GEN, P::TABW>(a, mp, dt, wbufs, live, y, Lr, Is);
                     if (live[0] && live[1]) {
                         float* q = pr;
 #pragma unroll

@@ -5,7 +5,7 @@ namespace bbx {
 
 template <bool MA, int AN, int TY, bool SU = false, bool PL = false, bool GE = false>
 static StepKernel make_br() {
-    using P = Plan<BBX_BR, MA, AN, TY, SU>;
+    using P = Plan<BBX_BR, MA, AN, TY, SU, GATES_F32, false, GE>;
     return StepKernel{reinterpret_cast<const void*>(&step_kernel<BBX_BR, MA, AN, TY, SU, PL, GE>), P::SMEM,
                       P::THREADS, TY, P::FLOW};
 }
