@@ -1221,6 +1221,11 @@ void grid_segments(const bbx_grid* g, int rows, int tissue, std::vector<Seg>* se
     }
 }
 
+// Does the grid's step gather from a V-table?
+bool reads_table(const bbx_grid* g) {
+    return g->model == BBX_BR_MRL || g->model == BBX_BR_FCA || (g->model == BBX_BR && g->tab_on);
+}
+
 // The kernel's view of a grid for tile rows `ty` (tensor maps depend on it).
 int encode_targs(const bbx_grid* g, int ty, TissueArgs* t) {
     if (!get_encoder()) return BBX_ERR_CUDA;
@@ -1297,8 +1302,7 @@ int encode_targs(const bbx_grid* g, int ty, TissueArgs* t) {
     t->c_iso = (float)(g->Dpar * ih2);
     model_kernel_params(g->model, g->par, t->mp);
     t->surr = (g->surr_on && g->model == BBX_BR) ? g->d_surr : nullptr;
-    t->tab = (g->model == BBX_BR_MRL || g->model == BBX_BR_FCA || (g->model == BBX_BR && g->tab_on)) ? g->d_tab
-                                                                                                    : nullptr;
+    t->tab = reads_table(g) ? g->d_tab : nullptr;
     return BBX_OK;
 }
 
@@ -1341,7 +1345,7 @@ void exchange_release(bbx_grid* g) {
 }
 
 int tab_refresh(bbx_grid* g) {
-    const bool want = g->model == BBX_BR_MRL || g->model == BBX_BR_FCA || (g->model == BBX_BR && g->tab_on);
+    const bool want = reads_table(g);
     if (!want) return BBX_OK;
     if (!g->d_tab) {  // room for both tables of BBX_BR_MRL
         if (dmalloc(&g->d_tab, sizeof(float4) * 8 * (size_t)kTabN) != cudaSuccess) {
@@ -2606,6 +2610,11 @@ int bbx_autotune(bbx_grid* g, double dt, double* best_ms) {
         // 400 against 345); on tissue at rest, which a grid often holds when it
         // is tuned, the difference can vanish in the memory's own scatter
         if (ty == 28 && !g->d_mask && g->aniso && g->S <= 2) continue;
+        // tables: 7 rows, whose warps gather entries together; 14 rows are faster
+        // only on tissue at rest, where every lane reads the same entry (in
+        // waves: 256x256x64 slab 140 us a step against 79, Markov model
+        // 181x428x43 188 against 128, 256^3 shell 144 against 104)
+        if (ty != 7 && reads_table(g)) continue;
         for (int zb : zbs) {
             if ((rc = bbx_set_tiling(g, ty, zb)) != BBX_OK) {
                 if (rc == BBX_ERR_UNSUPPORTED) {
