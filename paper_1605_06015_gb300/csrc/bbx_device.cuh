@@ -664,10 +664,16 @@ __device__ __forceinline__ void tab_entry(const float4* __restrict__ tab, float 
 // eight 64-byte segments, and half as many wavefronts again for the exchange.
 // In waves (V different everywhere): 256x256x64 slab 113 -> 78 us a step, with
 // 16-bit gates 110 -> 75, 256^3 shell 129 -> 110, with 16-bit gates 129 -> 104.
+// Where the warp's V lie within a few entries (tissue near rest) each lane
+// reads its own: its loads are then a line or two for the whole warp.
 __device__ __forceinline__ void tab_entry_warp(const float4* __restrict__ tab, float V, float4* buf, float* c) {
     const int lane = threadIdx.x & 31, p = lane & 3;
     float w;
     const int i = tab_index(V, &w);
+    if (__reduce_max_sync(0xffffffffu, i) - __reduce_min_sync(0xffffffffu, i) <= 3) {
+        tab_entry(tab, V, c);
+        return;
+    }
     float4 a[4], b[4];
     float wn[4];
 #pragma unroll
