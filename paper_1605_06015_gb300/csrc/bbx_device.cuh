@@ -2234,7 +2234,14 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
             if (!last_step) continue;
             // per-piece partial of the tissue sum, and a vote on timeouts
             const int pi = down ? piece_end - 1 - (pw - (n_walk - n_pieces)) : piece_begin + (pw - (n_walk - n_pieces));
-            double v = (x_in ? (double)vhi.x + (double)vlo.x : 0.0) + (x1_in ? (double)vhi.y + (double)vlo.y : 0.0);
+            // The two columns are joined in FP32, by TwoSum, before FP64: the FP64 pipe takes an SM's warps one
+            // after the other (a warp's instruction some 16 cycles), and joined in FP64, with four more
+            // instructions a warp, a one-step launch took 0.3 us longer with one CTA on an SM, 1 us with four
+            // (FHN sheets in 7-row tiles: 64x64 5.7 -> 6.0 us, 400x400 7.6 -> 8.7 us; as here 5.7 and 7.6).
+            F2 vs = {x_in ? vhi.x : 0.0f, x_in ? vlo.x : 0.0f};
+            two_sum_add(vs, x1_in ? vhi.y : 0.0f);
+            vs.lo += x1_in ? vlo.y : 0.0f;
+            double v = (double)vs.hi + (double)vs.lo;
             for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
             if (lane == 0) red_scratch[warp] = v;
             const bool any_to = consumers_sync_or(timed_out, NCT);
