@@ -1656,7 +1656,10 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
         int lp = 0;
         // the loads the first plane waits for, issued together: the first
         // piece (its slot always exists) and, for one grid, its t, n, parity
-        int4 pc_next = L.pieces[n_pieces > 0 ? piece_slot(0) : piece_begin];
+        // (a share walked upwards starts with its first slot, whose load need not wait for the count)
+        int4 pc_next;
+        if (down && n_pieces > 0) pc_next = L.pieces[piece_slot(0)];
+        else pc_next = L.pieces[piece_begin];
         TissueDyn d0 = {};
         bool ticketed = !L.single;  // a single-grid launch takes one start ticket per CTA
         if (L.single) {
