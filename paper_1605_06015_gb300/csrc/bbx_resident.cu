@@ -197,6 +197,28 @@ __device__ __forceinline__ bool try_wait_cluster(uint32_t bar, uint32_t parity) 
     return ok != 0;
 }
 
+// A sum of floats kept in three (TwoSum of the value into hi, of its rounding
+// error into lo, of that one's into lo2: about 70 bits).  The FP64 pipe takes
+// an SM's warps one after the other, a warp's instruction some 16 cycles; seven
+// of them a node and six a warp bounded short calls: 2 steps on a 200x200
+// sheet 16.6 us a call, 10.4 so, on 400x400 41.2 and 19.8.
+struct F3 {
+    float hi, lo, lo2;
+};
+__device__ __forceinline__ float res_two_sum_f(float a, float b, float* err) {
+    const float s = a + b, bb = s - a;
+    *err = (a - (s - bb)) + (b - bb);
+    return s;
+}
+__device__ __forceinline__ void f3_add(F3& a, F3 b) {
+    float e, f, g;
+    a.hi = res_two_sum_f(a.hi, b.hi, &e);
+    const float t = res_two_sum_f(a.lo, b.lo, &f);
+    a.lo = res_two_sum_f(t, e, &g);
+    a.lo2 += b.lo2 + (f + g);
+}
+__device__ __forceinline__ void f3_add(F3& a, float b) { f3_add(a, F3{b, 0.0f, 0.0f}); }
+
 // Warps of a CTA with np pairs of columns whose threads own row r of the band.
 __host__ __device__ __forceinline__ int row_warp0(int np, int R, int r) { return (r / R * np) / 32; }
 __host__ __device__ __forceinline__ int row_warps(int np, int R, int r) {
@@ -216,7 +238,7 @@ __global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(kResThreads, 1)
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
     extern __shared__ float sm[];
-    __shared__ double red_hi[kResThreads / 32];
+    __shared__ float red[3][kResThreads / 32];
     __shared__ double cl_part[NC];
     __shared__ alignas(8) uint64_t bar[2];
 
@@ -366,16 +388,16 @@ __global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(kResThreads, 1)
     // the new state into the buffer that becomes current, and the FP64 total of V
     const int cur1 = cur0 ^ (n_steps & 1);
     float* dst = T->state[cur1];
-    double hi = 0.0, lo = 0.0;
+    F3 sum = {0.0f, 0.0f, 0.0f};
 #pragma unroll
     for (int k = 0; k < R; ++k) {
         if (k >= rows) continue;
         const long long gi = (long long)(rb0 + r0 + k) * px + x;
         dst[gi] = u[k].x;
-        res_two_sum(hi, lo, (double)u[k].x);
+        f3_add(sum, u[k].x);
         if (x1_in) {
             dst[gi + 1] = u[k].y;
-            res_two_sum(hi, lo, (double)u[k].y);
+            f3_add(sum, u[k].y);
         }
 #pragma unroll
         for (int v = 1; v < S; ++v) {
@@ -385,15 +407,19 @@ __global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(kResThreads, 1)
             if (x1_in) dst[v * vol + gi + 1] = z.y;
         }
     }
-    double part = hi + lo;
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-    if (lane == 0) red_hi[warp] = part;
+    for (int o = 16; o > 0; o >>= 1)
+        f3_add(sum, F3{__shfl_xor_sync(0xffffffffu, sum.hi, o), __shfl_xor_sync(0xffffffffu, sum.lo, o),
+                       __shfl_xor_sync(0xffffffffu, sum.lo2, o)});
+    if (lane == 0) {
+        red[0][warp] = sum.hi;
+        red[1][warp] = sum.lo;
+        red[2][warp] = sum.lo2;
+    }
     __syncthreads();
-    if (tid == 0) {
-        double b = 0.0;
-        for (int k = 0; k < nwarp; ++k) b += red_hi[k];
-        double* root = cl.map_shared_rank(cl_part, 0);
-        root[rank] = b;
+    if (warp == 0) {
+        double b = lane < nwarp ? (double)red[0][lane] + ((double)red[1][lane] + (double)red[2][lane]) : 0.0;
+        for (int o = 16; o > 0; o >>= 1) b += __shfl_xor_sync(0xffffffffu, b, o);
+        if (lane == 0) cl.map_shared_rank(cl_part, 0)[rank] = b;
     }
     cl.sync();
     if (rank == 0 && tid == 0) {
