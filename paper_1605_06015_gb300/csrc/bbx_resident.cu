@@ -170,7 +170,8 @@ __global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(kResThreads, 1)
 // for step s+1 can come before this CTA's last warp has arrived for step s),
 // never two, since its step s+2 waits for this CTA's border warps of step s+1;
 // by then they have read step s's halo values and passed its barrier.  The arithmetic of a node is the tiled
-// step kernel's, operation for operation, so results are bitwise the same.
+// step kernel's, operation for operation, so results are bitwise the same, in both state buffers: the state
+// before the last step is written too (a program that owns the buffers may look at both).
 // What bounded the kernel above: 82 instructions a node (16 CTAs of 32 warps,
 // three quarters of the issue slots) and a cluster-wide barrier a step.
 
@@ -316,6 +317,28 @@ __global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(kResThreads, 1)
     bool timed_out = false;
     int p = 0;
     for (int s = 0; s < n_steps; ++s) {
+        if (s + 1 == n_steps) {
+            // The buffer that does not become current gets the state of the step before the last one, as when
+            // every step writes its buffer (the initial state, where it held that, was read before the first
+            // cl.sync).  (`here` is 0: it keeps these addresses out of the registers of the other steps.)
+            int here;
+            asm volatile("mov.u32 %0, 0;" : "=r"(here));
+            float* const other = T->state[cur0 ^ 1 ^ (n_steps & 1)] + here;
+            const long long g0 = (long long)(rb0 + r0 + here) * px + x;
+#pragma unroll
+            for (int k = 0; k < R; ++k) {
+                if (k >= rows) continue;
+                float* o = other + g0 + (long long)k * px;
+#pragma unroll
+                for (int v = 0; v < S; ++v) {
+                    const float2 z = v == 0 ? u[k]
+                                     : VREG ? w[VREG && v > 0 ? k * (S - 1) + v - 1 : 0]
+                                            : *reinterpret_cast<const float2*>(Wv + ((v - 1) * maxr + r0 + k) * 2 * np + x);
+                    o[v * vol] = z.x;
+                    if (x1_in) o[v * vol + 1] = z.y;
+                }
+            }
+        }
         const uint32_t prev = bar_a + 8u * (uint32_t)((s - 1) & 1), phase = (uint32_t)((s - 1) >> 1) & 1u;
         if (s > 0 && !timed_out && !try_wait_cluster(prev, phase)) {
             const long long c0 = clock64();

@@ -36,3 +36,27 @@ def test_total_is_the_sum_of_the_state(bbx, nx, ny):
     G.step(0.01, 30)
     V = G.read_state(0).astype(np.float64).ravel()
     assert abs(G.step_total() - math.fsum(V)) <= 24 * 2.0 ** -53 * math.fsum(np.abs(V))
+
+
+@pytest.mark.parametrize("nx,ny,model,n", [(33, 31, "fhn", 4), (100, 90, "barkley", 7), (199, 201, "zfk", 20), (300, 300, "fhn", 31),
+                                           (200, 200, "diffusion", 8), (511, 333, "fhn", 100)])
+def test_other_buffer_holds_the_state_before_the_last_step(bbx, nx, ny, model, n):
+    """A program that owns both buffers finds in them the last two states, as after n calls of one
+    step, and its values beside the rows are left alone."""
+    import torch
+    got = []
+    for one in (False, True):
+        G, st = _sheet(bbx, nx, ny, model)
+        px = G.get_info()["px"]
+        bufs = [torch.full((st.shape[0], 1, ny, px), 7.0, device="cuda") for _ in range(2)]
+        G.bind_state(*bufs)
+        G.write_all(st)
+        for b in bufs:
+            b[..., nx:] = 7.0
+        for _ in range(n if one else 1):
+            G.step(0.01, 1 if one else n)
+        G.step_total()
+        cur = 0 if G.state_device_ptr(0) == bufs[0].data_ptr() else 1
+        got.append([bufs[cur].cpu().numpy(), bufs[cur ^ 1].cpu().numpy()])
+    for a, b in zip(*got):
+        assert np.array_equal(a.view(np.uint32), b.view(np.uint32))
