@@ -220,17 +220,20 @@ int bbx_ppm_frame(bbx_grid* g, const int* layers, const double* lo, const double
 int bbx_phase_singularities(bbx_grid* g, int var_a, double iso_a, int var_b, double iso_b, float* xyz_dev,
                             int max_points, int* n_found);
 
-/* Resident multi-step mode for small sheets.  A call of bbx_step with two or
- * more steps on an unmasked isotropic sheet (nz = 1) of FHN, Barkley, ZFK or
- * pure diffusion with the unsplit scheme and Euler solver that fits the
- * registers and shared memory of one cluster of 16 CTAs runs all its
- * steps there by itself, with the tiled kernel's results bitwise and without
- * this switch.  With on = 1, larger sheets of that kind run in the shared
+/* Resident multi-step mode for small sheets.  A call of bbx_step on an
+ * unmasked isotropic sheet (nz = 1) of FHN, Barkley, ZFK or pure diffusion
+ * with the unsplit scheme and Euler solver that fits the registers and shared
+ * memory of one cluster of 16 CTAs (two variables up to about 520 x 520) runs
+ * its steps there by itself, without this switch, where the call has enough
+ * steps to be faster so (2 up to 200 x 200, 5 for 400 x 400, 15 for 512 x
+ * 512); the tiled kernel's results bitwise, in both state buffers.  With on =
+ * 1, every call of two or more steps on such a sheet does, and sheets that do
+ * not fit there (more than 2048 columns, or 8 to 15 rows) run in the shared
  * memory of such a cluster (8 CTAs where the GPU offers no 16-CTA clusters),
  * each CTA a band of rows, the rows next to its band read from the
  * neighbours' shared memory, so a step costs neither a kernel launch nor a
- * trip through DRAM: up to about 200 KB of state per CTA (for two variables,
- * nx * ny up to ~260 000 with 16 CTAs).  The results of these agree with the
+ * trip through DRAM: up to about 200 KB of state per CTA (only the buffer
+ * that becomes current is written then).  The results of these agree with the
  * tiled kernel to rounding, not bitwise.  The fused total, time, step count
  * and activation map are kept as by the tiled kernel.  When the grid stops
  * qualifying (fibres, a mask, another scheme), steps go back to the tiled
@@ -548,6 +551,22 @@ int bbx_state_device_ptr(bbx_grid* g, int var, void** dev_ptr);
  * BBX_ERR_TIMEOUT, which the next synchronising call returns.  No fault, trap
  * or hang reaches the GPU. */
 int bbx_debug_poison_first_load(bbx_grid* g, int on);
+
+/* Which kernels a call of bbx_step takes is chosen by the grid's size and the
+ * number of steps; the results are bitwise the same (but see
+ * bbx_set_resident).  For tests and measurements, bbx_debug_route chooses:
+ * one launch a step, several steps a launch where the grid's kernel has them,
+ * or the resident kernel in registers where the sheet fits (a route that does
+ * not apply falls back to the one before it).  bbx_debug_launches: the
+ * launches made so far by bbx_step for this grid, out[0] of one step, out[1]
+ * of several steps, out[2] resident in registers, out[3] resident in shared
+ * memory.  Errors: BBX_ERR_ARG. */
+#define BBX_ROUTE_AUTO 0
+#define BBX_ROUTE_STEPS 1
+#define BBX_ROUTE_SEVERAL 2
+#define BBX_ROUTE_REGISTERS 3
+int bbx_debug_route(bbx_grid* g, int route);
+int bbx_debug_launches(bbx_grid* g, long long* out);
 
 /* Clear the sticky device error bits (after a reported BBX_ERR_NAN or
  * BBX_ERR_TIMEOUT).  Synchronous. */

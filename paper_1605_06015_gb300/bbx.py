@@ -32,6 +32,7 @@ NVARS = {BBX_FHN: 2, BBX_BARKLEY: 2, BBX_BR: 8, BBX_ZFK: 1, BBX_DIFFUSION: 1, BB
 BBX_ACT_NONE = 2147483647
 BBX_SCHEME_UNSPLIT, BBX_SCHEME_LIE = 0, 1
 BBX_SOLVER_EULER, BBX_SOLVER_RK4 = 0, 1
+BBX_ROUTE_AUTO, BBX_ROUTE_STEPS, BBX_ROUTE_SEVERAL, BBX_ROUTE_REGISTERS = 0, 1, 2, 3
 BBX_GATES_FP32, BBX_GATES_FP16, BBX_GATES_UNORM16 = 0, 1, 2
 
 
@@ -83,6 +84,8 @@ def _load():
         "bbx_autotune": [P, D, ctypes.POINTER(D)],
         "bbx_state_device_ptr": [P, I, ctypes.POINTER(P)],
         "bbx_debug_poison_first_load": [P, I],
+        "bbx_debug_route": [P, I],
+        "bbx_debug_launches": [P, ctypes.POINTER(LL)],
         "bbx_clear_device_error": [P],
         "bbx_set_timestep": [P, D],
         "bbx_set_scheme": [P, I],
@@ -431,6 +434,18 @@ def bbx_state_device_ptr(g, var):
 
 def bbx_debug_poison_first_load(g, on):
     _check(_lib.bbx_debug_poison_first_load(g, int(bool(on))), "bbx_debug_poison_first_load")
+
+
+def bbx_debug_route(g, route):
+    """Test hook: BBX_ROUTE_* instead of the choice by size and number of steps."""
+    _check(_lib.bbx_debug_route(g, int(route)), "bbx_debug_route")
+
+
+def bbx_debug_launches(g):
+    """Test hook: launches of bbx_step so far (one step, several steps, resident in registers, in shared memory)."""
+    out = (ctypes.c_longlong * 4)()
+    _check(_lib.bbx_debug_launches(g, out), "bbx_debug_launches")
+    return list(out)
 
 
 def bbx_clear_device_error(g):

@@ -32,7 +32,7 @@ cudaError_t launch_ppm(const float* s0, const float* s1, const int* cur, const u
 cudaError_t resident_sheet_steps(int model, const TissueArgs* d_t, int nx, int ny, int n_steps, int* d_err,
                                  cudaStream_t s, bool check_only, bool* ok);
 cudaError_t resident_pair_steps(int model, const TissueArgs* d_t, int nx, int ny, int n_steps, int* d_err,
-                                cudaStream_t s, bool check_only, bool* ok);
+                                cudaStream_t s, bool check_only, bool* ok, int* from);
 cudaError_t launch_singz(const float* s0, const float* s1, const int* cur, long long off_a, long long off_b,
                          float iso_a, float iso_b, const uint8_t* mask, int nx, int ny, int nz, int px,
                          long long plane, float* xyz, int max_points, int* d_count, int num_sms, cudaStream_t s);
@@ -1021,6 +1021,9 @@ struct bbx_grid {
     int rk4 = 0;    // kinetics solver (bbx_set_solver)
     int resident = 0;  // multi-step resident kernel requested (bbx_set_resident)
     bool pairs_ok = false;  // the grid's shape runs in the register-resident kernel (looked up with the plan)
+    int pairs_from = 0;     // and is faster there in calls of this many steps or more
+    int route = BBX_ROUTE_AUTO;   // bbx_debug_route
+    long long launches[4] = {};   // bbx_debug_launches
 
     // z-slab of a decomposed grid: the first halo_lo and last halo_hi planes
     // are halo planes (a neighbour slab's boundary V, read by the stencil,
@@ -1401,7 +1404,8 @@ int prepare(bbx_grid* g) {
     g->pairs_ok = false;
     if (resident_shape(g)) {
         bool ok = false;
-        if (resident_pair_steps(g->model, nullptr, g->nx, g->ny, 0, nullptr, g->stream, true, &ok) != cudaSuccess)
+        if (resident_pair_steps(g->model, nullptr, g->nx, g->ny, 0, nullptr, g->stream, true, &ok, &g->pairs_from) !=
+            cudaSuccess)
             cudaGetLastError();
         else
             g->pairs_ok = ok;
@@ -2036,6 +2040,18 @@ int bbx_debug_poison_first_load(bbx_grid* g, int on) {
     return BBX_OK;
 }
 
+int bbx_debug_route(bbx_grid* g, int route) {
+    if (!g || route < BBX_ROUTE_AUTO || route > BBX_ROUTE_REGISTERS) return BBX_ERR_ARG;
+    g->route = route;
+    return BBX_OK;
+}
+
+int bbx_debug_launches(bbx_grid* g, long long* out) {
+    if (!g || !out) return BBX_ERR_ARG;
+    for (int k = 0; k < 4; ++k) out[k] = g->launches[k];
+    return BBX_OK;
+}
+
 int bbx_clear_device_error(bbx_grid* g) {
     if (!g) return BBX_ERR_ARG;
     BBX_CUDA(cudaMemsetAsync(g->d_err, 0, sizeof(int), g->stream));
@@ -2065,22 +2081,25 @@ int bbx_step(bbx_grid* g, double dt, int n_steps) {
         g->stepped = true;
         return BBX_OK;
     }
-    if (n_steps >= 2 && g->pairs_ok && resident_eligible(g)) {
-        // a sheet that fits: all its steps in one cluster's registers and shared
-        // memory (200^2, 20 steps a call: 1.8 us a step against 4.7 by tiles; 200
-        // steps: 1.1 us), the same results
+    if (n_steps >= 2 && g->pairs_ok && resident_eligible(g) &&
+        (g->route == BBX_ROUTE_REGISTERS ||
+         (g->route == BBX_ROUTE_AUTO && (g->resident || n_steps >= g->pairs_from)))) {
+        // a sheet that fits, in a call long enough (or where it was asked for): all
+        // its steps in one cluster's registers and shared memory (200^2, 20 steps a
+        // call: 1.6 us a step against 4.7 by tiles; 200 steps: 1.1 us), the same results
         while (n_steps > 0) {
             const int chunk = std::min(n_steps, 1 << 16);
             bool ok = false;
-            BBX_CUDA(resident_pair_steps(g->model, g->d_t, g->nx, g->ny, chunk, g->d_err, g->stream, false, &ok));
+            BBX_CUDA(resident_pair_steps(g->model, g->d_t, g->nx, g->ny, chunk, g->d_err, g->stream, false, &ok, nullptr));
             if (!ok) return BBX_ERR_STATE;
+            ++g->launches[2];
             n_steps -= chunk;
             g->h_cur ^= chunk & 1;
         }
         g->stepped = true;
         return BBX_OK;
     }
-    if (g->resident && n_steps >= 2 && resident_eligible(g)) {
+    if (g->resident && n_steps >= 2 && g->route == BBX_ROUTE_AUTO && resident_eligible(g)) {
         int done = 0;
         while (done < n_steps) {
             const int chunk = std::min(n_steps - done, 1 << 16);
@@ -2089,6 +2108,7 @@ int bbx_step(bbx_grid* g, double dt, int n_steps) {
                                                        false, &ok);
             if (e != cudaSuccess) return fail_cuda(e);
             if (!ok) break;  // not launchable after all: the tiled kernel takes the rest
+            ++g->launches[3];
             done += chunk;
             g->h_cur ^= chunk & 1;
         }
@@ -2107,7 +2127,7 @@ int bbx_step(bbx_grid* g, double dt, int n_steps) {
         L.reg_ctas = g->lp.ctas;
         L.reg_planes = g->lp.n_planes;
     }
-    const bool flow = n_steps >= 2 && g->lp.flow && !g->poison && !capturing(g->stream);
+    const bool flow = n_steps >= 2 && g->lp.flow && g->route != BBX_ROUTE_STEPS && !g->poison && !capturing(g->stream);
     while (flow && g->lp.flow && n_steps >= 2) {
         const int m = std::min(n_steps, kFlowSteps);
         L.cur_hint = g->h_cur;
@@ -2116,6 +2136,7 @@ int bbx_step(bbx_grid* g, double dt, int n_steps) {
             g->lp.flow = false;
             break;
         }
+        ++g->launches[1];
         g->h_cur ^= m & 1;
         n_steps -= m;
     }
@@ -2123,6 +2144,7 @@ int bbx_step(bbx_grid* g, double dt, int n_steps) {
         L.cur_hint = g->h_cur;
         const cudaError_t e = launch(g->lp, L, g->stream);
         if (e != cudaSuccess) return fail_cuda(e);
+        ++g->launches[0];
         g->h_cur ^= 1;
     }
     g->stepped = true;

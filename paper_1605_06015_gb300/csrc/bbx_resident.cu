@@ -8,6 +8,8 @@
 // section "Computation of intermediate expressions" with the 5-point
 // operator of an isotropic sheet (faces only; no-flux edges: a missing
 // neighbour contributes nothing).
+#include <limits.h>
+
 #include <cooperative_groups.h>
 
 #include "bbx_device.cuh"
@@ -466,9 +468,26 @@ inline int pair_rows(int nx, int ny, int NC) {
     return 0;
 }
 
+// From how many steps of a call this kernel is the faster route (the call's
+// fixed cost, 16 SMs loading and storing the sheet, against one launch a step).
+// Measured, us a call of n steps here and by tiles with the fastest height:
+// 200x200 n = 2 11.7 / 11.9; 256x256 n = 2 12.4 / 11.9, n = 3 14.5 / 17.8;
+// 340x340 n = 2 16.6 / 13.2, n = 3 18.6 / 19.8; one variable 512x512 n = 4
+// 25.8 / 25.2, n = 6 32 / 38.  With more than four rows a thread the second
+// variable is in shared memory, and registers spill, more with more rows:
+// 362x362 n = 3 22.6 / 20.2, n = 4 24.8 / 27.1; 400x400 n = 4 26.8 / 27.2, n = 6
+// 32 / 41; 450x450 n = 10 67 / 70; 512x512 n = 10 72 / 65, n = 20 124 / 128;
+// twelve rows: one variable 560x560 n = 10 68 / 67, n = 16 99 / 107, two
+// variables 520x520 n = 20 159 / 140.
+inline int pairs_from(int S, int R, int nx, int ny) {
+    const int n = nx * ny;  // (at most 16 x 1024 x 12 x 2)
+    if (R > 8) return S == 1 ? 11 : INT_MAX;
+    return 2 + n / (S == 1 || R <= 4 ? 65536 : (R <= 6 ? 50000 : 19000));
+}
+
 template <int MODEL, int NC, int R>
 cudaError_t pairs_try(const TissueArgs* d_t, int nx, int ny, int n_steps, int* d_err, cudaStream_t s, bool check_only,
-                      bool* ok) {
+                      bool* ok, int* from) {
     const int np = (nx + 1) / 2, maxr = (ny + NC - 1) / NC, pitch = 2 * np + kPairPad;
     const size_t smem = sizeof(float) * (2 * (size_t)(maxr + 2) * pitch +
                                          (pair_regs<MODEL>(R) ? 0 : (size_t)(Model<MODEL>::S - 1) * maxr * 2 * np));
@@ -493,6 +512,7 @@ cudaError_t pairs_try(const TissueArgs* d_t, int nx, int ny, int n_steps, int* d
             return cudaSuccess;
         }
         *ok = clusters >= 1;
+        *from = pairs_from(Model<MODEL>::S, R, nx, ny);
         return cudaSuccess;
     }
     *ok = true;
@@ -502,17 +522,17 @@ cudaError_t pairs_try(const TissueArgs* d_t, int nx, int ny, int n_steps, int* d
 
 template <int MODEL>
 cudaError_t pairs_launch(const TissueArgs* d_t, int nx, int ny, int n_steps, int* d_err, cudaStream_t s,
-                         bool check_only, bool* ok) {
+                         bool check_only, bool* ok, int* from) {
     constexpr int NC = kResCtasLarge;
     *ok = false;
     switch (pair_rows(nx, ny, NC)) {
-        case 1: return pairs_try<MODEL, NC, 1>(d_t, nx, ny, n_steps, d_err, s, check_only, ok);
-        case 2: return pairs_try<MODEL, NC, 2>(d_t, nx, ny, n_steps, d_err, s, check_only, ok);
-        case 3: return pairs_try<MODEL, NC, 3>(d_t, nx, ny, n_steps, d_err, s, check_only, ok);
-        case 4: return pairs_try<MODEL, NC, 4>(d_t, nx, ny, n_steps, d_err, s, check_only, ok);
-        case 6: return pairs_try<MODEL, NC, 6>(d_t, nx, ny, n_steps, d_err, s, check_only, ok);
-        case 8: return pairs_try<MODEL, NC, 8>(d_t, nx, ny, n_steps, d_err, s, check_only, ok);
-        case 12: return pairs_try<MODEL, NC, 12>(d_t, nx, ny, n_steps, d_err, s, check_only, ok);
+        case 1: return pairs_try<MODEL, NC, 1>(d_t, nx, ny, n_steps, d_err, s, check_only, ok, from);
+        case 2: return pairs_try<MODEL, NC, 2>(d_t, nx, ny, n_steps, d_err, s, check_only, ok, from);
+        case 3: return pairs_try<MODEL, NC, 3>(d_t, nx, ny, n_steps, d_err, s, check_only, ok, from);
+        case 4: return pairs_try<MODEL, NC, 4>(d_t, nx, ny, n_steps, d_err, s, check_only, ok, from);
+        case 6: return pairs_try<MODEL, NC, 6>(d_t, nx, ny, n_steps, d_err, s, check_only, ok, from);
+        case 8: return pairs_try<MODEL, NC, 8>(d_t, nx, ny, n_steps, d_err, s, check_only, ok, from);
+        case 12: return pairs_try<MODEL, NC, 12>(d_t, nx, ny, n_steps, d_err, s, check_only, ok, from);
     }
     return cudaSuccess;
 }
@@ -569,14 +589,15 @@ cudaError_t resident_launch(const TissueArgs* d_t, int nx, int ny, int n_steps, 
 // n_steps on a small isotropic, unmasked sheet with the register-resident
 // kernel, bitwise as the tiled kernel steps it.  check_only: report in *ok
 // whether the grid's shape runs there (and make the kernel ready for it; a
-// launch needs an earlier check of the same shape).
+// launch needs an earlier check of the same shape) and in *from from how many
+// steps of a call it is the faster route.
 cudaError_t resident_pair_steps(int model, const TissueArgs* d_t, int nx, int ny, int n_steps, int* d_err,
-                                cudaStream_t s, bool check_only, bool* ok) {
+                                cudaStream_t s, bool check_only, bool* ok, int* from) {
     switch (model) {
-        case BBX_FHN: return pairs_launch<BBX_FHN>(d_t, nx, ny, n_steps, d_err, s, check_only, ok);
-        case BBX_BARKLEY: return pairs_launch<BBX_BARKLEY>(d_t, nx, ny, n_steps, d_err, s, check_only, ok);
-        case BBX_ZFK: return pairs_launch<BBX_ZFK>(d_t, nx, ny, n_steps, d_err, s, check_only, ok);
-        case BBX_DIFFUSION: return pairs_launch<BBX_DIFFUSION>(d_t, nx, ny, n_steps, d_err, s, check_only, ok);
+        case BBX_FHN: return pairs_launch<BBX_FHN>(d_t, nx, ny, n_steps, d_err, s, check_only, ok, from);
+        case BBX_BARKLEY: return pairs_launch<BBX_BARKLEY>(d_t, nx, ny, n_steps, d_err, s, check_only, ok, from);
+        case BBX_ZFK: return pairs_launch<BBX_ZFK>(d_t, nx, ny, n_steps, d_err, s, check_only, ok, from);
+        case BBX_DIFFUSION: return pairs_launch<BBX_DIFFUSION>(d_t, nx, ny, n_steps, d_err, s, check_only, ok, from);
     }
     *ok = false;
     return cudaSuccess;
