@@ -291,8 +291,10 @@ int bbx_set_solver(bbx_grid* g, int solver);
 
 /* Advance n_steps explicit steps of size dt (asynchronous on the grid's
  * stream).  Unmasked grids of at most two variables take up to 64 steps in one
- * cooperative launch (one launch a step while the stream is being captured
- * into a graph); results are bitwise those of calls with one step.  Each step
+ * cooperative launch where that is faster: from two steps a call on with 3
+ * million nodes, in longer calls or not at all on smaller grids (and one
+ * launch a step while the stream is being captured into a graph); results are
+ * bitwise those of calls with one step.  Each step
  * also reduces the new V over tissue nodes into one double-precision partial
  * per piece of its schedule (the total is summed from them, in a fixed order,
  * by bbx_step_total).  Errors: BBX_ERR_STATE (no

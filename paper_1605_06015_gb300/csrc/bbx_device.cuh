@@ -51,7 +51,9 @@ struct TissueDyn {
     long long n;    // steps taken
     int cur;        // buffer holding the current state (0 or 1)
     int total_pending;  // 1: total is still to be summed from the per-piece
-                        // partials of the grid's last single-grid launch
+                        // partials of the grid's last single-grid launch:
+    int n_slots;
+    const double* partials;
 };
 
 // Host-written description of one grid for the step kernel (in device memory,
@@ -354,6 +356,8 @@ __device__ __forceinline__ void start_ticket(const LaunchArgs& L, const TissueDy
         d->t = tn;
         d->n = d0.n + L.n_steps;
         d->cur = d0.cur ^ (L.n_steps & 1);
+        d->n_slots = L.n_slots;
+        d->partials = L.partials;
         d->total_pending = 1;
         *L.ticket = 0u;
     }

@@ -4,6 +4,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -533,11 +534,12 @@ __global__ void k_total(const float* __restrict__ u, const uint8_t* __restrict__
 // The total of a grid's last single-grid step, summed from the step's
 // per-piece partials in slot order (unused slots hold 0) when it is asked
 // for; nothing happens if no total is pending.  One CTA.
-__global__ void k_finish_total(const double* __restrict__ partials, int n_slots, TissueDyn* dyn, int* err) {
+__global__ void k_finish_total(TissueDyn* dyn, int* err) {
     __shared__ double scratch[32];
     if (!dyn->total_pending) return;  // uniform: every thread reads the same flag
     double s = 0.0;
-    for (int k = threadIdx.x; k < n_slots; k += blockDim.x) s += partials[k];
+    const double* partials = dyn->partials;
+    for (int k = threadIdx.x; k < dyn->n_slots; k += blockDim.x) s += partials[k];
     const double total = block_sum_double(s, scratch);
     if (threadIdx.x == 0) {
         if (!isfinite(total)) atomicOr(err, ERRBIT_NAN);
@@ -919,6 +921,38 @@ cudaError_t launch(const LaunchPlan& lp, const LaunchArgs& L, cudaStream_t s) {
     return cudaLaunchKernelExC(&cfg, lp.k.fn, args);
 }
 
+// From how many steps of a call a grid takes several steps a launch (0: never).
+// A launch of several steps costs 5 us more than one of one step (20 us where a
+// step takes 200) and saves each further step the fill and drain of a launch,
+// 2 to 8 us; but a CTA's share of a step has to be long against the round trips
+// of the done flags (3 us), or the CTAs wait for one another every step.
+// Measured (us a step, one launch a step / several steps a launch, the best
+// tile height of each):
+// - 3 million nodes or more, share of 5 to 500 planes: never slower than the
+//   kernels of one step a launch were before, from n = 2 on (256x256x64 slab
+//   n = 2 26.3 / 25.7, n = 10 26.3 / 22.1; 192^3 n = 2 28.1 / 27.3; 8192x8192
+//   n = 4 200 / 201, n = 10 200 / 189);
+// - fewer, with long shares: 128^3 anisotropic, 16 planes n = 3 16.2 / 16.0;
+//   isotropic, 11 planes n = 6 13.3 / 13.6, n = 10 13.3 / 13.1; 1500x1500 and
+//   1400x1400, 3 to 14 planes, n = 10 12.0 / 12.1, n = 20 11.9 / 11.5;
+// - below 1.5 million nodes not (700x900 n = 20 8.9 / 9.8; 1024x1024 8.8 / 10.8;
+//   96^3 anisotropic 12.9 / 14.1);
+// - except where no CTA takes more than one plane and few CTAs exchange flags:
+//   sheets up to a CTA an SM (60 CTAs n = 10 6.1 / 6.1, 110 n = 20 6.1 / 5.8, 152
+//   n = 20 6.8 / 7.0), blocks (80 CTAs n = 6 7.1 / 7.1, 192 n = 10 8.0 / 7.6, 320
+//   n = 20 8.8 / 8.2).
+constexpr long long kFlowNodes = 3000000, kFlowNodesMin = 1500000;
+int flow_steps_from(long long nodes, long long planes, int ctas, int num_sms, bool planar) {
+    if (nodes >= kFlowNodes) return 2;
+    if (planes <= ctas) {
+        if (planar) return planes <= num_sms ? 4 + (int)planes / 8 : 0;
+        return std::max(8, (int)planes / 12);
+    }
+    if (nodes < kFlowNodesMin) return 0;
+    const long long share = planes / ctas;
+    return share >= 15 ? 3 : (share >= 8 ? 10 : 20);
+}
+
 // Select the kernel for a configuration, check it fits, and return the CTA
 // budget (resident CTAs on the whole GPU).
 int select_kernel(int model, bool masked, int aniso, int ty, int device, int num_sms, StepKernel* out,
@@ -1011,7 +1045,13 @@ struct bbx_grid {
     TissueArgs h_t;                // host copy of the kernel's view of this grid
     TissueArgs* d_t = nullptr;     // device copy
     TissueDyn* d_dyn = nullptr;    // device-updated time, step, parity, total
-    LaunchPlan lp;                 // single-grid launch
+    // lp: one step a launch, and several of grids with kFlowNodes nodes or more;
+    // lpf: several steps a launch of smaller grids, in calls of flow_from steps or
+    // more (the kernels without the sync warp, four CTAs an SM instead of three
+    // when isotropic, are the faster ones at one step a launch there: 400x400 6.5 us
+    // against 7.3, 128^3 13.3 against 14.4)
+    LaunchPlan lp, lpf;
+    int flow_from = 0;
     bool ready = false;            // h_t, d_t and lp match the current settings
     unsigned long long version = 1;  // bumped whenever the kernel's view changes
 
@@ -1382,24 +1422,45 @@ int prepare(bbx_grid* g) {
     int rc0 = finish_total(g);  // the plan's partials are about to be replaced
     if (rc0 || (rc0 = tab_refresh(g))) return rc0;
     BBX_CUDA(cudaStreamSynchronize(g->stream));
-    StepKernel k;
-    int ctas = 0;
     const bool surr = g->surr_on && g->model == BBX_BR;
-    int rc = BBX_ERR_UNSUPPORTED;
-    if (g->aniso && g->wsum_zero && g->wsum_elide && !g->d_mask)  // the variant without W-tilde sums, if built
-        rc = select_kernel(g->model, false, AN_NO_SUMS, g->ty, g->device, g->num_sms, &k, &ctas, surr, g->nz == 1,
-                           wants_general(g), g->gates);
-    if (rc == BBX_ERR_UNSUPPORTED)
-        rc = select_kernel(g->model, g->d_mask != nullptr, g->aniso ? AN_SUMS : AN_ISO, g->ty, g->device,
-                           g->num_sms, &k, &ctas, surr, g->nz == 1, wants_general(g), g->gates);
+    auto pick = [&](bool flow, StepKernel* k, int* ctas) {
+        int r = BBX_ERR_UNSUPPORTED;
+        if (g->aniso && g->wsum_zero && g->wsum_elide && !g->d_mask)  // the variant without W-tilde sums, if built
+            r = select_kernel(g->model, false, AN_NO_SUMS, g->ty, g->device, g->num_sms, k, ctas, surr, g->nz == 1,
+                              wants_general(g), g->gates, flow);
+        if (r == BBX_ERR_UNSUPPORTED)
+            r = select_kernel(g->model, g->d_mask != nullptr, g->aniso ? AN_SUMS : AN_ISO, g->ty, g->device,
+                              g->num_sms, k, ctas, surr, g->nz == 1, wants_general(g), g->gates, flow);
+        return r;
+    };
+    StepKernel kf;
+    int ctas = 0;
+    int rc = pick(true, &kf, &ctas);
     if (rc) return rc;
-    if ((rc = encode_targs(g, k.ty, &g->h_t))) return rc;
+    if ((rc = encode_targs(g, kf.ty, &g->h_t))) return rc;
     BBX_CUDA(cudaMemcpyAsync(g->d_t, &g->h_t, sizeof(TissueArgs), cudaMemcpyHostToDevice, g->stream));
     std::vector<Seg> segs;
-    grid_segments(g, k.ty, 0, &segs);
-    g->lp.k = k;
+    grid_segments(g, kf.ty, 0, &segs);
     std::vector<Lattice> lattice;
-    if (!g->d_mask) lattice.push_back(grid_lattice(g, k.ty));
+    if (!g->d_mask) lattice.push_back(grid_lattice(g, kf.ty));
+    g->flow_from = 0;
+    g->lp.k = kf;
+    if (kf.flow && !g->d_mask) {
+        const long long nodes = (long long)g->nx * g->ny * (g->nz - g->halo_lo - g->halo_hi);
+        long long planes = 0;
+        for (const Seg& sg : segs) planes += sg.z1 - sg.z0;
+        g->flow_from = flow_steps_from(nodes, planes, ctas, g->num_sms, g->nz == 1);
+        if (g->flow_from == 0 && g->route >= BBX_ROUTE_SEVERAL) g->flow_from = INT_MAX;  // (only asked for)
+        if (nodes < kFlowNodes) {
+            if (g->flow_from) {
+                g->lpf.k = kf;
+                if ((rc = build_plan(&g->lpf, segs, 1, ctas, lattice, g->device))) return rc;
+            }
+            if ((rc = pick(false, &g->lp.k, &ctas))) return rc;
+            lattice.clear();
+        }
+    }
+    if (!g->flow_from || !lattice.empty()) g->lpf.release();
     if ((rc = build_plan(&g->lp, segs, 1, ctas, lattice, g->device))) return rc;
     g->pairs_ok = false;
     if (resident_shape(g)) {
@@ -1455,7 +1516,7 @@ int write_dyn(bbx_grid* g, const TissueDyn& d) {
 // anything that reads the total or overwrites the partials.
 int finish_total(bbx_grid* g) {
     if (!g->lp.d_partials || g->lp.n_slots <= 0 || !g->d_dyn) return BBX_OK;
-    k_finish_total<<<1, 256, 0, g->stream>>>(g->lp.d_partials, g->lp.n_slots, g->d_dyn, g->d_err);
+    k_finish_total<<<1, 256, 0, g->stream>>>(g->d_dyn, g->d_err);
     BBX_CUDA(cudaGetLastError());
     return BBX_OK;
 }
@@ -1587,6 +1648,7 @@ void bbx_destroy_grid(bbx_grid* g) {
     cudaFree(g->d_dyn);
     cudaFree(g->d_surr);
     g->lp.release();
+    g->lpf.release();
     cudaFree(g->d_partials);
     cudaFree(g->d_ticket);
     cudaFree(g->d_total2);
@@ -2043,6 +2105,7 @@ int bbx_debug_poison_first_load(bbx_grid* g, int on) {
 int bbx_debug_route(bbx_grid* g, int route) {
     if (!g || route < BBX_ROUTE_AUTO || route > BBX_ROUTE_REGISTERS) return BBX_ERR_ARG;
     g->route = route;
+    g->ready = false;  // (a plan for several steps a launch is built where it is asked for)
     return BBX_OK;
 }
 
@@ -2116,30 +2179,39 @@ int bbx_step(bbx_grid* g, double dt, int n_steps) {
         n_steps -= done;
         if (n_steps == 0) return BBX_OK;
     }
-    LaunchArgs L = launch_args(g->lp, g->d_t, g->d_err, g->poison, &g->h_t);
-    if (!g->d_mask) {
-        // unmasked grid: whole columns in order (nz planes, or a sheet's nby
-        // tile rows), equal shares (build_plan)
-        L.reg_len = g->nz > 1 ? g->nz - g->halo_lo - g->halo_hi : (g->ny + g->lp.k.ty - 1) / g->lp.k.ty;
-        L.reg_z0 = g->nz > 1 ? g->halo_lo : 0;
-        L.reg_nbx = g->nbx;
-        L.reg_ty = g->lp.k.ty;
-        L.reg_ctas = g->lp.ctas;
-        L.reg_planes = g->lp.n_planes;
-    }
-    const bool flow = n_steps >= 2 && g->lp.flow && g->route != BBX_ROUTE_STEPS && !g->poison && !capturing(g->stream);
-    while (flow && g->lp.flow && n_steps >= 2) {
-        const int m = std::min(n_steps, kFlowSteps);
-        L.cur_hint = g->h_cur;
-        if (launch_flow(&g->lp, &L, m, g->stream) != cudaSuccess) {
-            cudaGetLastError();  // not launchable as a whole: one launch per step from here on
-            g->lp.flow = false;
-            break;
+    auto args = [&](const LaunchPlan& lp) {
+        LaunchArgs L = launch_args(lp, g->d_t, g->d_err, g->poison, &g->h_t);
+        if (!g->d_mask) {
+            // unmasked grid: whole columns in order (nz planes, or a sheet's nby
+            // tile rows), equal shares (build_plan)
+            L.reg_len = g->nz > 1 ? g->nz - g->halo_lo - g->halo_hi : (g->ny + lp.k.ty - 1) / lp.k.ty;
+            L.reg_z0 = g->nz > 1 ? g->halo_lo : 0;
+            L.reg_nbx = g->nbx;
+            L.reg_ty = lp.k.ty;
+            L.reg_ctas = lp.ctas;
+            L.reg_planes = lp.n_planes;
         }
-        ++g->launches[1];
-        g->h_cur ^= m & 1;
-        n_steps -= m;
+        return L;
+    };
+    LaunchPlan* lpf = g->lp.flow ? &g->lp : &g->lpf;
+    const int flow_from = g->route >= BBX_ROUTE_SEVERAL ? 2 : g->flow_from;
+    if (lpf->flow && flow_from && n_steps >= flow_from && g->route != BBX_ROUTE_STEPS && !g->poison &&
+        !capturing(g->stream)) {
+        LaunchArgs L = args(*lpf);
+        while (n_steps >= flow_from) {
+            const int m = std::min(n_steps, kFlowSteps);
+            L.cur_hint = g->h_cur;
+            if (launch_flow(lpf, &L, m, g->stream) != cudaSuccess) {
+                cudaGetLastError();  // not launchable as a whole: one launch per step from here on
+                lpf->flow = false;
+                break;
+            }
+            ++g->launches[1];
+            g->h_cur ^= m & 1;
+            n_steps -= m;
+        }
     }
+    LaunchArgs L = args(g->lp);
     for (int s = 0; s < n_steps; ++s) {
         L.cur_hint = g->h_cur;
         const cudaError_t e = launch(g->lp, L, g->stream);

@@ -81,3 +81,72 @@ def test_one_launch_a_step_asked_for(bbx, nx, ny):
     _same(A, B)
     with pytest.raises(bbx.BbxError):
         A.debug_route(4)
+
+
+def _block(bbx, model, shape, fibres, ty, setup=None):
+    from test_gpu_flow import _grid
+    mid = {"fhn": bbx.BBX_FHN, "barkley": bbx.BBX_BARKLEY, "br": bbx.BBX_BR, "zfk": bbx.BBX_ZFK,
+           "diffusion": bbx.BBX_DIFFUSION}[model]
+    return _grid(bbx, mid, shape, fibres, ty, setup)
+
+
+@pytest.mark.parametrize("model,shape,fibres,ty,n,several", [
+    ("fhn", (1, 900, 700), "none", 14, 5, False), ("fhn", (1, 900, 700), "none", 28, 64, False),
+    ("barkley", (1, 130, 200), "smooth", 14, 8, False), ("barkley", (1, 130, 200), "smooth", 14, 9, True),
+    ("barkley", (16, 64, 64), "rotational", 14, 7, False), ("barkley", (16, 64, 64), "rotational", 14, 8, True),
+    ("fhn", (96, 96, 96), "none", 28, 64, False), ("barkley", (128, 128, 128), "rotational", 7, 2, False),
+    ("barkley", (128, 128, 128), "rotational", 7, 3, True), ("fhn", (128, 128, 128), "none", 14, 6, False),
+    ("fhn", (1, 2048, 2048), "none", 28, 2, True), ("br", (9, 40, 64), "rotational", 7, 30, False)])
+def test_short_calls_on_small_grids_take_one_launch_a_step(bbx, model, shape, fibres, ty, n, several):
+    A, dt = _block(bbx, model, shape, fibres, ty)
+    B, _ = _block(bbx, model, shape, fibres, ty)
+    A.step(dt, n)
+    assert A.debug_launches() == ([0, 1, 0, 0] if several else [n, 0, 0, 0])
+    _one_by_one(B, dt, n)
+    assert B.debug_launches() == [n, 0, 0, 0]
+    _same(A, B)
+
+
+from test_gpu_flow import CASES  # noqa: E402
+
+SEVERAL = [c for c in CASES if c[1] != "br"] + [
+    ("sheet, 28 rows", "fhn", (1, 900, 700), "none", 28, None, 9),
+    ("isotropic block, 28 rows", "fhn", (21, 71, 130), "none", 28, None, 6),
+    ("anisotropic block, 28 rows", "barkley", (33, 57, 65), "smooth", 28, None, 7),
+    ("two columns, 28 rows", "zfk", (40, 29, 64), "none", 28, None, 5)]
+
+
+@pytest.mark.parametrize("name,model,shape,fibres,ty,setup,n", SEVERAL, ids=[c[0] for c in SEVERAL])
+def test_several_steps_a_launch_asked_for(bbx, name, model, shape, fibres, ty, setup, n):
+    """The cases of several steps a launch, and tiles of 28 rows, whatever the grid's size chooses; mixed
+    with launches of one step, whose totals are summed from another plan's pieces."""
+    A, dt = _block(bbx, model, shape, fibres, ty, setup)
+    B, _ = _block(bbx, model, shape, fibres, ty, setup)
+    A.debug_route(bbx.BBX_ROUTE_SEVERAL)
+    for m in (n, 1, n):  # the second call starts from the parity the first one left
+        A.step(dt, m)
+        _one_by_one(B, dt, m)
+        _same(A, B)
+    assert A.debug_launches()[:3] == [1 + 2 * (n % 64 == 1), 2 * (-(-n // 64)) - 2 * (n % 64 == 1), 0]
+
+
+def test_captured_one_step_launches_between_calls_of_several(bbx):
+    """A replay of captured one-step launches after a call of several steps leaves its own total."""
+    torch = pytest.importorskip("torch")
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        A, dt = _block(bbx, "barkley", (16, 64, 64), "rotational", 14)
+        B, _ = _block(bbx, "barkley", (16, 64, 64), "rotational", 14)
+        A.step(dt, 2)
+        s.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            A.step(dt, 12)
+        A.step(dt, 12)
+        A.step(dt, 20)
+        g.replay()
+        s.synchronize()
+        _one_by_one(B, dt, 46)
+        s.synchronize()
+        _same(A, B)
+        assert A.debug_launches() == [2 + 12, 2, 0, 0]
