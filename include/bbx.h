@@ -570,6 +570,12 @@ int bbx_debug_poison_first_load(bbx_grid* g, int on);
 int bbx_debug_route(bbx_grid* g, int route);
 int bbx_debug_launches(bbx_grid* g, long long* out);
 
+/* Fault injection: when on, launches of several steps of this grid, alone or
+ * as a member of a batch, are answered as if the device refused them (a
+ * process that was given fewer SMs since they were planned); the steps are
+ * then launched one by one.  Errors: BBX_ERR_ARG. */
+int bbx_debug_refuse_launches(bbx_grid* g, int on);
+
 /* Clear the sticky device error bits (after a reported BBX_ERR_NAN or
  * BBX_ERR_TIMEOUT).  Synchronous. */
 int bbx_clear_device_error(bbx_grid* g);

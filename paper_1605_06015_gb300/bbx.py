@@ -85,6 +85,7 @@ def _load():
         "bbx_state_device_ptr": [P, I, ctypes.POINTER(P)],
         "bbx_debug_poison_first_load": [P, I],
         "bbx_debug_route": [P, I],
+        "bbx_debug_refuse_launches": [P, I],
         "bbx_debug_launches": [P, ctypes.POINTER(LL)],
         "bbx_clear_device_error": [P],
         "bbx_set_timestep": [P, D],
@@ -439,6 +440,10 @@ def bbx_debug_poison_first_load(g, on):
 def bbx_debug_route(g, route):
     """Test hook: BBX_ROUTE_* instead of the choice by size and number of steps."""
     _check(_lib.bbx_debug_route(g, int(route)), "bbx_debug_route")
+
+
+def bbx_debug_refuse_launches(g, on):
+    _check(_lib.bbx_debug_refuse_launches(g, int(bool(on))), "bbx_debug_refuse_launches")
 
 
 def bbx_debug_launches(g):

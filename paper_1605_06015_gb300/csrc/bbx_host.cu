@@ -1064,6 +1064,7 @@ struct bbx_grid {
     int pairs_from = 0;     // and is faster there in calls of this many steps or more
     int route = BBX_ROUTE_AUTO;   // bbx_debug_route
     long long launches[4] = {};   // bbx_debug_launches
+    int refuse = 0;               // bbx_debug_refuse_launches
 
     // z-slab of a decomposed grid: the first halo_lo and last halo_hi planes
     // are halo planes (a neighbour slab's boundary V, read by the stencil,
@@ -2109,6 +2110,12 @@ int bbx_debug_route(bbx_grid* g, int route) {
     return BBX_OK;
 }
 
+int bbx_debug_refuse_launches(bbx_grid* g, int on) {
+    if (!g) return BBX_ERR_ARG;
+    g->refuse = on ? 1 : 0;
+    return BBX_OK;
+}
+
 int bbx_debug_launches(bbx_grid* g, long long* out) {
     if (!g || !out) return BBX_ERR_ARG;
     for (int k = 0; k < 4; ++k) out[k] = g->launches[k];
@@ -2153,14 +2160,18 @@ int bbx_step(bbx_grid* g, double dt, int n_steps) {
         while (n_steps > 0) {
             const int chunk = std::min(n_steps, 1 << 16);
             bool ok = false;
-            BBX_CUDA(resident_pair_steps(g->model, g->d_t, g->nx, g->ny, chunk, g->d_err, g->stream, false, &ok, nullptr));
-            if (!ok) return BBX_ERR_STATE;
+            if (g->refuse || resident_pair_steps(g->model, g->d_t, g->nx, g->ny, chunk, g->d_err, g->stream, false, &ok,
+                                                 nullptr) != cudaSuccess || !ok) {
+                cudaGetLastError();  // not launchable after all: the tiled kernel from here on
+                g->pairs_ok = false;
+                break;
+            }
             ++g->launches[2];
+            g->stepped = true;
             n_steps -= chunk;
             g->h_cur ^= chunk & 1;
         }
-        g->stepped = true;
-        return BBX_OK;
+        if (n_steps == 0) return BBX_OK;
     }
     if (g->resident && n_steps >= 2 && g->route == BBX_ROUTE_AUTO && resident_eligible(g)) {
         int done = 0;
@@ -2201,7 +2212,7 @@ int bbx_step(bbx_grid* g, double dt, int n_steps) {
         while (n_steps >= flow_from) {
             const int m = std::min(n_steps, kFlowSteps);
             L.cur_hint = g->h_cur;
-            if (launch_flow(lpf, &L, m, g->stream) != cudaSuccess) {
+            if (g->refuse || launch_flow(lpf, &L, m, g->stream) != cudaSuccess) {
                 cudaGetLastError();  // not launchable as a whole: one launch per step from here on
                 lpf->flow = false;
                 break;
@@ -2976,7 +2987,18 @@ int batch_launch_step(bbx_batch* b, int n_steps = 1) {
         }
         BBX_CUDA(cudaStreamWaitEvent(gr.s, b->fork, 0));
         LaunchArgs L = launch_args(gr.lp, gr.d_t, b->d_err, 0);
-        BBX_CUDA(n_steps > 1 ? launch_flow(&gr.lp, &L, n_steps, gr.s) : launch(gr.lp, L, gr.s));
+        bool whole = n_steps > 1;
+        if (whole) {
+            for (int m : gr.members) whole = whole && !b->grids[(size_t)m]->refuse;
+            whole = whole && launch_flow(&gr.lp, &L, n_steps, gr.s) == cudaSuccess;
+        }
+        if (!whole) {
+            if (n_steps > 1) {  // not launchable as a whole: one launch a step from here on
+                cudaGetLastError();
+                b->flow = false;
+            }
+            for (int s = 0; s < n_steps; ++s) BBX_CUDA(launch(gr.lp, L, gr.s));
+        }
         BBX_CUDA(cudaEventRecord(gr.done, gr.s));
         BBX_CUDA(cudaStreamWaitEvent(b->ps, gr.done, 0));
     }
@@ -3066,7 +3088,7 @@ int bbx_batch_step(bbx_batch* b, int n_steps) {
         if (!g->model || !(g->dt > 0.0)) return BBX_ERR_STATE;
         if (g->version != b->versions[i]) b->built = false;  // a member changed since the batch was built
     }
-    int rc;
+    int rc = BBX_OK;
     if (!b->built && (rc = batch_build(b, nullptr))) return rc;
     // without shared launches: graphs of up to 16 steps
     const bool flow = b->flow && n_steps >= 2 && !capturing(b->stream);
@@ -3076,23 +3098,26 @@ int bbx_batch_step(bbx_batch* b, int n_steps) {
     BBX_CUDA(cudaEventRecord(b->enter, b->stream));
     BBX_CUDA(cudaStreamWaitEvent(b->ps, b->enter, 0));
     int done = 0;
-    if (flow) {
-        while (n_steps - done >= 2) {
-            const int m = std::min(n_steps - done, kFlowSteps);
-            if ((rc = batch_launch_step(b, m))) return rc;
-            done += m;
-        }
-    } else if (chunk >= 2) {
-        for (; done + chunk <= n_steps; done += chunk) BBX_CUDA(cudaGraphLaunch(b->gexec, b->ps));
+    while (flow && b->flow && rc == BBX_OK && n_steps - done >= 2) {
+        const int m = std::min(n_steps - done, kFlowSteps);
+        if ((rc = batch_launch_step(b, m)) == BBX_OK) done += m;
     }
-    for (; done < n_steps; ++done)
-        if ((rc = batch_launch_step(b))) return rc;
-    BBX_CUDA(cudaEventRecord(b->leave, b->ps));
-    BBX_CUDA(cudaStreamWaitEvent(b->stream, b->leave, 0));
+    while (chunk >= 2 && rc == BBX_OK && done + chunk <= n_steps) {
+        const cudaError_t e = cudaGraphLaunch(b->gexec, b->ps);
+        if (e == cudaSuccess) done += chunk;
+        else rc = fail_cuda(e);
+    }
+    while (rc == BBX_OK && done < n_steps)
+        if ((rc = batch_launch_step(b)) == BBX_OK) ++done;
+    // (after an error too: the steps that were enqueued are ordered and counted)
+    const cudaError_t e0 = cudaEventRecord(b->leave, b->ps);
+    const cudaError_t e1 = e0 == cudaSuccess ? cudaStreamWaitEvent(b->stream, b->leave, 0) : e0;
     for (bbx_grid* g : b->grids) {
-        g->stepped = true;
-        g->h_cur ^= n_steps & 1;  // every batch step flips every member's parity
+        g->stepped = g->stepped || done > 0;
+        g->h_cur ^= done & 1;  // every batch step flips every member's parity
     }
+    if (rc) return rc;
+    BBX_CUDA(e1);
     return BBX_OK;
 }
 

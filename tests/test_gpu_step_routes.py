@@ -150,3 +150,42 @@ def test_captured_one_step_launches_between_calls_of_several(bbx):
         s.synchronize()
         _same(A, B)
         assert A.debug_launches() == [2 + 12, 2, 0, 0]
+
+
+@pytest.mark.parametrize("kind", ["sheet", "slab"])
+def test_refused_launches_fall_back_to_one_launch_a_step(bbx, kind):
+    def make():
+        return (_sheet(bbx, 150, 120, "fhn"), 0.01) if kind == "sheet" else _block(bbx, "barkley", (16, 64, 64), "rotational", 14)
+
+    (A, dt), (B, _) = make(), make()
+    A.step(dt, 20)
+    A.debug_refuse_launches(True)
+    A.step(dt, 21)
+    A.debug_refuse_launches(False)
+    A.step(dt, 3)
+    _one_by_one(B, dt, 44)
+    _same(A, B)
+    k = 2 if kind == "sheet" else 1
+    assert A.debug_launches()[k] == 1 and sum(A.debug_launches()) == 25
+
+
+def test_refused_batch_launches_fall_back(bbx):
+    def make():
+        gs = [_sheet(bbx, nx, ny, "fhn", seed=nx) for nx, ny in ((70, 33), (64, 129), (200, 17))]
+        for g in gs:
+            g.set_timestep(0.01)
+        return gs, bbx.Batch(gs)
+
+    (ga, A), (gb, B) = make(), make()
+    ga[1].debug_refuse_launches(True)
+    for n in (5, 130, 1, 18):
+        A.step(n)
+        for _ in range(n):
+            B.step(1)
+    A.sync()
+    B.sync()
+    for a, b in zip(ga, gb):
+        _same(a, b)
+        assert a.get_time()[1] == 154
+    A.close()
+    B.close()
