@@ -2706,6 +2706,10 @@ int bbx_autotune(bbx_grid* g, double dt, double* best_ms) {
             if (z <= g->nz) zbs.push_back(z);
         if (g->nz > 64) zbs.push_back(g->nz);
     }
+    // A sheet whose longer calls run in a resident kernel, which has no tiles, is
+    // tuned for the calls that take them: one launch a step.
+    const int route0 = g->route;
+    if (g->pairs_ok || g->resident) g->route = BBX_ROUTE_STEPS;
     double best = 1e30;
     int bty = g->ty, bzb = g->zb;
     rc = BBX_OK;
@@ -2743,6 +2747,7 @@ int bbx_autotune(bbx_grid* g, double dt, double* best_ms) {
         }
         if (rc) break;
     }
+    g->route = route0;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     int rc2 = bbx_set_tiling(g, bty, bzb);

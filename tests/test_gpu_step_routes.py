@@ -189,3 +189,17 @@ def test_refused_batch_launches_fall_back(bbx):
         assert a.get_time()[1] == 154
     A.close()
     B.close()
+
+
+@pytest.mark.parametrize("nx,ny,resident", [(200, 200, False), (500, 500, False), (64, 64, True), (2100, 12, True)])
+def test_autotuning_times_the_tiles_of_a_resident_sheet(bbx, nx, ny, resident):
+    """The resident kernels have no tiles: tuned with them, the height would be left to chance."""
+    A = _sheet(bbx, nx, ny, "fhn")
+    if resident:
+        A.set_resident(True)
+    st = A.read_all()
+    assert A.autotune(0.01) > 0.0
+    assert A.debug_launches() == [3 * (2 + 6), 0, 0, 0]
+    assert np.array_equal(A.read_all(), st) and A.get_time() == (0.0, 0)
+    A.step(0.01, 20)
+    assert A.debug_launches()[0] == 24 and sum(A.debug_launches()) == 25
