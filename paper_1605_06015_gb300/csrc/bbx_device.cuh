@@ -2284,7 +2284,8 @@ struct StepKernel {
     int smem;
     int threads;
     int ty;
-    bool flow = false;  // may take several steps in one launch
+    bool flow = false;    // may take several steps in one launch
+    bool gather = false;  // its warps gather table entries together
 };
 
 }  // namespace bbx

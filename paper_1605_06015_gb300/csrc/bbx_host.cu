@@ -2712,6 +2712,7 @@ int bbx_autotune(bbx_grid* g, double dt, double* best_ms) {
     if (g->pairs_ok || g->resident) g->route = BBX_ROUTE_STEPS;
     double best = 1e30;
     int bty = g->ty, bzb = g->zb;
+    bool gathers7 = false;
     rc = BBX_OK;
     for (int ty : tys) {
         // 28 rows of an unmasked anisotropic light model leave one CTA per SM
@@ -2719,11 +2720,15 @@ int bbx_autotune(bbx_grid* g, double dt, double* best_ms) {
         // 400 against 345); on tissue at rest, which a grid often holds when it
         // is tuned, the difference can vanish in the memory's own scatter
         if (ty == 28 && !g->d_mask && g->aniso && g->S <= 2) continue;
-        // tables: 7 rows, whose warps gather entries together; 14 rows are faster
-        // only on tissue at rest, where every lane reads the same entry (in
-        // waves: 256x256x64 slab 140 us a step against 79, Markov model
-        // 181x428x43 188 against 128, 256^3 shell 144 against 104)
-        if (ty != 7 && reads_table(g)) continue;
+        // tables: 7 rows where their warps gather entries together (Plan::TABW); other
+        // heights are faster on sheets at rest at most (us a step with 7 / 14 rows,
+        // in waves: 256x256x64 slab 79 / 137, Markov sodium 127 / 276, calcium gate
+        // 88 / 123, 256^3 shell 106 / 155, 1024x1024 sheet 22.8 / 32.4; at rest 58 /
+        // 72, 75 / 95, 73 / 79, 96 / 101, 16.1 / 15.2).  The masked anisotropic
+        // kernels of eleven variables gather with 14 rows only, and which height is
+        // faster depends on the tissue (Markov sodium, 211x163x97 block in waves 187 /
+        // 173, 256^3 shell 266 / 275): both are timed.
+        if (ty != 7 && gathers7 && reads_table(g)) continue;
         for (int zb : zbs) {
             if ((rc = bbx_set_tiling(g, ty, zb)) != BBX_OK) {
                 if (rc == BBX_ERR_UNSUPPORTED) {
@@ -2732,6 +2737,7 @@ int bbx_autotune(bbx_grid* g, double dt, double* best_ms) {
                 }
                 break;
             }
+            if (ty == 7) gathers7 = g->lp.k.gather;
             if ((rc = bbx_step(g, dt, 2)) != BBX_OK) break;
             cudaEventRecord(e0, g->stream);
             if ((rc = bbx_step(g, dt, 6)) != BBX_OK) break;

@@ -7,7 +7,7 @@ template <bool MA, int AN, int TY, bool SU = false, bool PL = false, bool GE = f
 static StepKernel make_br() {
     using P = Plan<BBX_BR, MA, AN, TY, SU, GATES_F32, false, GE>;
     return StepKernel{reinterpret_cast<const void*>(&step_kernel<BBX_BR, MA, AN, TY, SU, PL, GE>), P::SMEM,
-                      P::THREADS, TY, P::FLOW};
+                      P::THREADS, TY, P::FLOW, P::TABW};
 }
 
 // planar: grids with nz = 1 (tiles marched along y); general: the variant

@@ -10,7 +10,7 @@ template <bool MA, int AN, int TY, bool PL, bool GE, int GA>
 static StepKernel make_br16() {
     using P = Plan<BBX_BR, MA, AN, TY, false, GA, false, GE>;
     return StepKernel{reinterpret_cast<const void*>(&step_kernel<BBX_BR, MA, AN, TY, false, PL, GE, GA>), P::SMEM,
-                      P::THREADS, TY, P::FLOW};
+                      P::THREADS, TY, P::FLOW, P::TABW};
 }
 
 template <bool MA, int AN, int TY, int GA>

@@ -9,7 +9,7 @@ template <bool MA, int AN, int TY, bool PL = false>
 static StepKernel make_br_mrl() {
     using P = Plan<BBX_BR_MRL, MA, AN, TY, false>;
     return StepKernel{reinterpret_cast<const void*>(&step_kernel<BBX_BR_MRL, MA, AN, TY, false, PL, false>),
-                      P::SMEM, P::THREADS, TY, P::FLOW};
+                      P::SMEM, P::THREADS, TY, P::FLOW, P::TABW};
 }
 
 // Tile rows 7 and 14 (the eleven variables make a 28-row stage too large for

@@ -203,3 +203,41 @@ def test_autotuning_times_the_tiles_of_a_resident_sheet(bbx, nx, ny, resident):
     assert np.array_equal(A.read_all(), st) and A.get_time() == (0.0, 0)
     A.step(0.01, 20)
     assert A.debug_launches()[0] == 24 and sum(A.debug_launches()) == 25
+
+
+@pytest.mark.parametrize("model,aniso,heights", [("mrl", True, 2), ("fca", True, 2), ("mrl", False, 1), ("br", True, 1)])
+def test_autotuning_of_tables_keeps_to_seven_rows_only_where_they_gather(bbx, model, aniso, heights):
+    """Masked anisotropic grids of eleven variables gather table entries with 14 rows and not with 7."""
+    from paper_1605_06015_gb300 import workloads as wl
+    nx, ny, nz = 70, 20, 8
+    mask, fib = wl.random_geometry(nx, ny, nz, 5, tissue_frac=0.7)
+    G = bbx.Grid(nx, ny, nz, 0.2, mask)
+    G.set_fibres(fib if aniso else None, 0.1, 0.025 if aniso else 0.1)
+    G.set_ionic_model({"mrl": bbx.BBX_BR_MRL, "fca": bbx.BBX_BR_FCA, "br": bbx.BBX_BR}[model])
+    if model == "br":
+        G.set_tabulation(True)
+    G.autotune(0.02)
+    assert G.debug_launches() == [heights * 2 * (2 + 6), 0, 0, 0]  # two depths (4, 8)
+
+
+@pytest.mark.parametrize("model", ["mrl", "fca"])
+def test_gathered_entries_of_a_masked_anisotropic_grid(bbx, model):
+    """14 rows (gathered) against 7 (each lane its own entries): the same entries, bitwise."""
+    from paper_1605_06015_gb300 import workloads as wl
+    nx, ny, nz = 130, 29, 5
+    mask, fib = wl.random_geometry(nx, ny, nz, 6, tissue_frac=0.7)
+    rng = np.random.default_rng(32)
+    st = rng.uniform(0.0, 1.0, (11, nz, ny, nx)).astype(np.float32)
+    st[0] = rng.uniform(-140.0, 100.0, (nz, ny, nx))  # (the table: -120 .. 80)
+    st[1] = 10 ** rng.uniform(-7.2, -5.2, (nz, ny, nx))
+    out = []
+    for ty in (7, 14):
+        G = bbx.Grid(nx, ny, nz, 0.2, mask)
+        G.set_fibres(fib, 0.1, 0.025)
+        G.set_tiling(ty, 4)
+        G.set_ionic_model(bbx.BBX_BR_MRL if model == "mrl" else bbx.BBX_BR_FCA)
+        G.write_all(st)
+        G.step(0.02, 1)
+        out.append(G.read_all()[:, mask != 0])
+    assert np.isfinite(out[0]).all()
+    assert np.array_equal(out[0], out[1])
