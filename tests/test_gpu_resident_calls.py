@@ -60,3 +60,30 @@ def test_other_buffer_holds_the_state_before_the_last_step(bbx, nx, ny, model, n
         got.append([bufs[cur].cpu().numpy(), bufs[cur ^ 1].cpu().numpy()])
     for a, b in zip(*got):
         assert np.array_equal(a.view(np.uint32), b.view(np.uint32))
+
+
+@pytest.mark.parametrize("nx,ny,model", [(2100, 17, "fhn"), (2051, 40, "zfk"), (150, 12, "barkley"), (2100, 15, "fhn"), (7, 8, "diffusion")])
+def test_sheets_in_shared_memory(bbx, nx, ny, model):
+    """Sheets that the registers' kernel does not take (more than 2048 columns; 8 to 15 rows, a
+    cluster of 8): the kernel in shared memory, to rounding as calls of one step."""
+    A, st = _sheet(bbx, nx, ny, model)
+    B, _ = _sheet(bbx, nx, ny, model)
+    reg = (np.random.default_rng(2).random((1, ny, nx)) < 0.3).astype(np.uint8)
+    for G in (A, B):
+        G.write_all(st)
+        G.set_threshold(0.5)
+        G.set_stimulus(reg, 4.0, 0.015, 0.04)
+    A.set_resident(True)
+    for n in (7, 2, 4):
+        A.step(0.01, n)
+        for _ in range(n):
+            B.step(0.01, 1)
+    assert A.debug_launches() == [0, 0, 0, 3]
+    a, b = A.read_all().astype(np.float64), B.read_all().astype(np.float64)
+    # a rounding (2^-24 of 1.5) in each of some ten operations a step, 13 steps
+    assert np.abs(a - b).max() <= 13 * 10 * 1.5 * 2.0 ** -24
+    ta, tb = A.read_activation().astype(np.int64), B.read_activation().astype(np.int64)
+    ta[ta == bbx.BBX_ACT_NONE] = tb[tb == bbx.BBX_ACT_NONE] = 14
+    assert np.abs(ta - tb).max() <= 1 and (tb < 14).any()
+    assert A.get_time() == B.get_time()
+    assert abs(A.step_total() - a[0].sum()) <= 1e-12 * np.abs(a[0]).sum()
