@@ -811,10 +811,11 @@ int build_plan(LaunchPlan* lp, const std::vector<Seg>& segs, int n_tissues, int 
                          (bx > 0 ? 1 : 0) | (bx + 1 < la.nbx ? 2 : 0) | (by > 0 ? 4 : 0) | (by + 1 < la.nby ? 8 : 0)};
             }
         std::vector<int> zero_flags((size_t)off[(size_t)n_tissues], 0);
-        if ((rc = upload(&lp->d_flags, &lp->cap_flags, zero_flags))) return rc;
-        if ((rc = upload(&lp->d_piece_flags, &lp->cap_pflags, pf))) return rc;
+        if ((rc = upload(&lp->d_flags, &lp->cap_flags, zero_flags)) == BBX_OK)
+            rc = upload(&lp->d_piece_flags, &lp->cap_pflags, pf);
+        if (rc && rc != BBX_ERR_NOMEM) return rc;
         lp->epoch = 0;
-        lp->flow = true;
+        lp->flow = rc == BBX_OK;  // (no room for the flags: one launch a step)
     }
     lp->cta_stride = stride;
     lp->n_slots = (int)nslot;
@@ -1455,7 +1456,9 @@ int prepare(bbx_grid* g) {
         if (nodes < kFlowNodes) {
             if (g->flow_from) {
                 g->lpf.k = kf;
-                if ((rc = build_plan(&g->lpf, segs, 1, ctas, lattice, g->device))) return rc;
+                rc = build_plan(&g->lpf, segs, 1, ctas, lattice, g->device);
+                if (rc && rc != BBX_ERR_NOMEM) return rc;
+                if (rc) g->flow_from = 0;  // (no room for a second plan: one launch a step)
             }
             if ((rc = pick(false, &g->lp.k, &ctas))) return rc;
             lattice.clear();
