@@ -638,6 +638,9 @@ struct Seg {
     int tissue, x0, y0, z0, z1;
 };
 
+// (bbx_grid's plans)
+constexpr long long kFlowSheetMin = 250000, kFlowNodesLarge = 15000000;
+
 struct LaunchPlan {
     StepKernel k = {nullptr, 0, 0, 0};
     int ctas = 0;
@@ -929,10 +932,13 @@ cudaError_t launch(const LaunchPlan& lp, const LaunchArgs& L, cudaStream_t s) {
 // of the done flags (3 us), or the CTAs wait for one another every step.
 // Measured (us a step, one launch a step / several steps a launch, the best
 // tile height of each):
-// - 3 million nodes or more, share of 5 to 500 planes: never slower than the
-//   kernels of one step a launch were before, from n = 2 on (256x256x64 slab
-//   n = 2 26.3 / 25.7, n = 10 26.3 / 22.1; 192^3 n = 2 28.1 / 27.3; 8192x8192
-//   n = 4 200 / 201, n = 10 200 / 189);
+// - from 25 million nodes on a launch's own cost is little and the first step of
+//   several, which has no launch before it to overlap with, weighs: 8192x8192 n =
+//   2 200 / 210, n = 4 200 / 201, n = 10 200 / 189; 512x512x128 n = 4 96 / 100, n
+//   = 10 96 / 94; without W-tilde sums 512x512x128 n = 4 154 / 162, n = 10 154 / 155;
+// - from 3 million on: 256x256x64 slab n = 2 26.3 / 25.7, n = 10 26.3 / 22.1;
+//   192^3 n = 2 28.1 / 27.3; 400x400x100 n = 2 59.6 / 56.9, n = 10 59.5 / 50.9;
+//   3000x5000 n = 2 48.6 / 48.4, n = 3 48.6 / 45.8;
 // - fewer, with long shares: 128^3 anisotropic, 16 planes n = 3 16.2 / 16.0;
 //   isotropic, 11 planes n = 6 13.3 / 13.6, n = 10 13.3 / 13.1; 1500x1500 and
 //   1400x1400, 3 to 14 planes, n = 10 12.0 / 12.1, n = 20 11.9 / 11.5;
@@ -943,7 +949,8 @@ cudaError_t launch(const LaunchPlan& lp, const LaunchArgs& L, cudaStream_t s) {
 //   n = 20 6.8 / 7.0), blocks (80 CTAs n = 6 7.1 / 7.1, 192 n = 10 8.0 / 7.6, 320
 //   n = 20 8.8 / 8.2).
 constexpr long long kFlowNodes = 3000000, kFlowNodesMin = 1500000;
-int flow_steps_from(long long nodes, long long planes, int ctas, int num_sms, bool planar) {
+int flow_steps_from(long long nodes, long long planes, int ctas, int num_sms, bool planar, bool no_sums) {
+    if (nodes >= 25000000) return no_sums ? 10 : 4;
     if (nodes >= kFlowNodes) return 2;
     if (planes <= ctas) {
         if (planar) return planes <= num_sms ? 4 + (int)planes / 8 : 0;
@@ -1046,11 +1053,15 @@ struct bbx_grid {
     TissueArgs h_t;                // host copy of the kernel's view of this grid
     TissueArgs* d_t = nullptr;     // device copy
     TissueDyn* d_dyn = nullptr;    // device-updated time, step, parity, total
-    // lp: one step a launch, and several of grids with kFlowNodes nodes or more;
-    // lpf: several steps a launch of smaller grids, in calls of flow_from steps or
-    // more (the kernels without the sync warp, four CTAs an SM instead of three
-    // when isotropic, are the faster ones at one step a launch there: 400x400 6.5 us
-    // against 7.3, 128^3 13.3 against 14.4)
+    // lp: one step a launch; lpf: several, in calls of flow_from steps or more.  The
+    // kernels without the sync warp, four CTAs an SM instead of three when
+    // isotropic, are the faster ones at one step a launch of small and of large
+    // grids (400x400 6.5 us against 7.0, 128^3 13.3 against 13.6, 3000x5000 48.6 /
+    // 50.8, 512x512x256 184 / 202); from kFlowNodes nodes to kFlowNodesLarge, on
+    // isotropic sheets already from kFlowSheetMin, and where they have no variant
+    // without W-tilde sums, lp serves both (192^3 28.2 / 26.5, 4096x2048 27.7 / 27.4,
+    // 256x256x100 26.5 / 25.5, 512x512 6.5 / 6.2, 700x900 8.9 / 7.6, 1500x1500 11.9 /
+    // 10.4; 256x256x64 18.1 / 18.4).
     LaunchPlan lp, lpf;
     int flow_from = 0;
     bool ready = false;            // h_t, d_t and lp match the current settings
@@ -1425,11 +1436,13 @@ int prepare(bbx_grid* g) {
     if (rc0 || (rc0 = tab_refresh(g))) return rc0;
     BBX_CUDA(cudaStreamSynchronize(g->stream));
     const bool surr = g->surr_on && g->model == BBX_BR;
+    bool no_sums = false;  // picked: the variant without W-tilde sums
     auto pick = [&](bool flow, StepKernel* k, int* ctas) {
         int r = BBX_ERR_UNSUPPORTED;
         if (g->aniso && g->wsum_zero && g->wsum_elide && !g->d_mask)  // the variant without W-tilde sums, if built
             r = select_kernel(g->model, false, AN_NO_SUMS, g->ty, g->device, g->num_sms, k, ctas, surr, g->nz == 1,
                               wants_general(g), g->gates, flow);
+        no_sums = r == BBX_OK;
         if (r == BBX_ERR_UNSUPPORTED)
             r = select_kernel(g->model, g->d_mask != nullptr, g->aniso ? AN_SUMS : AN_ISO, g->ty, g->device,
                               g->num_sms, k, ctas, surr, g->nz == 1, wants_general(g), g->gates, flow);
@@ -1445,27 +1458,6 @@ int prepare(bbx_grid* g) {
     grid_segments(g, kf.ty, 0, &segs);
     std::vector<Lattice> lattice;
     if (!g->d_mask) lattice.push_back(grid_lattice(g, kf.ty));
-    g->flow_from = 0;
-    g->lp.k = kf;
-    if (kf.flow && !g->d_mask) {
-        const long long nodes = (long long)g->nx * g->ny * (g->nz - g->halo_lo - g->halo_hi);
-        long long planes = 0;
-        for (const Seg& sg : segs) planes += sg.z1 - sg.z0;
-        g->flow_from = flow_steps_from(nodes, planes, ctas, g->num_sms, g->nz == 1);
-        if (g->flow_from == 0 && g->route >= BBX_ROUTE_SEVERAL) g->flow_from = INT_MAX;  // (only asked for)
-        if (nodes < kFlowNodes) {
-            if (g->flow_from) {
-                g->lpf.k = kf;
-                rc = build_plan(&g->lpf, segs, 1, ctas, lattice, g->device);
-                if (rc && rc != BBX_ERR_NOMEM) return rc;
-                if (rc) g->flow_from = 0;  // (no room for a second plan: one launch a step)
-            }
-            if ((rc = pick(false, &g->lp.k, &ctas))) return rc;
-            lattice.clear();
-        }
-    }
-    if (!g->flow_from || !lattice.empty()) g->lpf.release();
-    if ((rc = build_plan(&g->lp, segs, 1, ctas, lattice, g->device))) return rc;
     g->pairs_ok = false;
     if (resident_shape(g)) {
         bool ok = false;
@@ -1475,6 +1467,30 @@ int prepare(bbx_grid* g) {
         else
             g->pairs_ok = ok;
     }
+    g->flow_from = 0;
+    g->lp.k = kf;
+    if (kf.flow && !g->d_mask) {
+        const long long nodes = (long long)g->nx * g->ny * (g->nz - g->halo_lo - g->halo_hi);
+        long long planes = 0;
+        for (const Seg& sg : segs) planes += sg.z1 - sg.z0;
+        g->flow_from = flow_steps_from(nodes, planes, ctas, g->num_sms, g->nz == 1, no_sums);
+        if (g->pairs_ok && g->pairs_from <= g->flow_from) g->flow_from = 0;  // (those calls run in registers)
+        if (g->flow_from == 0 && g->route >= BBX_ROUTE_SEVERAL) g->flow_from = INT_MAX;  // (only asked for)
+        const bool one_kernel = nodes >= kFlowNodes ? nodes < kFlowNodesLarge || no_sums
+                                                    : nodes >= kFlowSheetMin && g->nz == 1 && !g->aniso;
+        if (!one_kernel) {
+            if (g->flow_from) {
+                g->lpf.k = kf;
+                rc = build_plan(&g->lpf, segs, 1, ctas, lattice, g->device);
+                if (rc && rc != BBX_ERR_NOMEM) return rc;
+                if (rc) g->flow_from = 0;  // (no room for a second plan: one launch a step)
+            }
+            if ((rc = pick(false, &g->lp.k, &ctas))) return rc;
+        }
+        if (!one_kernel || !g->flow_from) lattice.clear();
+    }
+    if (!g->flow_from || !lattice.empty()) g->lpf.release();
+    if ((rc = build_plan(&g->lp, segs, 1, ctas, lattice, g->device))) return rc;
     BBX_CUDA(cudaStreamSynchronize(g->stream));
     g->ready = true;
     return BBX_OK;
