@@ -147,8 +147,9 @@ typedef struct {
  * .bbg status flag, section "Format of BeatBox geometry files"); nodes outside
  * the array are void.  cuda_stream: a cudaStream_t (NULL = legacy default).
  * Idle bricks (no tissue) are elided (section "Domain partitioning").
- * Allocates device memory for the mask and the brick list; the caller keeps
- * its buffer.  Errors: BBX_ERR_ARG (null out, nonpositive size or h,
+ * Allocates device memory for the mask (5 bytes a node of the box: its flags,
+ * and the step's word of each node's neighbours) and the brick list; the
+ * caller keeps its buffer.  Errors: BBX_ERR_ARG (null out, nonpositive size or h,
  * nx*ny*nz >= 2^31), BBX_ERR_NOMEM, BBX_ERR_CUDA. */
 int bbx_create_grid(bbx_grid** out, int nx, int ny, int nz, double h, const uint8_t* mask_host,
                     void* cuda_stream);

@@ -427,9 +427,8 @@ __device__ __forceinline__ void grid_piece_done(const LaunchArgs& L, int pi, int
 // producers advance t, n and the parity as soon as every CTA has read them
 // (start_ticket), and the grid's total is summed from the partials when it
 // is asked for.
-__device__ __forceinline__ void step_finalize(const LaunchArgs& L, double* scratch32) {
+__device__ __forceinline__ void step_finalize(const LaunchArgs& L) {
     __shared__ bool last;
-    (void)scratch32;
     if (L.single || L.n_empty == 0) return;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -666,10 +665,14 @@ __device__ __forceinline__ void tab_entry(const float4* __restrict__ tab, float 
 // these loads: where V differs from node to node, a lane reading its own
 // node's entries takes eight loads of 32 separate lines, this eight loads of
 // eight 64-byte segments, and half as many wavefronts again for the exchange.
-// In waves (V different everywhere): 256x256x64 slab 113 -> 78 us a step, with
-// 16-bit gates 110 -> 75, 256^3 shell 129 -> 110, with 16-bit gates 129 -> 104.
-// Where the warp's V lie within a few entries (tissue near rest) each lane
-// reads its own: its loads are then a line or two for the whole warp.
+// In waves (V different everywhere), each lane its own entries / gathered, us a
+// step: 256x256x64 slab 104 / 79, Markov sodium 197 / 128, 256^3 shell 131 / 106,
+// with 16-bit gates 127 / 104, 1024x1024 sheet 30.7 / 23.1.  Where the warp's V
+// lie within a few entries (tissue at rest) each lane reads its own: its loads
+// are then a line or two for the whole warp (slab at rest gathered 68, so 58;
+// Markov sodium 103 and 75).  A slab at rest but for one front is slower with
+// it, 63 / 66, with 16-bit gates 55 / 60: few warps look up, and each waits for
+// two exchanges (with a cold L2 72 / 80 and 65 / 76, Markov sodium 117 / 127).
 __device__ __forceinline__ void tab_entry_warp(const float4* __restrict__ tab, float V, float4* buf, float* c) {
     const int lane = threadIdx.x & 31, p = lane & 3;
     float w;
@@ -1097,10 +1100,11 @@ struct Model<BBX_BR_FCA> {
 constexpr int kTileX = 64;  // nodes per brick along x: 32 threads x 2 nodes
 // Several steps in one launch (FLOW variants): unmasked grids of the light
 // models (the others' steps are long next to a launch, and the further warp it
-// takes would cost the registers their consumers need).  The same grids in a
-// batch of several kernel types run the variants without the sync warp, one
-// launch a step: four CTAs per SM instead of three when isotropic (192 sheets
-// and 64 blocks 337 us a step against 365).
+// takes would cost the registers their consumers need).  The same grids run the
+// variants without the sync warp at one launch a step where that is faster (in
+// a batch of several kernel types, and by size when alone: bbx_grid's plans):
+// four CTAs per SM instead of three when isotropic (192 sheets and 64 blocks 337
+// us a step against 365).
 __host__ __device__ constexpr bool has_flow(bool masked, int s) { return !masked && s <= 2; }
 // Consumer warps per CTA (plus the producer warp, plus the sync warp) for a
 // tile of TY rows: 7 warps of 1 or 2 rows each for TY = 7, 14; for 28 rows 7
@@ -1225,8 +1229,8 @@ struct Plan {
     // ring B and leaves the rest to the L1 cache (Markov model, 181x428x43
     // slab: 204 us a step with four, 155 with three); its warps gather
     // together (tab_entry_warp) where their buffers cost none of these stages
-    // (256^3 tabulated shell: 110 us, 132 with two, 129 without the buffers
-    // and four).
+    // (256^3 tabulated shell, when it was chosen: 110 us, 132 with two stages, 129
+    // with four and without the buffers).
     static constexpr bool TAB = MODEL == BBX_BR_MRL || MODEL == BBX_BR_FCA || (MODEL == BBX_BR && GEN && !SURR);
     static constexpr int NB_TAB = ROOM >= 3 * B_STAGE + 5 * A_STAGE ? 3 : 2;
     static constexpr int TABW_BYTES = RY * 2048 + 2048;  // (2 KB: barriers and piece contexts)
@@ -1586,7 +1590,7 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((128u - (smem_addr(smem_raw) & 127u)) & 127u);
     unsigned char* bstages = smem + NS * P::A_STAGE;    // ring B
-    unsigned char* wbufs = bstages + NB * P::B_STAGE;   // surrogate buffers (SURR only)
+    unsigned char* wbufs = bstages + NB * P::B_STAGE;   // per consumer warp: the surrogate's, or table entries'
     PieceSlot* ring = reinterpret_cast<PieceSlot*>(smem + P::RING_OFF);
     // full (the copies have landed) and empty (the consumer warps are done)
     // barriers of a stage of ring A and of ring B
@@ -2042,11 +2046,11 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
                 const bool zn_ok = k + 1 < nz, zp_ok = k > 0;
                 const int nrows = ny - yb;  // rows of this thread inside the array
                 const float ncz = MASKED || (zn_ok && zp_ok) ? -2.0f : (zn_ok || zp_ok ? -1.0f : 0.0f);
-                // unmasked: some cross difference misses a neighbour on one side only (a row or plane at
-                // the array's border)
                 // unmasked: this thread's rows touch the array's border in y
                 const bool yborder = !MASKED && (yb == 0 || nrows <= CY);
                 const float2 ncp = add2(ncx, splat2(-2.0f + (PLANAR ? 0.0f : ncz)));  // (isotropic: all axes)
+                // unmasked: some cross difference misses a neighbour on one side only (a row or plane at
+                // the array's border)
                 const bool border = !MASKED && ANISO && (yborder || (!PLANAR && !(zn_ok && zp_ok)));
 
                 // Sliding window down the rows: plane k at x-1..x+2, the own pair of planes k+-1.
@@ -2275,7 +2279,7 @@ step_kernel(const __grid_constant__ LaunchArgs L) {
         for (int j = issuedb > NB ? issuedb - NB : 0; j < issuedb; ++j)
             (void)mbar_wait_bounded(fullb(j % NB), (j / NB) & 1, L.wait_limit);
     }
-    step_finalize(L, red_scratch);
+    step_finalize(L);
 }
 
 // host-visible description of one compiled step kernel

@@ -2175,7 +2175,7 @@ int bbx_step(bbx_grid* g, double dt, int n_steps) {
          (g->route == BBX_ROUTE_AUTO && (g->resident || n_steps >= g->pairs_from)))) {
         // a sheet that fits, in a call long enough (or where it was asked for): all
         // its steps in one cluster's registers and shared memory (200^2, 20 steps a
-        // call: 1.6 us a step against 4.7 by tiles; 200 steps: 1.1 us), the same results
+        // call: 1.6 us a step against 4.8 by tiles; 200 steps: 1.1 us), the same results
         while (n_steps > 0) {
             const int chunk = std::min(n_steps, 1 << 16);
             bool ok = false;
@@ -2735,9 +2735,10 @@ int bbx_autotune(bbx_grid* g, double dt, double* best_ms) {
     rc = BBX_OK;
     for (int ty : tys) {
         // 28 rows of an unmasked anisotropic light model leave one CTA per SM
-        // (256x256x64 slab 34 us a step against 22.8 with 14 rows, 512x512x256
-        // 400 against 345); on tissue at rest, which a grid often holds when it
-        // is tuned, the difference can vanish in the memory's own scatter
+        // (256x256x64 slab 29.7 us a step against 26 with 14 rows, in calls of 20
+        // steps 27.4 against 21.3; 512x512x256 305 against 306, 310 against 301); on
+        // tissue at rest, which a grid often holds when it is tuned, the difference
+        // can vanish in the memory's own scatter
         if (ty == 28 && !g->d_mask && g->aniso && g->S <= 2) continue;
         // tables: 7 rows where their warps gather entries together (Plan::TABW); other
         // heights are faster on sheets at rest at most (us a step with 7 / 14 rows,

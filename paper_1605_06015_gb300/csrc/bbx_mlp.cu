@@ -43,8 +43,8 @@ __device__ __forceinline__ long long sample_row(long long i, long long n, unsign
 // (12) floats, so that eight lanes' float4 of eight rows touch every bank once.  Each
 // sum keeps its order (over inputs, outputs or samples ascending, from the
 // bias or 0), so results are bitwise those of one output at a time.
-// A step of 4096 samples: 84 us before, 21 by tiles, about 14 with the weights'
-// loads all in flight at once.
+// A step of 4096 samples: 84 us before, 21 by tiles, 13 with the weights' loads
+// all in flight at once.
 constexpr int kW1P = 12, kW2P = 68;  // padded row lengths
 constexpr int kSmW1 = 0, kSmW2 = kSmW1 + 64 * kW1P, kSmW3 = kSmW2 + 64 * kW2P, kSmB1 = kSmW3 + 8 * kW2P,
               kSmB2 = kSmB1 + 64, kSmB3 = kSmB2 + 64, kSmX = kSmB3 + 8, kSmDy = kSmX + kSB * 8,

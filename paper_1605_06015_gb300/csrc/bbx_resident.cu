@@ -43,7 +43,7 @@ __global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(kResThreads, 1)
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
     extern __shared__ float sm[];
-    __shared__ double red_hi[kResThreads / 32], red_lo[kResThreads / 32];
+    __shared__ double red_hi[kResThreads / 32];
     __shared__ double cl_part[NC];
 
     const int nx = T->nx, ny = T->ny, px = T->px;
@@ -143,7 +143,6 @@ __global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(kResThreads, 1)
         double* root = cl.map_shared_rank(cl_part, 0);
         root[rank] = b;
     }
-    (void)red_lo;
     cl.sync();
     if (rank == 0 && threadIdx.x == 0) {
         double tot = 0.0;
@@ -230,14 +229,13 @@ __host__ __device__ __forceinline__ int row_warps(int np, int R, int r) {
 
 constexpr int kPairPad = 4;  // zero columns of a V row: two before x = 0, two after the last pair
 constexpr int kPairMaxSmem = 220 * 1024;
-template <int MODEL>
 __host__ __device__ constexpr bool pair_regs(int R) { return R <= 4; }
 
 template <int MODEL, int NC, int R>
 __global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(kResThreads, 1)
     k_resident_pairs(const TissueArgs* __restrict__ T, int n_steps, int* __restrict__ err, long long wait_limit) {
     constexpr int S = Model<MODEL>::S;
-    constexpr bool VREG = pair_regs<MODEL>(R);
+    constexpr bool VREG = pair_regs(R);
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
     extern __shared__ float sm[];
@@ -490,7 +488,7 @@ cudaError_t pairs_try(const TissueArgs* d_t, int nx, int ny, int n_steps, int* d
                       bool* ok, int* from) {
     const int np = (nx + 1) / 2, maxr = (ny + NC - 1) / NC, pitch = 2 * np + kPairPad;
     const size_t smem = sizeof(float) * (2 * (size_t)(maxr + 2) * pitch +
-                                         (pair_regs<MODEL>(R) ? 0 : (size_t)(Model<MODEL>::S - 1) * maxr * 2 * np));
+                                         (pair_regs(R) ? 0 : (size_t)(Model<MODEL>::S - 1) * maxr * 2 * np));
     *ok = false;
     if (smem > (size_t)kPairMaxSmem || ny < NC) return cudaSuccess;
     cudaLaunchConfig_t cfg = {};
