@@ -378,7 +378,8 @@ int bbx_set_tiling(bbx_grid* g, int tile_y, int tile_z);
  * steps each, state restored afterwards) and keep the fastest.  best_ms (may
  * be NULL) receives its time per step.  Sheets that a resident kernel takes in
  * longer calls (bbx_set_resident), which has no bricks, are timed at one
- * launch a step. */
+ * launch a step; so are grids whose longer calls take several steps a launch
+ * in a plan of their own, whose tile rows are then chosen by themselves. */
 int bbx_autotune(bbx_grid* g, double dt, double* best_ms);
 
 /* Set the time step used by bbx_batch_step (bbx_step sets it too).  Errors:

@@ -925,7 +925,8 @@ cudaError_t launch(const LaunchPlan& lp, const LaunchArgs& L, cudaStream_t s) {
     return cudaLaunchKernelExC(&cfg, lp.k.fn, args);
 }
 
-// From how many steps of a call a grid takes several steps a launch (0: never).
+// From how many steps of a call a grid takes several steps a launch (0: never),
+// where bbx_autotune has not measured it.
 // A launch of several steps costs 5 us more than one of one step (20 us where a
 // step takes 200) and saves each further step the fill and drain of a launch,
 // 2 to 8 us; but a CTA's share of a step has to be long against the round trips
@@ -958,7 +959,7 @@ int flow_steps_from(long long nodes, long long planes, int ctas, int num_sms, bo
     }
     if (nodes < kFlowNodesMin) return 0;
     const long long share = planes / ctas;
-    return share >= 15 ? 3 : (share >= 8 ? 10 : 20);
+    return share >= 15 ? 3 : 20;
 }
 
 // Select the kernel for a configuration, check it fits, and return the CTA
@@ -1051,6 +1052,7 @@ struct bbx_grid {
     std::vector<uint8_t> h_chunks;  // masked 3D grids: tissue flag of each 16-wide chunk of each brick band
 
     TissueArgs h_t;                // host copy of the kernel's view of this grid
+    TissueArgs h_tf;               // the same for lpf's tile rows
     TissueArgs* d_t = nullptr;     // device copy
     TissueDyn* d_dyn = nullptr;    // device-updated time, step, parity, total
     // lp: one step a launch; lpf: several, in calls of flow_from steps or more.  The
@@ -1064,6 +1066,9 @@ struct bbx_grid {
     // 10.4; 256x256x64 18.1 / 18.4).
     LaunchPlan lp, lpf;
     int flow_from = 0;
+    bool two_plans = false;
+    int ty_flow = 0;  // lpf's tile rows (0: lp's) and flow_from (0: flow_steps_from, INT_MAX: never), by bbx_autotune
+    int flow_measured = 0;
     bool ready = false;            // h_t, d_t and lp match the current settings
     unsigned long long version = 1;  // bumped whenever the kernel's view changes
 
@@ -1427,7 +1432,70 @@ bool resident_shape(const bbx_grid* g) {
            (g->model == BBX_FHN || g->model == BBX_BARKLEY || g->model == BBX_ZFK || g->model == BBX_DIFFUSION);
 }
 
-// Bring h_t, d_t and the single-grid launch plan in line with the settings.
+// Nodes a step computes.
+long long own_nodes(const bbx_grid* g) { return (long long)g->nx * g->ny * (g->nz - g->halo_lo - g->halo_hi); }
+
+// The step kernel of a grid for `ty` tile rows (flow: the variant that may take
+// several steps in one launch, where there is one) and its CTA budget; no_sums:
+// it is the variant without W-tilde sums.
+int pick_kernel(const bbx_grid* g, int ty, bool flow, StepKernel* k, int* ctas, bool* no_sums) {
+    const bool surr = g->surr_on && g->model == BBX_BR;
+    int r = BBX_ERR_UNSUPPORTED;
+    if (g->aniso && g->wsum_zero && g->wsum_elide && !g->d_mask)  // the variant without W-tilde sums, if built
+        r = select_kernel(g->model, false, AN_NO_SUMS, ty, g->device, g->num_sms, k, ctas, surr, g->nz == 1,
+                          wants_general(g), g->gates, flow);
+    *no_sums = r == BBX_OK;
+    if (r == BBX_ERR_UNSUPPORTED)
+        r = select_kernel(g->model, g->d_mask != nullptr, g->aniso ? AN_SUMS : AN_ISO, ty, g->device, g->num_sms, k,
+                          ctas, surr, g->nz == 1, wants_general(g), g->gates, flow);
+    return r;
+}
+
+// The plan for several steps a launch of a grid whose one-step launches have
+// their own (g->two_plans), and from how many steps of a call it is taken.
+int prepare_flow(bbx_grid* g) {
+    g->flow_from = 0;
+    g->lpf.flow = false;
+    if (!g->two_plans) {
+        g->lpf.release();
+        return BBX_OK;
+    }
+    int ctas = 0;
+    bool no_sums = false;
+    StepKernel k;
+    int rc = pick_kernel(g, g->ty_flow ? g->ty_flow : g->ty, true, &k, &ctas, &no_sums);
+    if (rc == BBX_ERR_UNSUPPORTED) rc = pick_kernel(g, g->ty, true, &k, &ctas, &no_sums);
+    if (rc) return rc;
+    std::vector<Seg> segs;
+    grid_segments(g, k.ty, 0, &segs);
+    long long planes = 0;
+    for (const Seg& sg : segs) planes += sg.z1 - sg.z0;
+    g->flow_from = g->flow_measured ? (g->flow_measured < INT_MAX ? g->flow_measured : 0)
+                                    : flow_steps_from(own_nodes(g), planes, ctas, g->num_sms, g->nz == 1, no_sums);
+    if (g->pairs_ok && g->pairs_from <= g->flow_from) g->flow_from = 0;  // (those calls run in registers)
+    if (g->flow_from == 0 && g->route >= BBX_ROUTE_SEVERAL) g->flow_from = INT_MAX;  // (only asked for)
+    if (g->flow_from == 0) {
+        g->lpf.release();
+        return BBX_OK;
+    }
+    if ((rc = encode_targs(g, k.ty, &g->h_tf))) return rc;
+    g->lpf.k = k;
+    rc = build_plan(&g->lpf, segs, 1, ctas, {grid_lattice(g, k.ty)}, g->device);
+    if (rc != BBX_ERR_NOMEM) return rc;
+    g->lpf.release();  // (no room for a second plan: one launch a step)
+    g->flow_from = 0;
+    return BBX_OK;
+}
+
+// The same for other tile rows (g->ty_flow) of a prepared grid.
+int replan_flow(bbx_grid* g) {
+    const int rc = finish_total(g);  // the plan's partials are about to be replaced
+    if (rc) return rc;
+    BBX_CUDA(cudaStreamSynchronize(g->stream));
+    return prepare_flow(g);
+}
+
+// Bring h_t, d_t and the single-grid launch plans in line with the settings.
 int prepare(bbx_grid* g) {
     g->ready = false;
     ++g->version;
@@ -1435,29 +1503,15 @@ int prepare(bbx_grid* g) {
     int rc0 = finish_total(g);  // the plan's partials are about to be replaced
     if (rc0 || (rc0 = tab_refresh(g))) return rc0;
     BBX_CUDA(cudaStreamSynchronize(g->stream));
-    const bool surr = g->surr_on && g->model == BBX_BR;
-    bool no_sums = false;  // picked: the variant without W-tilde sums
-    auto pick = [&](bool flow, StepKernel* k, int* ctas) {
-        int r = BBX_ERR_UNSUPPORTED;
-        if (g->aniso && g->wsum_zero && g->wsum_elide && !g->d_mask)  // the variant without W-tilde sums, if built
-            r = select_kernel(g->model, false, AN_NO_SUMS, g->ty, g->device, g->num_sms, k, ctas, surr, g->nz == 1,
-                              wants_general(g), g->gates, flow);
-        no_sums = r == BBX_OK;
-        if (r == BBX_ERR_UNSUPPORTED)
-            r = select_kernel(g->model, g->d_mask != nullptr, g->aniso ? AN_SUMS : AN_ISO, g->ty, g->device,
-                              g->num_sms, k, ctas, surr, g->nz == 1, wants_general(g), g->gates, flow);
-        return r;
-    };
-    StepKernel kf;
+    bool no_sums = false;
+    StepKernel k;
     int ctas = 0;
-    int rc = pick(true, &kf, &ctas);
+    int rc = pick_kernel(g, g->ty, true, &k, &ctas, &no_sums);
     if (rc) return rc;
-    if ((rc = encode_targs(g, kf.ty, &g->h_t))) return rc;
+    if ((rc = encode_targs(g, k.ty, &g->h_t))) return rc;
     BBX_CUDA(cudaMemcpyAsync(g->d_t, &g->h_t, sizeof(TissueArgs), cudaMemcpyHostToDevice, g->stream));
     std::vector<Seg> segs;
-    grid_segments(g, kf.ty, 0, &segs);
-    std::vector<Lattice> lattice;
-    if (!g->d_mask) lattice.push_back(grid_lattice(g, kf.ty));
+    grid_segments(g, k.ty, 0, &segs);
     g->pairs_ok = false;
     if (resident_shape(g)) {
         bool ok = false;
@@ -1467,29 +1521,22 @@ int prepare(bbx_grid* g) {
         else
             g->pairs_ok = ok;
     }
-    g->flow_from = 0;
-    g->lp.k = kf;
-    if (kf.flow && !g->d_mask) {
-        const long long nodes = (long long)g->nx * g->ny * (g->nz - g->halo_lo - g->halo_hi);
+    const long long nodes = own_nodes(g);
+    const bool light = k.flow && !g->d_mask;
+    g->two_plans = light && (nodes >= kFlowNodes ? nodes >= kFlowNodesLarge && !no_sums
+                                                 : nodes < kFlowSheetMin || g->nz > 1 || g->aniso);
+    if ((rc = prepare_flow(g))) return rc;
+    std::vector<Lattice> lattice;
+    if (g->two_plans) {
+        if ((rc = pick_kernel(g, g->ty, false, &k, &ctas, &no_sums))) return rc;
+    } else if (light) {
         long long planes = 0;
         for (const Seg& sg : segs) planes += sg.z1 - sg.z0;
         g->flow_from = flow_steps_from(nodes, planes, ctas, g->num_sms, g->nz == 1, no_sums);
-        if (g->pairs_ok && g->pairs_from <= g->flow_from) g->flow_from = 0;  // (those calls run in registers)
         if (g->flow_from == 0 && g->route >= BBX_ROUTE_SEVERAL) g->flow_from = INT_MAX;  // (only asked for)
-        const bool one_kernel = nodes >= kFlowNodes ? nodes < kFlowNodesLarge || no_sums
-                                                    : nodes >= kFlowSheetMin && g->nz == 1 && !g->aniso;
-        if (!one_kernel) {
-            if (g->flow_from) {
-                g->lpf.k = kf;
-                rc = build_plan(&g->lpf, segs, 1, ctas, lattice, g->device);
-                if (rc && rc != BBX_ERR_NOMEM) return rc;
-                if (rc) g->flow_from = 0;  // (no room for a second plan: one launch a step)
-            }
-            if ((rc = pick(false, &g->lp.k, &ctas))) return rc;
-        }
-        if (!one_kernel || !g->flow_from) lattice.clear();
+        if (g->flow_from) lattice.push_back(grid_lattice(g, k.ty));
     }
-    if (!g->flow_from || !lattice.empty()) g->lpf.release();
+    g->lp.k = k;
     if ((rc = build_plan(&g->lp, segs, 1, ctas, lattice, g->device))) return rc;
     BBX_CUDA(cudaStreamSynchronize(g->stream));
     g->ready = true;
@@ -1503,15 +1550,17 @@ int refresh_targs(bbx_grid* g) {
     int rc = tab_refresh(g);
     if (rc) return rc;
     ++g->version;
-    g->h_t.t_on = g->t_on;
-    g->h_t.t_off = g->t_off;
-    g->h_t.dt_d = g->dt;
-    g->h_t.dt = (float)g->dt;
-    g->h_t.theta = (float)g->theta;
-    g->h_t.split = g->split;
-    g->h_t.rk4 = g->rk4;
-    g->h_t.stim = g->d_stim;
-    g->h_t.stim_amp = g->d_stim ? (float)g->stim_amp : 0.0f;
+    for (TissueArgs* t : {&g->h_t, &g->h_tf}) {
+        t->t_on = g->t_on;
+        t->t_off = g->t_off;
+        t->dt_d = g->dt;
+        t->dt = (float)g->dt;
+        t->theta = (float)g->theta;
+        t->split = g->split;
+        t->rk4 = g->rk4;
+        t->stim = g->d_stim;
+        t->stim_amp = g->d_stim ? (float)g->stim_amp : 0.0f;
+    }
     BBX_CUDA(cudaMemcpyAsync(g->d_t, &g->h_t, sizeof(TissueArgs), cudaMemcpyHostToDevice, g->stream));
     BBX_CUDA(cudaStreamSynchronize(g->stream));
     return BBX_OK;
@@ -2210,7 +2259,7 @@ int bbx_step(bbx_grid* g, double dt, int n_steps) {
         if (n_steps == 0) return BBX_OK;
     }
     auto args = [&](const LaunchPlan& lp) {
-        LaunchArgs L = launch_args(lp, g->d_t, g->d_err, g->poison, &g->h_t);
+        LaunchArgs L = launch_args(lp, g->d_t, g->d_err, g->poison, &lp == &g->lpf ? &g->h_tf : &g->h_t);
         if (!g->d_mask) {
             // unmasked grid: whole columns in order (nz planes, or a sheet's nby
             // tile rows), equal shares (build_plan)
@@ -2554,6 +2603,7 @@ int bbx_read_active_bricks(bbx_grid* g, int32_t* out, size_t cap, long long* cou
 int bbx_set_tiling(bbx_grid* g, int tile_y, int tile_z) {
     if (!g || (tile_y != 7 && tile_y != 14 && tile_y != 28) || tile_z < 1) return BBX_ERR_ARG;
     const int old_ty = g->ty, old_zb = g->zb;
+    g->ty_flow = g->flow_measured = 0;
     g->ty = tile_y;
     g->zb = tile_z > g->nz ? g->nz : tile_z;
     int rc = build_bricks(g);
@@ -2725,10 +2775,10 @@ int bbx_autotune(bbx_grid* g, double dt, double* best_ms) {
             if (z <= g->nz) zbs.push_back(z);
         if (g->nz > 64) zbs.push_back(g->nz);
     }
-    // A sheet whose longer calls run in a resident kernel, which has no tiles, is
-    // tuned for the calls that take them: one launch a step.
+    // Where longer calls have their own plan, or run in a resident kernel, which has
+    // no tiles, the tile is that of one launch a step.
     const int route0 = g->route;
-    if (g->pairs_ok || g->resident) g->route = BBX_ROUTE_STEPS;
+    if (g->two_plans || g->pairs_ok || g->resident) g->route = BBX_ROUTE_STEPS;
     double best = 1e30;
     int bty = g->ty, bzb = g->zb;
     bool gathers7 = false;
@@ -2773,10 +2823,47 @@ int bbx_autotune(bbx_grid* g, double dt, double* best_ms) {
         }
         if (rc) break;
     }
+    int rc2 = bbx_set_tiling(g, bty, bzb);
     g->route = route0;
+    if (rc == BBX_OK && rc2 == BBX_OK && g->two_plans && route0 == BBX_ROUTE_AUTO && !g->resident &&
+        !(g->pairs_ok && g->pairs_from <= 16)) {
+        // Several steps a launch: its own tile rows, and from how many steps of a
+        // call it is faster, by calls of 4 and of 16 steps (64x64x16 slab: 7 rows are
+        // the fastest at one step a launch, 6.8 us against 7.7 with 28, and 28 at ten
+        // steps a launch, 6.2 us against 7.4; 100x60x20 never)
+        double best16 = 1e30, from = 1e30;
+        int btyf = 0;
+        g->route = BBX_ROUTE_SEVERAL;
+        for (int ty : tys) {
+            g->ty_flow = ty;
+            if ((rc = replan_flow(g)) != BBX_OK) break;
+            if (!g->lpf.flow || g->lpf.k.ty != ty) continue;
+            float t[2] = {0.f, 0.f};
+            if ((rc = bbx_step(g, dt, 4)) != BBX_OK) break;
+            for (int k = 0; k < 2; ++k) {
+                cudaEventRecord(e0, g->stream);
+                if ((rc = bbx_step(g, dt, k ? 16 : 4)) != BBX_OK) break;
+                cudaEventRecord(e1, g->stream);
+                cudaEventSynchronize(e1);
+                cudaEventElapsedTime(&t[k], e0, e1);
+            }
+            if (rc) break;
+            if (t[1] < best16) {
+                best16 = t[1];
+                btyf = ty;
+                // a further step; the call's own cost is t[0] - 4 step, and 3 us for a cooperative launch
+                // behind other work, which these events do not see
+                const double step = (t[1] - t[0]) / 12.0, own = t[0] - 4.0 * step + 0.003;
+                from = step < 0.98 * best ? std::max(2.0, std::ceil(own / (best - step))) : 1e30;
+            }
+        }
+        g->route = route0;
+        g->ty_flow = btyf;
+        g->flow_measured = from < 1e6 ? (int)from : (btyf ? INT_MAX : 0);
+        rc2 = replan_flow(g);
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    int rc2 = bbx_set_tiling(g, bty, bzb);
     cudaMemcpyAsync(g->d_state[0], save, sbytes, cudaMemcpyDeviceToDevice, g->stream);
     cudaMemcpyAsync(g->d_state[1], save, sbytes, cudaMemcpyDeviceToDevice, g->stream);
     cudaMemcpyAsync(g->d_act, save_act, sizeof(int32_t) * g->vol, cudaMemcpyDeviceToDevice, g->stream);

@@ -242,3 +242,27 @@ def test_gathered_entries_of_a_masked_anisotropic_grid(bbx, model):
         out.append(G.read_all()[:, mask != 0])
     assert np.isfinite(out[0]).all()
     assert np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("shape,fibres", [((16, 64, 64), "rotational"), ((20, 70, 66), "none"), ((1, 300, 200), "smooth"),
+                                          ((130, 100, 90), "none")])
+def test_autotuned_plans_of_one_and_of_several_steps(bbx, shape, fibres):
+    """The two plans have tile rows of their own; calls that mix them give the results of one-step calls,
+    the total of a call from its own plan's pieces, and settings changed in between reach both."""
+    A, dt = _block(bbx, "barkley", shape, fibres, 14)
+    B, _ = _block(bbx, "barkley", shape, fibres, 14)
+    A.autotune(dt)
+    for k, n in enumerate((64, 1, 70, 2)):
+        if k == 2:
+            for G in (A, B):
+                G.set_stimulus((np.random.default_rng(8).random(shape) < 0.2).astype(np.uint8), 3.0, 0.0, 1.0)
+                G.set_threshold(0.4)
+        A.step(dt, n)
+        _one_by_one(B, dt, n)
+        _same(A, B)
+    A.autotune(dt)
+    A.set_scheme(1)
+    B.set_scheme(1)
+    A.step(dt, 24)
+    _one_by_one(B, dt, 24)
+    _same(A, B)
