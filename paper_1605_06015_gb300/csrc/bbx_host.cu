@@ -2830,17 +2830,19 @@ int bbx_autotune(bbx_grid* g, double dt, double* best_ms) {
         // Several steps a launch: its own tile rows, and from how many steps of a
         // call it is faster, by calls of 4 and of 16 steps (64x64x16 slab: 7 rows are
         // the fastest at one step a launch, 6.8 us against 7.7 with 28, and 28 at ten
-        // steps a launch, 6.2 us against 7.4; 100x60x20 never)
-        double best16 = 1e30, from = 1e30;
-        int btyf = 0;
+        // steps a launch, 6.2 us against 7.4; 100x60x20 never).  On large grids, where
+        // a step takes long, the rows by calls of 4 steps alone.
+        const bool small = own_nodes(g) < kFlowNodes;
+        double bestf = 1e30;
+        int btyf = 0, from = 0;
         g->route = BBX_ROUTE_SEVERAL;
         for (int ty : tys) {
             g->ty_flow = ty;
             if ((rc = replan_flow(g)) != BBX_OK) break;
             if (!g->lpf.flow || g->lpf.k.ty != ty) continue;
             float t[2] = {0.f, 0.f};
-            if ((rc = bbx_step(g, dt, 4)) != BBX_OK) break;
-            for (int k = 0; k < 2; ++k) {
+            if ((rc = bbx_step(g, dt, 2)) != BBX_OK) break;
+            for (int k = 0; k < (small ? 2 : 1); ++k) {
                 cudaEventRecord(e0, g->stream);
                 if ((rc = bbx_step(g, dt, k ? 16 : 4)) != BBX_OK) break;
                 cudaEventRecord(e1, g->stream);
@@ -2848,18 +2850,18 @@ int bbx_autotune(bbx_grid* g, double dt, double* best_ms) {
                 cudaEventElapsedTime(&t[k], e0, e1);
             }
             if (rc) break;
-            if (t[1] < best16) {
-                best16 = t[1];
+            if (t[small] < bestf) {
+                bestf = t[small];
                 btyf = ty;
                 // a further step; the call's own cost is t[0] - 4 step, and 3 us for a cooperative launch
                 // behind other work, which these events do not see
                 const double step = (t[1] - t[0]) / 12.0, own = t[0] - 4.0 * step + 0.003;
-                from = step < 0.98 * best ? std::max(2.0, std::ceil(own / (best - step))) : 1e30;
+                if (small) from = step < 0.98 * best ? (int)std::max(2.0, std::ceil(std::min(1e6, own / (best - step)))) : INT_MAX;
             }
         }
         g->route = route0;
         g->ty_flow = btyf;
-        g->flow_measured = from < 1e6 ? (int)from : (btyf ? INT_MAX : 0);
+        g->flow_measured = from;
         rc2 = replan_flow(g);
     }
     cudaEventDestroy(e0);
