@@ -639,7 +639,7 @@ struct Seg {
 };
 
 // (bbx_grid's plans)
-constexpr long long kFlowSheetMin = 250000, kFlowNodesLarge = 15000000;
+constexpr long long kFlowSheetMin = 250000;
 
 struct LaunchPlan {
     StepKernel k = {nullptr, 0, 0, 0};
@@ -933,13 +933,12 @@ cudaError_t launch(const LaunchPlan& lp, const LaunchArgs& L, cudaStream_t s) {
 // of the done flags (3 us), or the CTAs wait for one another every step.
 // Measured (us a step, one launch a step / several steps a launch, the best
 // tile height of each):
-// - from 25 million nodes on a launch's own cost is little and the first step of
-//   several, which has no launch before it to overlap with, weighs: 8192x8192 n =
-//   2 200 / 210, n = 4 200 / 201, n = 10 200 / 189; 512x512x128 n = 4 96 / 100, n
-//   = 10 96 / 94; without W-tilde sums 512x512x128 n = 4 154 / 162, n = 10 154 / 155;
-// - from 3 million on: 256x256x64 slab n = 2 26.3 / 25.7, n = 10 26.3 / 22.1;
+// - from 3 million nodes on: 256x256x64 slab n = 2 26.3 / 25.7, n = 10 26.3 / 22.1;
 //   192^3 n = 2 28.1 / 27.3; 400x400x100 n = 2 59.6 / 56.9, n = 10 59.5 / 50.9;
-//   3000x5000 n = 2 48.6 / 48.4, n = 3 48.6 / 45.8;
+//   3000x5000 n = 2 48.6 / 48.4, n = 3 48.6 / 45.8; of the largest only longer calls
+//   (8192x8192 n = 4 200 / 201, n = 10 200 / 189; 512x512x128 n = 4 96 / 100, n = 10
+//   96 / 94), but these go with the tile rows chosen at rest: in waves 8192x8192 n
+//   = 4 214 / 200;
 // - fewer, with long shares: 128^3 anisotropic, 16 planes n = 3 16.2 / 16.0;
 //   isotropic, 11 planes n = 6 13.3 / 13.6, n = 10 13.3 / 13.1; 1500x1500 and
 //   1400x1400, 3 to 14 planes, n = 10 12.0 / 12.1, n = 20 11.9 / 11.5;
@@ -950,8 +949,7 @@ cudaError_t launch(const LaunchPlan& lp, const LaunchArgs& L, cudaStream_t s) {
 //   n = 20 6.8 / 7.0), blocks (80 CTAs n = 6 7.1 / 7.1, 192 n = 10 8.0 / 7.6, 320
 //   n = 20 8.8 / 8.2).
 constexpr long long kFlowNodes = 3000000, kFlowNodesMin = 1500000;
-int flow_steps_from(long long nodes, long long planes, int ctas, int num_sms, bool planar, bool no_sums) {
-    if (nodes >= 25000000) return no_sums ? 10 : 4;
+int flow_steps_from(long long nodes, long long planes, int ctas, int num_sms, bool planar) {
     if (nodes >= kFlowNodes) return 2;
     if (planes <= ctas) {
         if (planar) return planes <= num_sms ? 4 + (int)planes / 8 : 0;
@@ -1057,13 +1055,11 @@ struct bbx_grid {
     TissueDyn* d_dyn = nullptr;    // device-updated time, step, parity, total
     // lp: one step a launch; lpf: several, in calls of flow_from steps or more.  The
     // kernels without the sync warp, four CTAs an SM instead of three when
-    // isotropic, are the faster ones at one step a launch of small and of large
-    // grids (400x400 6.5 us against 7.0, 128^3 13.3 against 13.6, 3000x5000 48.6 /
-    // 50.8, 512x512x256 184 / 202); from kFlowNodes nodes to kFlowNodesLarge, on
-    // isotropic sheets already from kFlowSheetMin, and where they have no variant
-    // without W-tilde sums, lp serves both (192^3 28.2 / 26.5, 4096x2048 27.7 / 27.4,
-    // 256x256x100 26.5 / 25.5, 512x512 6.5 / 6.2, 700x900 8.9 / 7.6, 1500x1500 11.9 /
-    // 10.4; 256x256x64 18.1 / 18.4).
+    // isotropic, are the faster ones at one step a launch of small grids (400x400
+    // 6.5 us against 7.0, 128^3 13.3 against 13.6).  From kFlowNodes nodes, on
+    // isotropic sheets already from kFlowSheetMin, lp serves both (192^3 28.2 / 26.5,
+    // 4096x2048 27.7 / 27.4, 512x512 6.5 / 6.2, 700x900 8.9 / 7.6, 1500x1500 11.9 /
+    // 10.4; 256x256x64 18.1 / 18.4, 3000x5000 48.6 / 50.8, and 512x512x256 184 / 202).
     LaunchPlan lp, lpf;
     int flow_from = 0;
     bool two_plans = false;
@@ -1436,15 +1432,13 @@ bool resident_shape(const bbx_grid* g) {
 long long own_nodes(const bbx_grid* g) { return (long long)g->nx * g->ny * (g->nz - g->halo_lo - g->halo_hi); }
 
 // The step kernel of a grid for `ty` tile rows (flow: the variant that may take
-// several steps in one launch, where there is one) and its CTA budget; no_sums:
-// it is the variant without W-tilde sums.
-int pick_kernel(const bbx_grid* g, int ty, bool flow, StepKernel* k, int* ctas, bool* no_sums) {
+// several steps in one launch, where there is one) and its CTA budget.
+int pick_kernel(const bbx_grid* g, int ty, bool flow, StepKernel* k, int* ctas) {
     const bool surr = g->surr_on && g->model == BBX_BR;
     int r = BBX_ERR_UNSUPPORTED;
     if (g->aniso && g->wsum_zero && g->wsum_elide && !g->d_mask)  // the variant without W-tilde sums, if built
         r = select_kernel(g->model, false, AN_NO_SUMS, ty, g->device, g->num_sms, k, ctas, surr, g->nz == 1,
                           wants_general(g), g->gates, flow);
-    *no_sums = r == BBX_OK;
     if (r == BBX_ERR_UNSUPPORTED)
         r = select_kernel(g->model, g->d_mask != nullptr, g->aniso ? AN_SUMS : AN_ISO, ty, g->device, g->num_sms, k,
                           ctas, surr, g->nz == 1, wants_general(g), g->gates, flow);
@@ -1461,17 +1455,16 @@ int prepare_flow(bbx_grid* g) {
         return BBX_OK;
     }
     int ctas = 0;
-    bool no_sums = false;
     StepKernel k;
-    int rc = pick_kernel(g, g->ty_flow ? g->ty_flow : g->ty, true, &k, &ctas, &no_sums);
-    if (rc == BBX_ERR_UNSUPPORTED) rc = pick_kernel(g, g->ty, true, &k, &ctas, &no_sums);
+    int rc = pick_kernel(g, g->ty_flow ? g->ty_flow : g->ty, true, &k, &ctas);
+    if (rc == BBX_ERR_UNSUPPORTED) rc = pick_kernel(g, g->ty, true, &k, &ctas);
     if (rc) return rc;
     std::vector<Seg> segs;
     grid_segments(g, k.ty, 0, &segs);
     long long planes = 0;
     for (const Seg& sg : segs) planes += sg.z1 - sg.z0;
     g->flow_from = g->flow_measured ? (g->flow_measured < INT_MAX ? g->flow_measured : 0)
-                                    : flow_steps_from(own_nodes(g), planes, ctas, g->num_sms, g->nz == 1, no_sums);
+                                    : flow_steps_from(own_nodes(g), planes, ctas, g->num_sms, g->nz == 1);
     if (g->pairs_ok && g->pairs_from <= g->flow_from) g->flow_from = 0;  // (those calls run in registers)
     if (g->flow_from == 0 && g->route >= BBX_ROUTE_SEVERAL) g->flow_from = INT_MAX;  // (only asked for)
     if (g->flow_from == 0) {
@@ -1503,10 +1496,9 @@ int prepare(bbx_grid* g) {
     int rc0 = finish_total(g);  // the plan's partials are about to be replaced
     if (rc0 || (rc0 = tab_refresh(g))) return rc0;
     BBX_CUDA(cudaStreamSynchronize(g->stream));
-    bool no_sums = false;
     StepKernel k;
     int ctas = 0;
-    int rc = pick_kernel(g, g->ty, true, &k, &ctas, &no_sums);
+    int rc = pick_kernel(g, g->ty, true, &k, &ctas);
     if (rc) return rc;
     if ((rc = encode_targs(g, k.ty, &g->h_t))) return rc;
     BBX_CUDA(cudaMemcpyAsync(g->d_t, &g->h_t, sizeof(TissueArgs), cudaMemcpyHostToDevice, g->stream));
@@ -1523,16 +1515,15 @@ int prepare(bbx_grid* g) {
     }
     const long long nodes = own_nodes(g);
     const bool light = k.flow && !g->d_mask;
-    g->two_plans = light && (nodes >= kFlowNodes ? nodes >= kFlowNodesLarge && !no_sums
-                                                 : nodes < kFlowSheetMin || g->nz > 1 || g->aniso);
+    g->two_plans = light && nodes < kFlowNodes && (nodes < kFlowSheetMin || g->nz > 1 || g->aniso);
     if ((rc = prepare_flow(g))) return rc;
     std::vector<Lattice> lattice;
     if (g->two_plans) {
-        if ((rc = pick_kernel(g, g->ty, false, &k, &ctas, &no_sums))) return rc;
+        if ((rc = pick_kernel(g, g->ty, false, &k, &ctas))) return rc;
     } else if (light) {
         long long planes = 0;
         for (const Seg& sg : segs) planes += sg.z1 - sg.z0;
-        g->flow_from = flow_steps_from(nodes, planes, ctas, g->num_sms, g->nz == 1, no_sums);
+        g->flow_from = flow_steps_from(nodes, planes, ctas, g->num_sms, g->nz == 1);
         if (g->flow_from == 0 && g->route >= BBX_ROUTE_SEVERAL) g->flow_from = INT_MAX;  // (only asked for)
         if (g->flow_from) lattice.push_back(grid_lattice(g, k.ty));
     }
@@ -2827,13 +2818,11 @@ int bbx_autotune(bbx_grid* g, double dt, double* best_ms) {
     g->route = route0;
     if (rc == BBX_OK && rc2 == BBX_OK && g->two_plans && route0 == BBX_ROUTE_AUTO && !g->resident &&
         !(g->pairs_ok && g->pairs_from <= 16)) {
-        // Several steps a launch: its own tile rows, and from how many steps of a
-        // call it is faster, by calls of 4 and of 16 steps (64x64x16 slab: 7 rows are
-        // the fastest at one step a launch, 6.8 us against 7.7 with 28, and 28 at ten
-        // steps a launch, 6.2 us against 7.4; 100x60x20 never).  On large grids, where
-        // a step takes long, the rows by calls of 4 steps alone.
-        const bool small = own_nodes(g) < kFlowNodes;
-        double bestf = 1e30;
+        // Several steps a launch: its own tile rows, and from how many steps of a call
+        // it is faster, by calls of 4 and of 16 steps (64x64x16 slab: 7 rows are the
+        // fastest at one step a launch, 6.8 us against 7.7 with 28, and 28 at ten steps
+        // a launch, 6.2 us against 7.4; 100x60x20 never)
+        double best16 = 1e30;
         int btyf = 0, from = 0;
         g->route = BBX_ROUTE_SEVERAL;
         for (int ty : tys) {
@@ -2841,8 +2830,8 @@ int bbx_autotune(bbx_grid* g, double dt, double* best_ms) {
             if ((rc = replan_flow(g)) != BBX_OK) break;
             if (!g->lpf.flow || g->lpf.k.ty != ty) continue;
             float t[2] = {0.f, 0.f};
-            if ((rc = bbx_step(g, dt, 2)) != BBX_OK) break;
-            for (int k = 0; k < (small ? 2 : 1); ++k) {
+            if ((rc = bbx_step(g, dt, 4)) != BBX_OK) break;
+            for (int k = 0; k < 2; ++k) {
                 cudaEventRecord(e0, g->stream);
                 if ((rc = bbx_step(g, dt, k ? 16 : 4)) != BBX_OK) break;
                 cudaEventRecord(e1, g->stream);
@@ -2850,13 +2839,13 @@ int bbx_autotune(bbx_grid* g, double dt, double* best_ms) {
                 cudaEventElapsedTime(&t[k], e0, e1);
             }
             if (rc) break;
-            if (t[small] < bestf) {
-                bestf = t[small];
+            if (t[1] < best16) {
+                best16 = t[1];
                 btyf = ty;
                 // a further step; the call's own cost is t[0] - 4 step, and 3 us for a cooperative launch
                 // behind other work, which these events do not see
                 const double step = (t[1] - t[0]) / 12.0, own = t[0] - 4.0 * step + 0.003;
-                if (small) from = step < 0.98 * best ? (int)std::max(2.0, std::ceil(std::min(1e6, own / (best - step)))) : INT_MAX;
+                from = step < 0.98 * best ? (int)std::max(2.0, std::ceil(std::min(1e6, own / (best - step)))) : INT_MAX;
             }
         }
         g->route = route0;
