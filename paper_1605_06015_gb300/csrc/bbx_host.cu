@@ -925,8 +925,10 @@ cudaError_t launch(const LaunchPlan& lp, const LaunchArgs& L, cudaStream_t s) {
     return cudaLaunchKernelExC(&cfg, lp.k.fn, args);
 }
 
-// From how many steps of a call a grid takes several steps a launch (0: never),
-// where bbx_autotune has not measured it.
+// From how many steps of a call a grid takes several steps a launch (0: never):
+// from kFlowNodes nodes 2; smaller isotropic sheets that keep one plan (bbx_grid's
+// plans) never; the others by flow_steps_from, where bbx_autotune has not measured
+// it.
 // A launch of several steps costs 5 us more than one of one step (20 us where a
 // step takes 200) and saves each further step the fill and drain of a launch,
 // 2 to 8 us; but a CTA's share of a step has to be long against the round trips
@@ -940,8 +942,10 @@ cudaError_t launch(const LaunchPlan& lp, const LaunchArgs& L, cudaStream_t s) {
 //   96 / 94), but these go with the tile rows chosen at rest: in waves 8192x8192 n
 //   = 4 214 / 200;
 // - fewer, with long shares: 128^3 anisotropic, 16 planes n = 3 16.2 / 16.0;
-//   isotropic, 11 planes n = 6 13.3 / 13.6, n = 10 13.3 / 13.1; 1500x1500 and
-//   1400x1400, 3 to 14 planes, n = 10 12.0 / 12.1, n = 20 11.9 / 11.5;
+//   isotropic, 11 planes n = 6 13.3 / 13.6, n = 10 13.3 / 13.1; 1400x1400 with
+//   fibres, 7 to 14 planes, n = 10 12.0 / 12.8, n = 20 12.0 / 11.8;
+// - isotropic sheets, whose kernel with 28 rows is as fast at one step a launch,
+//   not: 1500x1500 n = 20 10.3 / 12.2;
 // - below 1.5 million nodes not (700x900 n = 20 8.9 / 9.8; 1024x1024 8.8 / 10.8;
 //   96^3 anisotropic 12.9 / 14.1);
 // - except where no CTA takes more than one plane and few CTAs exchange flags:
@@ -950,7 +954,6 @@ cudaError_t launch(const LaunchPlan& lp, const LaunchArgs& L, cudaStream_t s) {
 //   n = 20 8.8 / 8.2).
 constexpr long long kFlowNodes = 3000000, kFlowNodesMin = 1500000;
 int flow_steps_from(long long nodes, long long planes, int ctas, int num_sms, bool planar) {
-    if (nodes >= kFlowNodes) return 2;
     if (planes <= ctas) {
         if (planar) return planes <= num_sms ? 4 + (int)planes / 8 : 0;
         return std::max(8, (int)planes / 12);
@@ -1057,7 +1060,7 @@ struct bbx_grid {
     // kernels without the sync warp, four CTAs an SM instead of three when
     // isotropic, are the faster ones at one step a launch of small grids (400x400
     // 6.5 us against 7.0, 128^3 13.3 against 13.6).  From kFlowNodes nodes, on
-    // isotropic sheets already from kFlowSheetMin, lp serves both (192^3 28.2 / 26.5,
+    // isotropic sheets (28 rows) already from kFlowSheetMin, lp serves both (192^3 28.2 / 26.5,
     // 4096x2048 27.7 / 27.4, 512x512 6.5 / 6.2, 700x900 8.9 / 7.6, 1500x1500 11.9 /
     // 10.4; 256x256x64 18.1 / 18.4, 3000x5000 48.6 / 50.8, and 512x512x256 184 / 202).
     LaunchPlan lp, lpf;
@@ -1515,15 +1518,13 @@ int prepare(bbx_grid* g) {
     }
     const long long nodes = own_nodes(g);
     const bool light = k.flow && !g->d_mask;
-    g->two_plans = light && nodes < kFlowNodes && (nodes < kFlowSheetMin || g->nz > 1 || g->aniso);
+    g->two_plans = light && nodes < kFlowNodes && (nodes < kFlowSheetMin || g->nz > 1 || g->aniso || wants_general(g));
     if ((rc = prepare_flow(g))) return rc;
     std::vector<Lattice> lattice;
     if (g->two_plans) {
         if ((rc = pick_kernel(g, g->ty, false, &k, &ctas))) return rc;
     } else if (light) {
-        long long planes = 0;
-        for (const Seg& sg : segs) planes += sg.z1 - sg.z0;
-        g->flow_from = flow_steps_from(nodes, planes, ctas, g->num_sms, g->nz == 1);
+        g->flow_from = nodes >= kFlowNodes ? 2 : 0;
         if (g->flow_from == 0 && g->route >= BBX_ROUTE_SEVERAL) g->flow_from = INT_MAX;  // (only asked for)
         if (g->flow_from) lattice.push_back(grid_lattice(g, k.ty));
     }
