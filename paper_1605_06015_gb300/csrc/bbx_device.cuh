@@ -50,10 +50,9 @@ struct TissueDyn {
     double total;   // tissue sum of V after the most recent step
     long long n;    // steps taken
     int cur;        // buffer holding the current state (0 or 1)
-    int total_pending;  // 1: total is still to be summed from the per-piece
-                        // partials of the grid's last single-grid launch:
-    int n_slots;
-    const double* partials;
+    int total_pending;  // not 0: total is still to be summed from the per-piece
+                        // partials of the grid's last single-grid launch (1, 2:
+                        // of which of the grid's plans)
 };
 
 // Host-written description of one grid for the step kernel (in device memory,
@@ -139,6 +138,7 @@ struct LaunchArgs {
     const PieceFlags* piece_flags;  // per slot
     int* flags;          // per grid column and computed plane: the last step done, as a running number
     int epoch;           // that number before this launch's first step
+    int total_mark;      // single-grid launch: total_pending after it
 };
 
 struct Coef {
@@ -356,9 +356,7 @@ __device__ __forceinline__ void start_ticket(const LaunchArgs& L, const TissueDy
         d->t = tn;
         d->n = d0.n + L.n_steps;
         d->cur = d0.cur ^ (L.n_steps & 1);
-        d->n_slots = L.n_slots;
-        d->partials = L.partials;
-        d->total_pending = 1;
+        d->total_pending = L.total_mark;
         *L.ticket = 0u;
     }
 }

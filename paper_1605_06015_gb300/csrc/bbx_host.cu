@@ -534,12 +534,15 @@ __global__ void k_total(const float* __restrict__ u, const uint8_t* __restrict__
 // The total of a grid's last single-grid step, summed from the step's
 // per-piece partials in slot order (unused slots hold 0) when it is asked
 // for; nothing happens if no total is pending.  One CTA.
-__global__ void k_finish_total(TissueDyn* dyn, int* err) {
+__global__ void k_finish_total(const double* __restrict__ partials1, int n_slots1, const double* __restrict__ partials2,
+                               int n_slots2, TissueDyn* dyn, int* err) {
     __shared__ double scratch[32];
-    if (!dyn->total_pending) return;  // uniform: every thread reads the same flag
+    const int mark = dyn->total_pending;
+    if (!mark) return;  // uniform: every thread reads the same flag
     double s = 0.0;
-    const double* partials = dyn->partials;
-    for (int k = threadIdx.x; k < dyn->n_slots; k += blockDim.x) s += partials[k];
+    const double* partials = mark == 2 ? partials2 : partials1;
+    const int n_slots = mark == 2 ? n_slots2 : n_slots1;
+    for (int k = threadIdx.x; k < n_slots; k += blockDim.x) s += partials[k];
     const double total = block_sum_double(s, scratch);
     if (threadIdx.x == 0) {
         if (!isfinite(total)) atomicOr(err, ERRBIT_NAN);
@@ -865,6 +868,7 @@ LaunchArgs launch_args(const LaunchPlan& lp, const TissueArgs* d_tissues, int* d
     L.cur_hint = -1;
     L.wait_limit = poison ? kPoisonWaitLimit : kWaitLimitCycles;
     L.n_steps = 1;
+    L.total_mark = 1;
     L.flags = lp.d_flags;
     L.piece_flags = lp.d_piece_flags;
     return L;
@@ -1577,7 +1581,8 @@ int write_dyn(bbx_grid* g, const TissueDyn& d) {
 // anything that reads the total or overwrites the partials.
 int finish_total(bbx_grid* g) {
     if (!g->lp.d_partials || g->lp.n_slots <= 0 || !g->d_dyn) return BBX_OK;
-    k_finish_total<<<1, 256, 0, g->stream>>>(g->d_dyn, g->d_err);
+    k_finish_total<<<1, 256, 0, g->stream>>>(g->lp.d_partials, g->lp.n_slots, g->lpf.d_partials, g->lpf.n_slots, g->d_dyn,
+                                             g->d_err);
     BBX_CUDA(cudaGetLastError());
     return BBX_OK;
 }
@@ -2252,6 +2257,7 @@ int bbx_step(bbx_grid* g, double dt, int n_steps) {
     }
     auto args = [&](const LaunchPlan& lp) {
         LaunchArgs L = launch_args(lp, g->d_t, g->d_err, g->poison, &lp == &g->lpf ? &g->h_tf : &g->h_t);
+        L.total_mark = &lp == &g->lpf ? 2 : 1;
         if (!g->d_mask) {
             // unmasked grid: whole columns in order (nz planes, or a sheet's nby
             // tile rows), equal shares (build_plan)
